@@ -208,8 +208,10 @@ void qcd_destroy(qcd_ctx* c) {
   devbuf_free(c->gaugeF);
   devbuf_free(c->cloverD);
   devbuf_free(c->cloverF);
-  devbuf_free(c->gaugeH);
-  devbuf_free(c->cloverH);
+  devbuf_free(c->sap_img16.buf);
+  devbuf_free(c->sap_img32.buf);
+  devbuf_free(c->flinks);
+  devbuf_free(c->sap_vec);
   for (int i = 0; i < 8; i++) {
     devbuf_free(c->wsD[i]);
     devbuf_free(c->wsF[i]);
@@ -250,6 +252,7 @@ qcd_status qcd_load_gauge(qcd_ctx* c, const double* U, int U_on_device, double c
     QCD_CUDA_OK(cudaMemcpyAsync(c->stage.p, U, bytes, cudaMemcpyHostToDevice, c->stream));
     Ud = (const double*)c->stage.p;
   }
+  c->gauge_id++;   // the block images of the previous field are out of date
   QCD_TRY(layout_gauge_import(c, Ud));
   QCD_TRY(layout_clover_build(c));
   QCD_CUDA_OK(cudaStreamSynchronize(c->stream));

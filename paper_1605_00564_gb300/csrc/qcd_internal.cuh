@@ -421,8 +421,14 @@ struct ProfRec {
   double bytes, flops;
 };
 
+struct SapImage {
+  DevBuf buf;
+  int block[4] = {0, 0, 0, 0};
+  uint64_t gauge_id = 0;
+};
+
 struct SapGraph {
-  const void *rho_src, *rho, *psi, *delta, *gauge, *clover;
+  const void *rho_src, *rho, *psi, *delta, *gauge, *clover, *img, *flinks, *vec;
   const int* mask;
   int nrhs, ncy, nmr, accumulate, half, prec, block[4];
   double kappa;
@@ -443,12 +449,13 @@ struct qcd_ctx {
   qcd_solver_params params;
   // fields
   DevBuf gaugeD, gaugeF, cloverD, cloverF;
-  // FP16 copies for the sloppy SAP block solves (layout.cu): links as the nine
-  // (re, im) entries of the full matrix (third row reconstructed in FP32 from
-  // the FP32 rows, then rounded), [4][V] uint4 of entries 0-3, [4][V] uint4 of
-  // entries 4-7, [4][V] uint32 of entry 8 (36 B per link); clover as
-  // [9][V] uint4 of eight FP16 reals (144 B per site)
-  DevBuf gaugeH, cloverH;
+  // SAP block images of the links and clover term (sap.cu), 16-bit and FP32,
+  // and the FP32 links across the faces of 4^4 blocks; rebuilt when gauge_id
+  // (counted up by every qcd_load_gauge) or the block shape differs
+  uint64_t gauge_id = 0, flinks_id = 0;
+  SapImage sap_img16, sap_img32;
+  DevBuf flinks;
+  DevBuf sap_vec;     // block-ordered working vectors of the 4^4 sweep
   // workspaces (grown on demand, kept until destroy)
   DevBuf wsD[8];      // FP64 spinors (nrhs each)
   DevBuf wsF[8];      // FP32 spinors

@@ -27,7 +27,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
-#include "qcd_internal.cuh"
+#include "spin_pair.cuh"
 
 namespace {
 
@@ -216,142 +216,248 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sap_sweep(const char* __restrict
 }
 
 // ---------------------------------------------------------------------------
-// Shared-memory-resident variant (FP32 arithmetic).  The block's links (two
-// rows each) and clover term are staged in shared memory once per sweep, so
-// the n_mr MR steps read only shared memory.  S selects the storage of the
-// staged copies: float (exact single precision) or __half (16-bit copies of
-// links and clover, half the shared memory, two CTAs per SM; the
-// preconditioner is then a slightly different operator, which the flexible
-// outer GCR tolerates).
+// FP32 sweeps in two-lane arithmetic (spin_pair.cuh).
+//
+// Links and clover term come from a block image: for each block (all black
+// blocks first, blk-th block of a colour as in the sweep) its sites' words in
+// the order of the local index, so a block is one contiguous run.  Read from the
+// lexicographic fields a warp's 32 sites of a 4^4 block are eight pieces of 64
+// bytes in as many lines, and every word of a site is another page: such loads
+// took 22,000 of the 56,000 clock cycles of a CTA.  S selects the image and how
+// the MR steps use it:
+//   __half     16-bit copies (uint4 [4][vb] entries 0-3 of the four links, uint4
+//              [4][vb] entries 4-7, half2 [4][vb] entry 8, uint4 [9][vb] clover;
+//              288 B a site), staged whole in shared memory.  The preconditioner
+//              is then a slightly different operator, which the flexible outer
+//              GCR tolerates;
+//   float      FP32 (float4 [12][vb] link rows 0 and 1, float4 [18][vb] clover in
+//              the order of CloverPairs; 480 B a site): links staged, clover
+//              read from the image (L2) at every step.  With both staged a 4^4
+//              block takes 172 KB and an SM holds one CTA, whose loads and
+//              barriers nothing hides;
+//   FromImage  the FP32 image read from L2 at every step (blocks of more than 256
+//              sites, whose copies exceed shared memory);
+//   FromField  the same from the lexicographic fields, where there is no memory
+//              for an image.
+// Either staged form leaves room for two CTAs of a 4^4 block per SM.
 // ---------------------------------------------------------------------------
+struct FromImage {};
+struct FromField {};
+
 template <typename S>
-struct Stage;
-template <>
-struct Stage<float> {
-  using W = float4;   // four reals
-  using C = float2;   // one complex
-  static __device__ inline W put(float4 v) { return v; }
-  static __device__ inline float4 get(W w) { return w; }
-  static __device__ inline C putc(Cplx<float> z) { return make_float2(z.re, z.im); }
-  static __device__ inline Cplx<float> getc(C w) { return cmk(w.x, w.y); }
-};
-template <>
-struct Stage<__half> {
-  using W = uint2;
-  static __device__ inline W put(float4 v) {
-    __half2 a = __floats2half2_rn(v.x, v.y), b = __floats2half2_rn(v.z, v.w);
-    W w;
-    w.x = *reinterpret_cast<unsigned*>(&a);
-    w.y = *reinterpret_cast<unsigned*>(&b);
-    return w;
-  }
-  static __device__ inline float4 get(W w) {
-    float2 a = __half22float2(*reinterpret_cast<__half2*>(&w.x));
-    float2 b = __half22float2(*reinterpret_cast<__half2*>(&w.y));
-    return make_float4(a.x, a.y, b.x, b.y);
-  }
-  using C = __half2;
-  static __device__ inline C putc(Cplx<float> z) { return __floats2half2_rn(z.re, z.im); }
-  static __device__ inline Cplx<float> getc(C w) {
-    float2 a = __half22float2(w);
-    return cmk(a.x, a.y);
-  }
+struct Stage {   // bytes of shared memory per site for links and clover term
+  static constexpr int bytes = std::is_same<S, __half>::value ? 288 : std::is_same<S, float>::value ? 192 : 0;
 };
 
-// Storage of the block residual shared between neighbouring threads:
-// FP32 complex, or bf16 pairs (FP32 exponent range, 8-bit mantissa; each
-// thread keeps its own residual in FP32 registers, only the neighbours'
-// contributions to p = D_L r see the rounding).
-template <bool BF>
-struct RStore;
-template <>
-struct RStore<false> {
-  using T = Cplx<float>;
-  static __device__ inline T put(Cplx<float> z) { return z; }
-  static __device__ inline Cplx<float> get(T t) { return t; }
+// where a block's links and clover term are (the members S uses)
+struct BlockFields {
+  const void* lk;         // links: shared memory or the block's image
+  const void* cl;         // clover: likewise
+  const float4* gauge;    // lexicographic fields (FromField)
+  const float4* clover;
 };
-template <>
-struct RStore<true> {
-  using T = __nv_bfloat162;
-  static __device__ inline T put(Cplx<float> z) { return __floats2bfloat162_rn(z.re, z.im); }
-  static __device__ inline Cplx<float> get(T t) {
-    float2 f = __bfloat1622float2(t);
-    return cmk(f.x, f.y);
-  }
-};
-// FP32: 16-byte records, word q of site l at ((float4*)r_s)[q * vb + l] holding
-// components 2q and 2q + 1 (one 128-bit load per two components); bf16: one
-// 4-byte word per component at r_s[k * vb + l]
+
+__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(smem)), "l"(gmem)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// The block residual shared between neighbouring threads, six records q = 3 c + a
+// (chirality, colour) per site at [q * vb + l]: (re0, re1, im0, im1) of the two
+// spins as FP32 (one 128-bit load), or as bf16 (FP32 exponent range, 8-bit
+// mantissa, 64 bits; each thread keeps its own residual in FP32 registers,
+// only the neighbours' contributions to p = D_L r see the rounding).
 template <bool BF>
-__device__ inline Spinor<float> rs_load(const typename RStore<BF>::T* r_s, int vb, int l) {
-  Spinor<float> o;
+__device__ __forceinline__ float4 rs_rec(const void* r_s, int vb, int l, int q) {
   if (BF) {
-#pragma unroll
-    for (int k = 0; k < 12; k++) o.c[k] = RStore<BF>::get(r_s[k * vb + l]);
+    const uint2 w = ((const uint2*)r_s)[q * vb + l];
+    const float2 re = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.x));
+    const float2 im = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w.y));
+    return make_float4(re.x, re.y, im.x, im.y);
+  }
+  return ((const float4*)r_s)[q * vb + l];
+}
+template <bool BF>
+__device__ __forceinline__ void rs_put(void* r_s, int vb, int l, int q, float4 v) {
+  if (BF) {
+    const __nv_bfloat162 re = __floats2bfloat162_rn(v.x, v.y), im = __floats2bfloat162_rn(v.z, v.w);
+    ((uint2*)r_s)[q * vb + l] =
+        make_uint2(*reinterpret_cast<const unsigned*>(&re), *reinterpret_cast<const unsigned*>(&im));
   } else {
-    const float4* w = reinterpret_cast<const float4*>(r_s);
+    ((float4*)r_s)[q * vb + l] = v;
+  }
+}
+template <bool BF>
+__device__ __forceinline__ void rs_store(void* r_s, int vb, int l, const PairSpinor& v) {
 #pragma unroll
-    for (int q = 0; q < 6; q++) {
-      const float4 v = w[q * vb + l];
-      o.c[2 * q] = cmk(v.x, v.y);
-      o.c[2 * q + 1] = cmk(v.z, v.w);
+  for (int q = 0; q < 6; q++) rs_put<BF>(r_s, vb, l, q, pair_rec(v, q));
+}
+
+// o = A r at site l of the block (s of the lattice)
+template <typename S>
+__device__ __forceinline__ void block_clover(const BlockFields& f, int V, int s, int vb, int l, const PairSpinor& r,
+                                             PairSpinor& o) {
+#pragma unroll
+  for (int c = 0; c < 2; c++) {
+    if constexpr (std::is_same<S, __half>::value) {
+      uint4 h[5];   // words 18 c .. 18 c + 17 of the site's 36
+#pragma unroll
+      for (int k = 0; k < 5; k++) h[k] = ((const uint4*)f.cl)[(4 * c + k) * vb + l];
+      pair_clover_block(clover_pairs([&](int j) {
+                          const int w = j + 2 * c;
+                          const uint4 v = h[w >> 2];
+                          return __half22float2(bits_h2((w & 3) == 0 ? v.x : (w & 3) == 1 ? v.y : (w & 3) == 2 ? v.z : v.w));
+                        }),
+                        c, r, o);
+    } else if constexpr (std::is_same<S, FromField>::value) {
+      float4 h[9];
+#pragma unroll
+      for (int k = 0; k < 9; k++) h[k] = __ldg(f.clover + (size_t)(9 * c + k) * V + s);
+      pair_clover_block(
+          clover_pairs([&](int j) { return (j & 1) ? p2(h[j >> 1].z, h[j >> 1].w) : p2(h[j >> 1].x, h[j >> 1].y); }), c,
+          r, o);
+    } else {
+      float4 h[9];
+#pragma unroll
+      for (int k = 0; k < 9; k++) h[k] = __ldg((const float4*)f.cl + (9 * c + k) * vb + l);
+      auto pr = [&](int j) { return (j & 1) ? p2(h[j >> 1].z, h[j >> 1].w) : p2(h[j >> 1].x, h[j >> 1].y); };
+      CloverPairs m;
+#pragma unroll
+      for (int k = 0; k < 3; k++) {
+        m.d[k] = pr(k);
+        m.lr[k] = pr(3 + k);
+        m.li[k] = pr(6 + k);
+        m.e[k] = pr(9 + k);
+        m.orr[k] = pr(12 + k);
+        m.oi[k] = pr(15 + k);
+      }
+      pair_clover_block(m, c, r, o);
     }
   }
-  return o;
 }
-template <bool BF>
-__device__ inline void rs_store(typename RStore<BF>::T* r_s, int vb, int l, const Spinor<float>& v) {
-  if (BF) {
-#pragma unroll
-    for (int k = 0; k < 12; k++) r_s[k * vb + l] = RStore<BF>::put(v.c[k]);
+
+// p += scale * (1 + SIGN gamma_MU) U r(ln): the hop from block site ln over
+// link MU of block site ll (lattice site sl), U or U^+
+template <typename S, bool BF, int MU, int SIGN, bool DAG>
+__device__ __forceinline__ void block_hop_pair(PairSpinor& p, const void* r_s, const BlockFields& f, int V, int vb,
+                                               int ln, int ll, int sl, float scale) {
+  auto rec = [&](int q) { return rs_rec<BF>(r_s, vb, ln, q); };
+  if constexpr (std::is_same<S, __half>::value) {
+    // entries 0-3, 4-7 and 8 as (re, im) halves
+    const uint4* lk = (const uint4*)f.lk + MU * vb + ll;
+    const uint4 a = lk[0], b = lk[4 * vb];
+    const unsigned e8 = ((const unsigned*)((const uint4*)f.lk + 8 * vb))[MU * vb + ll];
+    const unsigned w[9] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, e8};
+    pair_hop<MU, SIGN, DAG>(p, rec, [&](int k) { return __half22float2(bits_h2(w[k])); }, scale);
+  } else if constexpr (std::is_same<S, FromField>::value) {
+    const float4* lk = f.gauge + (size_t)3 * MU * V + sl;
+    const LinkRows U = link_rows(__ldg(lk), __ldg(lk + V), __ldg(lk + 2 * (size_t)V));
+    pair_hop<MU, SIGN, DAG>(p, rec, [&](int k) { return U.m[k]; }, scale);
   } else {
-    float4* w = reinterpret_cast<float4*>(r_s);
-#pragma unroll
-    for (int q = 0; q < 6; q++)
-      w[q * vb + l] = make_float4(v.c[2 * q].re, v.c[2 * q].im, v.c[2 * q + 1].re, v.c[2 * q + 1].im);
+    const float4* lk = (const float4*)f.lk + 3 * MU * vb + ll;
+    const LinkRows U = link_rows(lk[0], lk[vb], lk[2 * vb]);
+    pair_hop<MU, SIGN, DAG>(p, rec, [&](int k) { return U.m[k]; }, scale);
   }
-}
-
-// the full 3x3 link (staged with its third row already reconstructed)
-template <typename S>
-__device__ inline SU3<float> smem_link(const typename Stage<S>::C* lk, int vb, int mu, int l) {
-  const typename Stage<S>::C* p = lk + (size_t)mu * 9 * vb;
-  SU3<float> U;
-#pragma unroll
-  for (int k = 0; k < 9; k++) U.m[k / 3][k % 3] = Stage<S>::getc(p[(size_t)k * vb + l]);
-  return U;
-}
-
-template <typename S>
-__device__ inline Spinor<float> smem_clover_apply(const typename Stage<S>::W* cl, int vb, int l,
-                                                  const Spinor<float>& p) {
-  Spinor<float> o;
-#pragma unroll
-  for (int b = 0; b < 2; b++) {
-    float c[36];
-#pragma unroll
-    for (int k = 0; k < 9; k++) {
-      float4 v = Stage<S>::get(cl[(size_t)(9 * b + k) * vb + l]);
-      c[4 * k] = v.x; c[4 * k + 1] = v.y; c[4 * k + 2] = v.z; c[4 * k + 3] = v.w;
-    }
-    clover_block_apply(c, 0, &p.c[6 * b], &o.c[6 * b]);
-  }
-  return o;
 }
 
 template <typename S, bool BF, int MU>
-__device__ inline void smem_block_hop(Spinor<float>& p, const typename RStore<BF>::T* r_s,
-                                      const typename Stage<S>::C* lk, const SapGeom& sg, int l, const int lc[4],
-                                      float scale) {
-  if (lc[MU] < sg.b[MU] - 1) {
-    HalfSpinor<float> h = project<MU, -1>(rs_load<BF>(r_s, sg.vb, l + sg.lst[MU]));
-    h = su3_mul(smem_link<S>(lk, sg.vb, MU, l), h);
-    accum_recon<MU, -1>(p, h, scale);
+__device__ __forceinline__ void block_hops(PairSpinor& p, const void* r_s, const BlockFields& f, const SapGeom& sg,
+                                           const Geom& g, int s, int l, const int lc[4], float scale) {
+  if (lc[MU] < sg.b[MU] - 1)
+    block_hop_pair<S, BF, MU, -1, false>(p, r_s, f, g.V, sg.vb, l + sg.lst[MU], l, s, scale);
+  if (lc[MU] > 0)
+    block_hop_pair<S, BF, MU, +1, true>(p, r_s, f, g.V, sg.vb, l - sg.lst[MU], l - sg.lst[MU], s - g.stride[MU],
+                                        scale);
+}
+
+// n_mr minimal-residual steps on a block from x = 0: r the site's residual (in
+// r_s too, behind a barrier that this function begins with), x the increment
+template <typename S, bool BF>
+__device__ __forceinline__ void mr_steps(PairSpinor& r, PairSpinor& x, void* r_s, const BlockFields& f,
+                                         const SapGeom& sg, const Geom& g, int s, int l, const int lc[4], float kappa,
+                                         int nmr, float4* red) {
+  const int vb = sg.vb;
+#pragma unroll
+  for (int b = 0; b < 2; b++)
+#pragma unroll
+    for (int a = 0; a < 3; a++) x.re[b][a] = x.im[b][a] = p2(0.f, 0.f);
+  const int warp = l >> 5, lane = l & 31, nw = (vb + 31) >> 5;
+  for (int step = 0; step < nmr; step++) {
+    __syncthreads();
+    PairSpinor p;
+    block_clover<S>(f, g.V, s, vb, l, r, p);
+    block_hops<S, BF, 0>(p, r_s, f, sg, g, s, l, lc, -kappa);
+    block_hops<S, BF, 1>(p, r_s, f, sg, g, s, l, lc, -kappa);
+    block_hops<S, BF, 2>(p, r_s, f, sg, g, s, l, lc, -kappa);
+    block_hops<S, BF, 3>(p, r_s, f, sg, g, s, l, lc, -kappa);
+    float2 prr = p2(0.f, 0.f), pri = p2(0.f, 0.f), ppp = p2(0.f, 0.f);
+#pragma unroll
+    for (int b = 0; b < 2; b++)
+#pragma unroll
+      for (int a = 0; a < 3; a++) {
+        prr = pfma(p.re[b][a], r.re[b][a], prr);
+        prr = pfma(p.im[b][a], r.im[b][a], prr);
+        pri = pfma(p.re[b][a], r.im[b][a], pri);
+        pri = pfma(pneg(p.im[b][a]), r.re[b][a], pri);
+        ppp = pfma(p.re[b][a], p.re[b][a], ppp);
+        ppp = pfma(p.im[b][a], p.im[b][a], ppp);
+      }
+    const float pr_re = warp_sum(prr.x + prr.y), pr_im = warp_sum(pri.x + pri.y), pp = warp_sum(ppp.x + ppp.y);
+    if (lane == 0) red[warp] = make_float4(pr_re, pr_im, pp, 0.f);
+    __syncthreads();
+    float a_re = 0, a_im = 0, n2 = 0;
+    for (int w = 0; w < nw; w++) {
+      const float4 v = red[w];
+      a_re += v.x;
+      a_im += v.y;
+      n2 += v.z;
+    }
+    // a quotient, not a reciprocal: far from a point source both sums can be
+    // denormal, where 1 / n2 overflows but a_re / n2 stays finite
+    const float al_re = n2 > 0.f ? a_re / n2 : 0.f, al_im = n2 > 0.f ? a_im / n2 : 0.f;
+#pragma unroll
+    for (int b = 0; b < 2; b++)
+#pragma unroll
+      for (int a = 0; a < 3; a++) {
+        x.re[b][a] = pfma(pbc(al_re), r.re[b][a], x.re[b][a]);
+        x.re[b][a] = pfma(pbc(-al_im), r.im[b][a], x.re[b][a]);
+        x.im[b][a] = pfma(pbc(al_re), r.im[b][a], x.im[b][a]);
+        x.im[b][a] = pfma(pbc(al_im), r.re[b][a], x.im[b][a]);
+        r.re[b][a] = pfma(pbc(-al_re), p.re[b][a], r.re[b][a]);
+        r.re[b][a] = pfma(pbc(al_im), p.im[b][a], r.re[b][a]);
+        r.im[b][a] = pfma(pbc(-al_re), p.im[b][a], r.im[b][a]);
+        r.im[b][a] = pfma(pbc(-al_im), p.re[b][a], r.im[b][a]);
+      }
+    // every thread read its neighbours' residual for p before the barrier
+    // above, so the new residual can be stored now; the next step's first
+    // barrier orders the store (and the reads of red[]) before any later use
+    if (step + 1 < nmr) rs_store<BF>(r_s, vb, l, r);
   }
-  if (lc[MU] > 0) {
-    HalfSpinor<float> h = project<MU, +1>(rs_load<BF>(r_s, sg.vb, l - sg.lst[MU]));
-    h = su3_dag_mul(smem_link<S>(lk, sg.vb, MU, l - sg.lst[MU]), h);
-    accum_recon<MU, +1>(p, h, scale);
+}
+
+// r += scale * (hop from delta at lattice site sn over link MU of site sl)
+template <int MU, int SIGN, bool DAG>
+__device__ __forceinline__ void delta_hop(PairSpinor& r, const char* delta, const float4* gauge, int V, int sn, int sl,
+                                          float scale) {
+  const PairSpinor d = pair_load(delta, V, sn);
+  const float4* lk = gauge + (size_t)3 * MU * V + sl;
+  const LinkRows U = link_rows(__ldg(lk), __ldg(lk + V), __ldg(lk + 2 * (size_t)V));
+  pair_hop<MU, SIGN, DAG>(r, [&](int q) { return pair_rec(d, q); }, [&](int k) { return U.m[k]; }, scale);
+}
+
+// the boundary term of one direction for this thread's own site
+template <int MU>
+__device__ __forceinline__ void own_gather_dir(PairSpinor& r, const SapGeom& sg, const Geom& g, const char* delta,
+                                               const float4* gauge, int s, const int c[4], const int lc[4],
+                                               float kappa) {
+  if (lc[MU] == sg.b[MU] - 1)
+    delta_hop<MU, -1, false>(r, delta, gauge, g.V, site_fwd(g, s, c, MU), s,
+                             (MU == 0 && c[0] == g.L[0] - 1) ? (float)g.bc_t * kappa : kappa);
+  if (lc[MU] == 0) {
+    const int sb = site_bwd(g, s, c, MU);
+    delta_hop<MU, +1, true>(r, delta, gauge, g.V, sb, sb, (MU == 0 && c[0] == 0) ? (float)g.bc_t * kappa : kappa);
   }
 }
 
@@ -362,7 +468,7 @@ __device__ inline void smem_block_hop(Spinor<float>& p, const typename RStore<BF
 // site's residual is read, updated and written back by that thread, in the
 // same arithmetic as a per-site update.  co: the block's first site.
 template <int MU>
-__device__ inline void smem_gather_dir(Cplx<float>* r_s, const SapGeom& sg, const Geom& g, const char* delta,
+__device__ inline void smem_gather_dir(void* r_s, const SapGeom& sg, const Geom& g, const char* delta,
                                        const float4* gauge, const int co[4], int l, float kappa) {
   const int nface = sg.vb / sg.b[MU];
   if (l >= 2 * nface) return;
@@ -383,49 +489,51 @@ __device__ inline void smem_gather_dir(Cplx<float>* r_s, const SapGeom& sg, cons
 #pragma unroll
   for (int mu = 0; mu < 4; mu++) c[mu] = co[mu] + lc[mu];
   const int s = ((c[0] * g.L[3] + c[3]) * g.L[2] + c[2]) * g.L[1] + c[1];
-  Spinor<float> r = rs_load<false>(r_s, sg.vb, ls);
+  PairSpinor r;
+#pragma unroll
+  for (int q = 0; q < 6; q++) {
+    const float4 v = rs_rec<false>(r_s, sg.vb, ls, q);
+    r.re[q / 3][q % 3] = p2(v.x, v.y);
+    r.im[q / 3][q % 3] = p2(v.z, v.w);
+  }
   if (fwd) {
-    const int sf = site_fwd(g, s, c, MU);
-    const float sign = (MU == 0 && c[0] == g.L[0] - 1) ? (float)g.bc_t * kappa : kappa;
-    HalfSpinor<float> h = project<MU, -1>(FieldsF::load_spinor(delta, g.V, sf));
-    h = su3_mul(FieldsF::load_link(gauge, g.V, MU, s), h);
-    accum_recon<MU, -1>(r, h, sign);
+    delta_hop<MU, -1, false>(r, delta, gauge, g.V, site_fwd(g, s, c, MU), s,
+                             (MU == 0 && c[0] == g.L[0] - 1) ? (float)g.bc_t * kappa : kappa);
   } else {
     const int sb = site_bwd(g, s, c, MU);
-    const float sign = (MU == 0 && c[0] == 0) ? (float)g.bc_t * kappa : kappa;
-    HalfSpinor<float> h = project<MU, +1>(FieldsF::load_spinor(delta, g.V, sb));
-    h = su3_dag_mul(FieldsF::load_link(gauge, g.V, MU, sb), h);
-    accum_recon<MU, +1>(r, h, sign);
+    delta_hop<MU, +1, true>(r, delta, gauge, g.V, sb, sb, (MU == 0 && c[0] == 0) ? (float)g.bc_t * kappa : kappa);
   }
   rs_store<false>(r_s, sg.vb, ls, r);
 }
 
-// B4 = true: the block is 4^4, known at compile time, so every shared-memory
-// offset (component stride vb, neighbour strides) is an immediate.
-template <typename S, bool BF, bool B4, int MAXT, int MINB>
+// the blk-th block of a colour
+__device__ __forceinline__ void block_of(const SapGeom& sg, int colour, int blk, int bc[4]) {
+  const int nbx2 = sg.nb[1] >> 1;
+  int q = blk / nbx2;
+  const int j = blk - q * nbx2;
+  bc[2] = q % sg.nb[2];
+  q /= sg.nb[2];
+  bc[3] = q % sg.nb[3];
+  bc[0] = q / sg.nb[3];
+  bc[1] = 2 * j + ((colour + bc[0] + bc[3] + bc[2]) & 1);
+}
+// its number within its colour
+__device__ __forceinline__ int block_number(const SapGeom& sg, const int bc[4]) {
+  return ((bc[0] * sg.nb[3] + bc[3]) * sg.nb[2] + bc[2]) * (sg.nb[1] >> 1) + (bc[1] >> 1);
+}
+
+// Any block shape: rho, psi and delta in the lexicographic layout.  img: the
+// block image of S.
+template <typename S, bool BF, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
-    k_sap_sweep_smem(const char* __restrict__ rho_src, char* __restrict__ rho, char* __restrict__ psi,
-                     char* __restrict__ delta,
-                     const float4* __restrict__ gauge, const float4* __restrict__ clover,
-                     const uint4* __restrict__ gaugeH, const uint4* __restrict__ cloverH, Geom g, SapGeom sg_in,
-                     int colour, int gather, int psi_init, float kappa, int nmr, int nrhs, const int* mask) {
-  SapGeom sg = sg_in;
-  if (B4) {
-    sg.b[0] = sg.b[1] = sg.b[2] = sg.b[3] = 4;
-    sg.lst[1] = 1;
-    sg.lst[2] = 4;
-    sg.lst[3] = 16;
-    sg.lst[0] = 64;
-    sg.vb = 256;
-  }
-  using W = typename Stage<S>::W;
-  using CW = typename Stage<S>::C;
+    k_sap_sweep_pair(const char* __restrict__ rho_src, char* __restrict__ rho, char* __restrict__ psi,
+                     char* __restrict__ delta, const float4* __restrict__ gauge, const float4* __restrict__ clover,
+                     const unsigned char* __restrict__ img, Geom g, SapGeom sg, int colour, int gather, int psi_init,
+                     int last, float kappa, int nmr, int nrhs, const int* mask) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int vb = sg.vb;
-  using RT = typename RStore<BF>::T;
-  RT* r_s = (RT*)smem_raw;
-  CW* lk_s = (CW*)(smem_raw + (size_t)12 * vb * sizeof(RT));              // [4][9][vb]
-  W* cl_s = (W*)(lk_s + (size_t)36 * vb);                                 // [18][vb]
+  void* r_s = smem_raw;
+  unsigned char* lk_s = smem_raw + (size_t)vb * (BF ? 48 : 96);
   __shared__ float4 red[32];   // per warp: (p, r) re, im, (p, p)
 
   const int rhs = blockIdx.x % nrhs;   // RHS fastest, as in k_sap_sweep
@@ -437,15 +545,8 @@ __global__ void __launch_bounds__(MAXT, MINB)
   psi += off;
   delta += off;
 
-  const int nbx2 = sg.nb[1] >> 1;
-  int q = blk / nbx2;
-  const int j = blk - q * nbx2;
-  const int by = q % sg.nb[2];
-  q /= sg.nb[2];
-  const int bz = q % sg.nb[3];
-  const int bt = q / sg.nb[3];
-  const int bx = 2 * j + ((colour + bt + bz + by) & 1);
-
+  int bc[4];
+  block_of(sg, colour, blk, bc);
   const int l = threadIdx.x;
   int lc[4], c[4];
   {
@@ -455,132 +556,427 @@ __global__ void __launch_bounds__(MAXT, MINB)
     lc[3] = r % sg.b[3];
     lc[0] = r / sg.b[3];
   }
-  c[0] = bt * sg.b[0] + lc[0];
-  c[1] = bx * sg.b[1] + lc[1];
-  c[2] = by * sg.b[2] + lc[2];
-  c[3] = bz * sg.b[3] + lc[3];
+#pragma unroll
+  for (int mu = 0; mu < 4; mu++) c[mu] = bc[mu] * sg.b[mu] + lc[mu];
   const int s = ((c[0] * g.L[3] + c[3]) * g.L[2] + c[2]) * g.L[1] + c[1];
 
-  // stage this site's four links (full 3x3) and its clover term: 16-bit
-  // copies straight from their FP16 copies in HBM (rounded once at gauge
-  // load, as the FP32 path rounds them here), FP32 copies from the FP32 fields
-  if (std::is_same<S, __half>::value) {
-    const uint4* gB = gaugeH + 4 * (size_t)g.V;
-    const unsigned* gC = (const unsigned*)(gB + 4 * (size_t)g.V);
-    unsigned* lw = (unsigned*)lk_s;
+  BlockFields f = {nullptr, nullptr, gauge, clover};
+  const size_t bidx = (size_t)colour * (gridDim.x / nrhs) + blk;
+  if constexpr (std::is_same<S, __half>::value) {
+    img += bidx * 288 * vb;
 #pragma unroll
-    for (int mu = 0; mu < 4; mu++) {
-      const uint4 a = __ldg(gaugeH + (size_t)mu * g.V + s), b = __ldg(gB + (size_t)mu * g.V + s);
-      const unsigned h8 = __ldg(gC + (size_t)mu * g.V + s);
-      const unsigned w[9] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, h8};
+    for (int k = 0; k < 18; k++) cp_async16(lk_s + 16 * (k * vb + l), img + 16 * (k * vb + l));
+    f.lk = lk_s;
+    f.cl = lk_s + 144 * vb;
+  } else if constexpr (!std::is_same<S, FromField>::value) {
+    img += bidx * 480 * vb;
+    f.lk = img;
+    f.cl = img + 192 * vb;
+    if constexpr (std::is_same<S, float>::value) {
 #pragma unroll
-      for (int k = 0; k < 9; k++) lw[(size_t)(9 * mu + k) * vb + l] = w[k];
+      for (int k = 0; k < 12; k++) cp_async16(lk_s + 16 * (k * vb + l), img + 16 * (k * vb + l));
+      f.lk = lk_s;
     }
-    uint2* cw = (uint2*)cl_s;
-#pragma unroll
-    for (int k = 0; k < 9; k++) {
-      const uint4 v = __ldg(cloverH + (size_t)k * g.V + s);
-      cw[(size_t)(2 * k) * vb + l] = make_uint2(v.x, v.y);
-      cw[(size_t)(2 * k + 1) * vb + l] = make_uint2(v.z, v.w);
-    }
-  } else {
-#pragma unroll
-    for (int mu = 0; mu < 4; mu++) {
-      SU3<float> U = FieldsF::load_link(gauge, g.V, mu, s);
-#pragma unroll
-      for (int k = 0; k < 9; k++) lk_s[(size_t)(9 * mu + k) * vb + l] = Stage<S>::putc(U.m[k / 3][k % 3]);
-    }
-#pragma unroll
-    for (int k = 0; k < 18; k++) cl_s[(size_t)k * vb + l] = Stage<S>::put(__ldg(clover + (size_t)k * g.V + s));
   }
 
-  Spinor<float> r = FieldsF::load_spinor(rho_src, g.V, s);
-  if (BF) {
-    // bf16 shared residual: the site's own residual stays FP32 in registers
+  PairSpinor r = pair_load(rho_src, g.V, s);
+  if (BF || Stage<S>::bytes == 0) {
+    // the site's own residual stays FP32 in registers
     if (gather) {
-      face_hop<FieldsF, 0>(r, delta, sg, gauge, g, s, c, lc, kappa);
-      face_hop<FieldsF, 1>(r, delta, sg, gauge, g, s, c, lc, kappa);
-      face_hop<FieldsF, 2>(r, delta, sg, gauge, g, s, c, lc, kappa);
-      face_hop<FieldsF, 3>(r, delta, sg, gauge, g, s, c, lc, kappa);
+      own_gather_dir<0>(r, sg, g, delta, gauge, s, c, lc, kappa);
+      own_gather_dir<1>(r, sg, g, delta, gauge, s, c, lc, kappa);
+      own_gather_dir<2>(r, sg, g, delta, gauge, s, c, lc, kappa);
+      own_gather_dir<3>(r, sg, g, delta, gauge, s, c, lc, kappa);
     }
     rs_store<BF>(r_s, vb, l, r);
   } else {
     rs_store<BF>(r_s, vb, l, r);
     if (gather) {
       // boundary term in four rounds (one direction each, both faces at once)
-      Cplx<float>* rf = (Cplx<float>*)r_s;
       const int co[4] = {c[0] - lc[0], c[1] - lc[1], c[2] - lc[2], c[3] - lc[3]};
       __syncthreads();
-      smem_gather_dir<0>(rf, sg, g, delta, gauge, co, l, kappa);
+      smem_gather_dir<0>(r_s, sg, g, delta, gauge, co, l, kappa);
       __syncthreads();
-      smem_gather_dir<1>(rf, sg, g, delta, gauge, co, l, kappa);
+      smem_gather_dir<1>(r_s, sg, g, delta, gauge, co, l, kappa);
       __syncthreads();
-      smem_gather_dir<2>(rf, sg, g, delta, gauge, co, l, kappa);
+      smem_gather_dir<2>(r_s, sg, g, delta, gauge, co, l, kappa);
       __syncthreads();
-      smem_gather_dir<3>(rf, sg, g, delta, gauge, co, l, kappa);
+      smem_gather_dir<3>(r_s, sg, g, delta, gauge, co, l, kappa);
       __syncthreads();
-      r = rs_load<BF>(r_s, vb, l);
+#pragma unroll
+      for (int k = 0; k < 6; k++) {
+        const float4 v = rs_rec<BF>(r_s, vb, l, k);
+        r.re[k / 3][k % 3] = p2(v.x, v.y);
+        r.im[k / 3][k % 3] = p2(v.z, v.w);
+      }
     }
   }
+  cp_async_wait();   // this thread's copies; the barrier of the first MR step covers the others'
 
-  Spinor<float> x;
-#pragma unroll
-  for (int k = 0; k < 12; k++) x.c[k] = cmk(0.f, 0.f);
-
-  const int warp = l >> 5, lane = l & 31, nw = (vb + 31) >> 5;
-  for (int step = 0; step < nmr; step++) {
-    __syncthreads();
-    Spinor<float> p = smem_clover_apply<S>(cl_s, vb, l, r);
-    smem_block_hop<S, BF, 0>(p, r_s, lk_s, sg, l, lc, -kappa);
-    smem_block_hop<S, BF, 1>(p, r_s, lk_s, sg, l, lc, -kappa);
-    smem_block_hop<S, BF, 2>(p, r_s, lk_s, sg, l, lc, -kappa);
-    smem_block_hop<S, BF, 3>(p, r_s, lk_s, sg, l, lc, -kappa);
-    Cplx<float> pr = cmk(0.f, 0.f);
-    float pp = 0;
-#pragma unroll
-    for (int k = 0; k < 12; k++) {
-      cmac_conj(pr, p.c[k], r.c[k]);
-      pp = fmaf(p.c[k].re, p.c[k].re, pp);
-      pp = fmaf(p.c[k].im, p.c[k].im, pp);
-    }
-    float pr_re = pr.re, pr_im = pr.im;
-    pr_re = warp_sum(pr_re);
-    pr_im = warp_sum(pr_im);
-    pp = warp_sum(pp);
-    if (lane == 0) red[warp] = make_float4(pr_re, pr_im, pp, 0.f);
-    __syncthreads();
-    float a_re = 0, a_im = 0, n2 = 0;
-    for (int w = 0; w < nw; w++) {
-      const float4 v = red[w];
-      a_re += v.x;
-      a_im += v.y;
-      n2 += v.z;
-    }
-    // a quotient, not a reciprocal: far from a point source both sums can be
-    // denormal, where 1 / n2 overflows but a_re / n2 stays finite
-    Cplx<float> alpha = n2 > 0.f ? cmk(a_re / n2, a_im / n2) : cmk(0.f, 0.f);
-    const Cplx<float> malpha = -alpha;
-#pragma unroll
-    for (int k = 0; k < 12; k++) {
-      cmac(x.c[k], alpha, r.c[k]);
-      cmac(r.c[k], malpha, p.c[k]);
-    }
-    // every thread read its neighbours' residual for p before the barrier
-    // above, so the new residual can be stored now; the next step's first
-    // barrier orders the store (and the reads of red[]) before any later use
-    rs_store<BF>(r_s, vb, l, r);
-  }
+  PairSpinor x;
+  mr_steps<S, BF>(r, x, r_s, f, sg, g, s, l, lc, kappa, nmr, red);
 
   if (psi_init) {
-    FieldsF::store_spinor(psi, g.V, s, x);
+    pair_store(psi, g.V, s, x);
   } else {
-    Spinor<float> y = FieldsF::load_spinor(psi, g.V, s);
-#pragma unroll
-    for (int k = 0; k < 12; k++) y.c[k] = y.c[k] + x.c[k];
-    FieldsF::store_spinor(psi, g.V, s, y);
+    PairSpinor y = pair_load(psi, g.V, s);
+    pair_add(y, x);
+    pair_store(psi, g.V, s, y);
   }
-  FieldsF::store_spinor(rho, g.V, s, r);
-  FieldsF::store_spinor(delta, g.V, s, x);
+  // the last cycle's residuals and the last half-cycle's delta have no reader
+  if (last < 1) pair_store(rho, g.V, s, r);
+  if (last < 2) pair_store(delta, g.V, s, x);
+}
+
+// 4^4 blocks.  Between the first and the last cycle everything a CTA reads and
+// writes is a contiguous run of its block:
+//   rho_b, psi_b  [rhs][block][record q][256] float4, the residual and the sum
+//                 of the increments (the first cycle reads the caller's
+//                 lexicographic residual, the last one writes its psi);
+//   faces         what the neighbours of the other colour need of delta: per
+//                 block of a colour, face f = 2 mu + side (side 0: the sites at
+//                 -mu, 1: at +mu) and colour a the half spinors of the 64 face
+//                 sites, [rhs][colour][block][8][3][64] float4, projected with
+//                 1 - gamma_mu (side 0, for the block at -mu) or 1 + gamma_mu;
+//   flinks        the FP32 links across a block's own faces in the same order,
+//                 [block][8][link row word 3][64] float4.
+// Boundary term: 8 faces x 64 sites are 16 tasks of a warp, two per warp (warp
+// w: side (w >> 1) & 1, half w & 1, mu = w >> 2 and 2 + (w >> 2)): read the
+// neighbour's half spinor and the link, multiply, leave the product in shared
+// memory; after a barrier every site adds those of the faces it lies on, in the
+// order t, x, y, z.  The products take the block residual's place before it is
+// stored.  All loads of a CTA are issued before the first wait.
+//
+// Bound by the FP32 pipe: per site and MR step 1,242 multiply-adds of the operator
+// and the MR update and 207 conversions of 16-bit words, which only half of the
+// pipe takes.  Measured against the same sweep on lexicographic vectors in
+// scalar arithmetic: 32^3x64, 12 RHS, 16-bit copies 44.4 -> 33.7 ms per
+// application (5 cycles); 24^3x48, one RHS, FP32 copies 225 -> 119 us per
+// half-cycle.  (Two-lane arithmetic alone, still loading lexicographic pieces, gave
+// nothing: the loads were the bound.)
+struct SapB4 {
+  const char* rho_src;
+  float4 *rho_b, *psi_b, *faces;
+  char* psi;
+  const unsigned char* img;
+  const float4* flinks;
+  int colour, gather, first, last, accumulate;   // last: 1 the last cycle, 2 its second half
+};
+
+template <int MU>
+__device__ __forceinline__ int face_site_of(int l) {   // index of site l on a mu face (the other three coordinates)
+  return MU == 0 ? (l & 63) : MU == 1 ? (l >> 2) : MU == 2 ? ((l & 3) | ((l >> 4) << 2)) : ((l & 15) | ((l >> 6) << 4));
+}
+template <int MU>
+__device__ __forceinline__ void face_add(PairSpinor& r, const float4* buf, const Geom& g, int t, const int lc[4], int l,
+                                         float kappa) {
+  const int tf = face_site_of<MU>(l);
+  if (lc[MU] == 3) {
+    const float s = (MU == 0 && t == g.L[0] - 1) ? (float)g.bc_t * kappa : kappa;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+      const float4 v = buf[(3 * (2 * MU + 1) + a) * 64 + tf];
+      pair_recon<MU, -1>(r, a, p2(v.x, v.y), p2(v.z, v.w), s);
+    }
+  }
+  if (lc[MU] == 0) {
+    const float s = (MU == 0 && t == 0) ? (float)g.bc_t * kappa : kappa;
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+      const float4 v = buf[(3 * (2 * MU) + a) * 64 + tf];
+      pair_recon<MU, +1>(r, a, p2(v.x, v.y), p2(v.z, v.w), s);
+    }
+  }
+}
+// the projections of delta = x the neighbours will read
+template <int MU>
+__device__ __forceinline__ void face_store(float4* out, const PairSpinor& x, const int lc[4], int l) {
+  const int tf = face_site_of<MU>(l);
+  float2 hr, hi;
+  if (lc[MU] == 0) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+      pair_project<MU, -1>(x.re[0][a], x.im[0][a], x.re[1][a], x.im[1][a], hr, hi);
+      out[(3 * (2 * MU) + a) * 64 + tf] = make_float4(hr.x, hr.y, hi.x, hi.y);
+    }
+  }
+  if (lc[MU] == 3) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+      pair_project<MU, +1>(x.re[0][a], x.im[0][a], x.re[1][a], x.im[1][a], hr, hi);
+      out[(3 * (2 * MU + 1) + a) * 64 + tf] = make_float4(hr.x, hr.y, hi.x, hi.y);
+    }
+  }
+}
+// U h (side 1) or U^+ h (side 0) of a half spinor in three records
+__device__ __forceinline__ void face_mul(const float4 (&h)[3], const float4 (&u)[3], int side, float4* out) {
+  const LinkRows U = link_rows(u[0], u[1], u[2]);
+  auto mul = [&](auto link) {
+#pragma unroll
+    for (int a = 0; a < 3; a++) {
+      float2 gr = p2(0.f, 0.f), gi = p2(0.f, 0.f);
+#pragma unroll
+      for (int b = 0; b < 3; b++) {
+        const float2 w = link(a, b), hr = p2(h[b].x, h[b].y), hi = p2(h[b].z, h[b].w);
+        gr = pfma(pbc(w.x), hr, gr);
+        gr = pfma(pbc(-w.y), hi, gr);
+        gi = pfma(pbc(w.x), hi, gi);
+        gi = pfma(pbc(w.y), hr, gi);
+      }
+      out[a * 64] = make_float4(gr.x, gr.y, gi.x, gi.y);
+    }
+  };
+  if (side) mul([&](int a, int b) { return U.m[3 * a + b]; });
+  else mul([&](int a, int b) { return p2(U.m[3 * b + a].x, -U.m[3 * b + a].y); });
+}
+
+template <typename S, bool BF>
+__global__ void __launch_bounds__(256, 2)
+    k_sap_sweep_b4(SapB4 A, Geom g, SapGeom sg, float kappa, int nmr, int nrhs, const int* mask) {
+  sg.b[0] = sg.b[1] = sg.b[2] = sg.b[3] = 4;
+  sg.lst[1] = 1;
+  sg.lst[2] = 4;
+  sg.lst[3] = 16;
+  sg.lst[0] = 64;
+  sg.vb = 256;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  void* r_s = smem_raw;                          // 24 KB: boundary products, then the residual
+  unsigned char* lk_s = smem_raw + 96 * 256;
+  __shared__ float4 red[8];
+
+  const int rhs = blockIdx.x % nrhs;   // RHS fastest, as in k_sap_sweep
+  const int blk = blockIdx.x / nrhs;
+  if (mask && !mask[rhs]) return;
+  const int nhalf = gridDim.x / nrhs;
+  const size_t bidx = (size_t)A.colour * nhalf + blk;
+  const int l = threadIdx.x;
+
+  BlockFields f = {lk_s, lk_s + 144 * 256, nullptr, nullptr};
+  {
+    const unsigned char* img = A.img + bidx * (size_t)((std::is_same<S, __half>::value ? 288 : 480) * 256);
+#pragma unroll
+    for (int k = 0; k < (std::is_same<S, __half>::value ? 18 : 12); k++)
+      cp_async16(lk_s + 16 * (k * 256 + l), img + 16 * (k * 256 + l));
+    if (!std::is_same<S, __half>::value) f.cl = img + 192 * 256;
+  }
+  const size_t voff = ((size_t)rhs * 2 * nhalf + bidx) * 6 * 256 + l;   // block-ordered vectors
+  float4* rho_b = A.rho_b + voff;
+  float4* psi_b = A.psi_b + voff;
+  if (!A.first) {
+#pragma unroll
+    for (int q = 0; q < 6; q++) prefetch_l2(psi_b + q * 256);
+  }
+
+  int bc[4];
+  block_of(sg, A.colour, blk, bc);
+  const int lc[4] = {l >> 6, l & 3, (l >> 2) & 3, (l >> 4) & 3};
+  const int t = 4 * bc[0] + lc[0];
+  const int s = ((t * g.L[3] + 4 * bc[3] + lc[3]) * g.L[2] + 4 * bc[2] + lc[2]) * g.L[1] + 4 * bc[1] + lc[1];
+
+  float4 rw[6];
+  if (A.first) {
+    load_words(A.rho_src + (size_t)rhs * FieldsF::spinor_bytes * g.V, g.V, s, rw);
+  } else {
+#pragma unroll
+    for (int q = 0; q < 6; q++) rw[q] = rho_b[q * 256];
+  }
+  auto residual = [&]() {
+    if (A.first) return pair_from_words(rw);
+    PairSpinor o;
+#pragma unroll
+    for (int q = 0; q < 6; q++) {
+      o.re[q / 3][q % 3] = p2(rw[q].x, rw[q].y);
+      o.im[q / 3][q % 3] = p2(rw[q].z, rw[q].w);
+    }
+    return o;
+  };
+  PairSpinor r;
+  if (A.gather) {
+    float4* buf = (float4*)r_s;
+    const int w = l >> 5, side = (w >> 1) & 1, tf = ((w & 1) << 5) | (l & 31);
+    float4 h[2][3], u[2][3];
+#pragma unroll
+    for (int i = 0; i < 2; i++) {
+      const int mu = 2 * i + (w >> 2);
+      int nbc[4] = {bc[0], bc[1], bc[2], bc[3]};
+#pragma unroll
+      for (int m = 0; m < 4; m++)
+        if (m == mu) nbc[m] = side ? (bc[m] == sg.nb[m] - 1 ? 0 : bc[m] + 1) : (bc[m] == 0 ? sg.nb[m] - 1 : bc[m] - 1);
+      const float4* hp =
+          A.faces + (((size_t)rhs * 2 + 1 - A.colour) * nhalf + block_number(sg, nbc)) * 1536 + (2 * mu + 1 - side) * 192 + tf;
+      const float4* up = A.flinks + bidx * 1536 + (2 * mu + side) * 192 + tf;
+#pragma unroll
+      for (int a = 0; a < 3; a++) {
+        h[i][a] = hp[a * 64];
+        u[i][a] = __ldg(up + a * 64);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 2; i++) face_mul(h[i], u[i], side, buf + (2 * (2 * i + (w >> 2)) + side) * 192 + tf);
+    __syncthreads();
+    r = residual();
+    face_add<0>(r, buf, g, t, lc, l, kappa);
+    face_add<1>(r, buf, g, t, lc, l, kappa);
+    face_add<2>(r, buf, g, t, lc, l, kappa);
+    face_add<3>(r, buf, g, t, lc, l, kappa);
+    __syncthreads();   // the products are read before the residual takes their place
+  } else {
+    r = residual();
+  }
+  rs_store<BF>(r_s, 256, l, r);
+  cp_async_wait();   // this thread's copies; the barrier of the first MR step covers the others'
+
+  PairSpinor x;
+  mr_steps<S, BF>(r, x, r_s, f, sg, g, s, l, lc, kappa, nmr, red);
+
+  if (A.last < 2) {
+    float4* out = A.faces + (((size_t)rhs * 2 + A.colour) * nhalf + blk) * 1536;
+    face_store<0>(out, x, lc, l);
+    face_store<1>(out, x, lc, l);
+    face_store<2>(out, x, lc, l);
+    face_store<3>(out, x, lc, l);
+  }
+  if (A.last < 1) {
+#pragma unroll
+    for (int q = 0; q < 6; q++) rho_b[q * 256] = pair_rec(r, q);
+  }
+  if (!A.first) {
+    PairSpinor y;
+#pragma unroll
+    for (int q = 0; q < 6; q++) {
+      const float4 v = psi_b[q * 256];
+      y.re[q / 3][q % 3] = p2(v.x, v.y);
+      y.im[q / 3][q % 3] = p2(v.z, v.w);
+    }
+    pair_add(x, y);
+  }
+  if (A.last < 1) {
+#pragma unroll
+    for (int q = 0; q < 6; q++) psi_b[q * 256] = pair_rec(x, q);
+  } else {
+    char* psi = A.psi + (size_t)rhs * FieldsF::spinor_bytes * g.V;
+    if (A.accumulate) pair_add(x, pair_load(psi, g.V, s));
+    pair_store(psi, g.V, s, x);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// The block images (built when a sweep first needs them, again after a new
+// gauge field or block shape).  One thread per site, in image order.
+// ---------------------------------------------------------------------------
+template <typename S>
+__global__ void k_block_image(const float4* __restrict__ gauge, const float4* __restrict__ clover, Geom g, SapGeom sg,
+                              unsigned char* __restrict__ img) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= g.V) return;
+  const int bidx = i / sg.vb, l = i - bidx * sg.vb, nhalf = g.V / sg.vb / 2, vb = sg.vb;
+  int bc[4], r = l;
+  block_of(sg, bidx >= nhalf, bidx >= nhalf ? bidx - nhalf : bidx, bc);
+  const int x = r % sg.b[1]; r /= sg.b[1];
+  const int y = r % sg.b[2]; r /= sg.b[2];
+  const int z = r % sg.b[3], t = r / sg.b[3];
+  const int s = (((bc[0] * sg.b[0] + t) * g.L[3] + bc[3] * sg.b[3] + z) * g.L[2] + bc[2] * sg.b[2] + y) * g.L[1] +
+                bc[1] * sg.b[1] + x;
+  if constexpr (std::is_same<S, __half>::value) {
+    img += (size_t)bidx * 288 * vb;
+    uint4* o = (uint4*)img;
+    unsigned* o8 = (unsigned*)(o + 8 * vb);
+#pragma unroll
+    for (int mu = 0; mu < 4; mu++) {
+      const SU3<float> U = FieldsF::load_link(gauge, g.V, mu, s);
+      unsigned h[9];
+#pragma unroll
+      for (int k = 0; k < 9; k++) h[k] = h2_bits(__floats2half2_rn(U.m[k / 3][k % 3].re, U.m[k / 3][k % 3].im));
+      o[mu * vb + l] = make_uint4(h[0], h[1], h[2], h[3]);
+      o[(4 + mu) * vb + l] = make_uint4(h[4], h[5], h[6], h[7]);
+      o8[mu * vb + l] = h[8];
+    }
+#pragma unroll
+    for (int k = 0; k < 9; k++) {
+      const float4 a = clover[(size_t)(2 * k) * g.V + s], b = clover[(size_t)(2 * k + 1) * g.V + s];
+      o[(9 + k) * vb + l] =
+          make_uint4(h2_bits(__floats2half2_rn(a.x, a.y)), h2_bits(__floats2half2_rn(a.z, a.w)),
+                     h2_bits(__floats2half2_rn(b.x, b.y)), h2_bits(__floats2half2_rn(b.z, b.w)));
+    }
+  } else {
+    float4* o = (float4*)(img + (size_t)bidx * 480 * vb);
+#pragma unroll
+    for (int k = 0; k < 12; k++) o[k * vb + l] = gauge[(size_t)k * g.V + s];
+#pragma unroll
+    for (int c = 0; c < 2; c++) {
+      float4 h[9];
+#pragma unroll
+      for (int k = 0; k < 9; k++) h[k] = clover[(size_t)(9 * c + k) * g.V + s];
+      const CloverPairs m = clover_pairs(
+          [&](int j) { return (j & 1) ? p2(h[j >> 1].z, h[j >> 1].w) : p2(h[j >> 1].x, h[j >> 1].y); });
+      const float2 w[18] = {m.d[0], m.d[1], m.d[2], m.lr[0], m.lr[1], m.lr[2], m.li[0], m.li[1], m.li[2],
+                            m.e[0], m.e[1], m.e[2], m.orr[0], m.orr[1], m.orr[2], m.oi[0], m.oi[1], m.oi[2]};
+#pragma unroll
+      for (int k = 0; k < 9; k++)
+        o[(12 + 9 * c + k) * vb + l] = make_float4(w[2 * k].x, w[2 * k].y, w[2 * k + 1].x, w[2 * k + 1].y);
+    }
+  }
+}
+
+// flinks of 4^4 blocks: one thread per (block, face, face site)
+__global__ void k_face_links(const float4* __restrict__ gauge, Geom g, SapGeom sg, float4* __restrict__ out) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= (size_t)2 * g.V) return;   // 512 face sites per 256-site block
+  const int bidx = (int)(i >> 9), f = (int)(i >> 6) & 7, tf = (int)i & 63, nhalf = g.V / 512;
+  const int mu = f >> 1, side = f & 1, e = side ? 3 : 0;
+  int bc[4], c[4];
+  block_of(sg, bidx >= nhalf, bidx >= nhalf ? bidx - nhalf : bidx, bc);
+  const int a = tf & 3, b = (tf >> 2) & 3, d = tf >> 4;
+  c[0] = 4 * bc[0] + (mu == 0 ? e : d);
+  c[1] = 4 * bc[1] + (mu == 1 ? e : a);
+  c[2] = 4 * bc[2] + (mu == 2 ? e : mu == 1 ? a : b);
+  c[3] = 4 * bc[3] + (mu == 3 ? e : mu == 0 ? d : b);
+  int s = ((c[0] * g.L[3] + c[3]) * g.L[2] + c[2]) * g.L[1] + c[1];
+  if (!side) s = site_bwd(g, s, c, mu);
+#pragma unroll
+  for (int k = 0; k < 3; k++) out[((size_t)bidx * 24 + 3 * f + k) * 64 + tf] = gauge[(size_t)(3 * mu + k) * g.V + s];
+}
+
+// Brings the context's block image for these blocks up to date; *img = nullptr
+// when there is no memory for it.  flinks only for 4^4 blocks.
+qcd_status block_image(qcd_ctx* c, const SapGeom& sg, bool half, bool faces, const unsigned char** img,
+                       const float4** flinks) {
+  SapImage& m = half ? c->sap_img16 : c->sap_img32;
+  const size_t V = c->g.V;
+  bool same = m.gauge_id == c->gauge_id && m.buf.p;
+  for (int mu = 0; mu < 4; mu++) same = same && m.block[mu] == sg.b[mu];
+  *img = nullptr;
+  if (!same) {
+    m.gauge_id = 0;
+    const qcd_status st = devbuf_ensure(m.buf, V * (half ? 288 : 480));
+    if (st == QCD_ERR_OOM) return QCD_OK;
+    QCD_TRY(st);
+    ProfScope ps(c, FAM_LAYOUT, (double)V * (480 + (half ? 288 : 480)), 0.0);
+    const unsigned grid = (unsigned)((V + 127) / 128);
+    if (half)
+      k_block_image<__half><<<grid, 128, 0, c->stream>>>((const float4*)c->gaugeF.p, (const float4*)c->cloverF.p, c->g,
+                                                         sg, (unsigned char*)m.buf.p);
+    else
+      k_block_image<float><<<grid, 128, 0, c->stream>>>((const float4*)c->gaugeF.p, (const float4*)c->cloverF.p, c->g,
+                                                        sg, (unsigned char*)m.buf.p);
+    QCD_CUDA_OK(cudaGetLastError());
+    for (int mu = 0; mu < 4; mu++) m.block[mu] = sg.b[mu];
+    m.gauge_id = c->gauge_id;
+  }
+  if (faces && c->flinks_id != c->gauge_id) {
+    c->flinks_id = 0;
+    const qcd_status st = devbuf_ensure(c->flinks, V * 96);
+    if (st == QCD_ERR_OOM) return QCD_OK;
+    QCD_TRY(st);
+    ProfScope ps(c, FAM_LAYOUT, (double)V * 192, 0.0);
+    k_face_links<<<(unsigned)((2 * V + 255) / 256), 256, 0, c->stream>>>((const float4*)c->gaugeF.p, c->g, sg,
+                                                                         (float4*)c->flinks.p);
+    QCD_CUDA_OK(cudaGetLastError());
+    c->flinks_id = c->gauge_id;
+  }
+  *img = (const unsigned char*)m.buf.p;
+  if (flinks) *flinks = (const float4*)c->flinks.p;
+  return QCD_OK;
 }
 
 template <typename F>
@@ -599,14 +995,6 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   sg.lst[3] = sg.b[1] * sg.b[2];
   sg.lst[0] = sg.b[1] * sg.b[2] * sg.b[3];
   const int nblocks = sg.nb[0] * sg.nb[1] * sg.nb[2] * sg.nb[3];
-  const size_t smem = (size_t)12 * sg.vb * sizeof(Cplx<typename F::R>);
-  // the register budget per thread follows from the block volume; FP32 fits
-  // 128 registers without spilling, so 256-site blocks run two CTAs per SM
-  constexpr int MINB256 = sizeof(typename F::R) == 4 ? 2 : 1;
-  auto kern = sg.vb <= 256   ? k_sap_sweep<F, 256, MINB256>
-              : sg.vb <= 512 ? k_sap_sweep<F, 512, 1>
-                             : k_sap_sweep<F, 1024, 1>;
-  QCD_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const dim3 grid((unsigned)(nblocks / 2) * (unsigned)nrhs);
   // Algorithmic cost of one half-cycle (the minimum each launch must move):
   // per active site and RHS, rho read and written, psi read and written (only
@@ -627,37 +1015,86 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   const double flops_gather = 165.0 * face;
   const double flops_site = P.nmr * (1320.0 * (1.0 - face / 8.0) + 504.0 + 192.0) + flops_gather;
   const int fam = sizeof(typename F::R) == 8 ? FAM_SAP_D : FAM_SAP_F;
-  // FP32 with blocks of at most 256 sites: the shared-memory-resident kernel
-  const bool resident = sizeof(typename F::R) == 4 && sg.vb <= 256;
+  constexpr bool f32 = sizeof(typename F::R) == 4;
   const bool b4 = sg.b[0] == 4 && sg.b[1] == 4 && sg.b[2] == 4 && sg.b[3] == 4;
-  auto kres = P.sap_half == 2   ? (b4 ? k_sap_sweep_smem<__half, true, true, 256, 2> : k_sap_sweep_smem<__half, true, false, 256, 2>)
-              : P.sap_half == 1 ? (b4 ? k_sap_sweep_smem<__half, false, true, 256, 2>
-                                      : k_sap_sweep_smem<__half, false, false, 256, 2>)
-                                : (b4 ? k_sap_sweep_smem<float, false, true, 256, 1>
-                                      : k_sap_sweep_smem<float, false, false, 256, 1>);
-  const size_t smem_res = (size_t)sg.vb * ((P.sap_half == 2 ? 48 : 96) + (P.sap_half ? 144 + 144 : 288 + 288));
+  // FP32 blocks of at most 256 sites are staged in shared memory; without memory
+  // for the FP32 image (FromField), or for the block-ordered vectors of a 4^4
+  // block, the sweep runs on the lexicographic fields
+  const bool h16 = f32 && P.sap_half && sg.vb <= 256;
+  const unsigned char* img = nullptr;
+  SapB4 A = {};
+  bool use_b4 = false;
+  if constexpr (f32) {
+    QCD_TRY(block_image(c, sg, h16, b4, &img, &A.flinks));
+    if (h16 && !img) return QCD_ERR_OOM;
+    if (b4 && img) {
+      // psi_b, and rho_b where the caller's residual is its own working copy
+      const size_t vec = (size_t)c->g.V * 96 * nrhs;
+      const bool own = rho_src != rho;
+      const qcd_status st = devbuf_ensure(c->sap_vec, own ? vec : 2 * vec);
+      if (st != QCD_OK && st != QCD_ERR_OOM) return st;
+      use_b4 = st == QCD_OK;
+      A.rho_src = rho_src;
+      A.psi_b = (float4*)c->sap_vec.p;
+      A.rho_b = own ? (float4*)rho : A.psi_b + vec / 16;
+      A.faces = (float4*)delta;
+      A.psi = psi;
+      A.img = img;
+      A.accumulate = accumulate;
+    }
+  }
+  const bool staged = f32 && sg.vb <= 256 && img;
+  // the register budget per thread follows from the block volume
+  auto kernD = sg.vb <= 256   ? k_sap_sweep<FieldsD, 256, 1>
+               : sg.vb <= 512 ? k_sap_sweep<FieldsD, 512, 1>
+                              : k_sap_sweep<FieldsD, 1024, 1>;
+  auto kernB = !h16 ? k_sap_sweep_b4<float, false>
+                     : (P.sap_half == 2 ? k_sap_sweep_b4<__half, true> : k_sap_sweep_b4<__half, false>);
+  auto kernF = staged ? (!h16              ? k_sap_sweep_pair<float, false, 256, 2>
+                         : P.sap_half == 2 ? k_sap_sweep_pair<__half, true, 256, 2>
+                                           : k_sap_sweep_pair<__half, false, 256, 2>)
+               : img  ? (sg.vb <= 512 ? k_sap_sweep_pair<FromImage, false, 512, 1>
+                                      : k_sap_sweep_pair<FromImage, false, 1024, 1>)
+                      : (sg.vb <= 512 ? k_sap_sweep_pair<FromField, false, 512, 1>
+                                      : k_sap_sweep_pair<FromField, false, 1024, 1>);
+  const size_t smem = (size_t)sg.vb * (!f32      ? 192
+                                       : !staged ? 96
+                                       : !h16    ? 96 + Stage<float>::bytes
+                                                 : (P.sap_half == 2 && !use_b4 ? 48 : 96) + Stage<__half>::bytes);
   // links and clover term read per active site and launch: their FP16 copies
   // (36 B per link, 144 B clover) for the 16-bit staged blocks, else FP32
-  const double gcb = (resident && P.sap_half) ? 4 * 36.0 + 144.0 : 4 * lb + cb;
-  if (resident)
-    QCD_CUDA_OK(cudaFuncSetAttribute(kres, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_res));
+  const double gcb = h16 ? 4 * 36.0 + 144.0 : 4 * lb + cb;
+  if constexpr (f32)
+    QCD_CUDA_OK(use_b4 ? cudaFuncSetAttribute(kernB, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
+                       : cudaFuncSetAttribute(kernF, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  else
+    QCD_CUDA_OK(cudaFuncSetAttribute(kernD, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   auto issue = [&]() -> qcd_status {
     for (int cy = 0; cy < P.ncy; cy++)
       for (int col = 0; col < 2; col++) {
         const int first = cy == 0 && !accumulate;
         const int gather = !(cy == 0 && col == 0);   // no boundary term before the first half-cycle
         const double bytes_rhs = sb * (2 + (first ? 1 : 2) + 1 + (gather ? f_face : 0.0));
+        const int last = cy < P.ncy - 1 ? 0 : 1 + col;   // 1: the last cycle, 2: its second half
         ProfScope ps(c, fam, half * (nactive * bytes_rhs + gcb),
                      half * nactive * (flops_site - (gather ? 0.0 : flops_gather)));
         const char* rin = cy == 0 ? rho_src : rho;   // the first cycle reads the caller's residual
-        if (resident)
-          kres<<<grid, sg.vb, smem_res, c->stream>>>(rin, rho, psi, delta, (const float4*)gauge, (const float4*)clover,
-                                                     (const uint4*)c->gaugeH.p, (const uint4*)c->cloverH.p, c->g, sg,
-                                                     col, gather, first, (float)c->kappa, P.nmr, nrhs, mask);
+        if constexpr (f32) {
+          if (use_b4) {
+            A.colour = col;
+            A.gather = gather;
+            A.first = cy == 0;
+            A.last = last;
+            kernB<<<grid, 256, smem, c->stream>>>(A, c->g, sg, (float)c->kappa, P.nmr, nrhs, mask);
+          } else {
+            kernF<<<grid, sg.vb, smem, c->stream>>>(rin, rho, psi, delta, (const float4*)gauge, (const float4*)clover,
+                                                    img, c->g, sg, col, gather, first, last, (float)c->kappa, P.nmr,
+                                                    nrhs, mask);
+          }
+        }
         else
-          kern<<<grid, sg.vb, smem, c->stream>>>(rin, rho, psi, delta, gauge, clover, c->g, sg, col,
-                                                 gather, first, (typename F::R)c->kappa, P.nmr, nrhs,
-                                                 mask);
+          kernD<<<grid, sg.vb, smem, c->stream>>>(rin, rho, psi, delta, gauge, clover, c->g, sg, col, gather, first,
+                                                  c->kappa, P.nmr, nrhs, mask);
         QCD_CUDA_OK(cudaGetLastError());
       }
     return QCD_OK;
@@ -667,6 +1104,7 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   SapGraph key;
   key.rho_src = rho_src;
   key.rho = rho; key.psi = psi; key.delta = delta; key.gauge = gauge; key.clover = clover; key.mask = mask;
+  key.img = img; key.flinks = A.flinks; key.vec = use_b4 ? c->sap_vec.p : nullptr;
   key.nrhs = nrhs; key.ncy = P.ncy; key.nmr = P.nmr; key.accumulate = accumulate; key.half = P.sap_half;
   key.prec = (int)sizeof(typename F::R);
   for (int mu = 0; mu < 4; mu++) key.block[mu] = P.block[mu];
@@ -674,7 +1112,8 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   cudaGraphExec_t exec = nullptr;
   for (auto& gph : c->sap_graphs)
     if (gph.rho_src == key.rho_src && gph.rho == key.rho && gph.psi == key.psi && gph.delta == key.delta && gph.gauge == key.gauge &&
-        gph.clover == key.clover && gph.mask == key.mask && gph.nrhs == key.nrhs && gph.ncy == key.ncy &&
+        gph.clover == key.clover && gph.mask == key.mask && gph.img == key.img && gph.flinks == key.flinks &&
+        gph.vec == key.vec && gph.nrhs == key.nrhs && gph.ncy == key.ncy &&
         gph.nmr == key.nmr && gph.accumulate == key.accumulate && gph.half == key.half && gph.prec == key.prec &&
         gph.kappa == key.kappa && memcmp(gph.block, key.block, sizeof(key.block)) == 0) {
       exec = gph.exec;

@@ -323,7 +323,9 @@ int solver_tile(qcd_ctx* c, int nrhs) {
   size_t freeb = 0, totalb = 0;
   cudaMemGetInfo(&freeb, &totalb);
   const int pchi = (P.precision == QCD_PREC_F32 && P.basis_half) ? QCD_PREC_H16 : P.precision;
-  size_t per = 4 * spinor_bytes(c, QCD_PREC_F64) + ((size_t)P.nkv + 3) * spinor_bytes(c, P.precision) +
+  // (FP32: one more vector for the block-ordered increments of the 4^4 SAP sweep)
+  size_t per = 4 * spinor_bytes(c, QCD_PREC_F64) +
+               ((size_t)P.nkv + 3 + (P.precision == QCD_PREC_F32)) * spinor_bytes(c, P.precision) +
                (size_t)P.nkv * spinor_bytes(c, pchi);
   size_t budget = freeb > ((size_t)4 << 30) ? freeb - ((size_t)4 << 30) : freeb / 2;
   int t = (int)(budget / (per ? per : 1));
