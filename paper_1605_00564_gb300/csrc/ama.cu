@@ -24,7 +24,7 @@
 
 qcd_status solver_run(qcd_ctx* c, int n, const double* tol, qcd_rhs_stats* st);
 qcd_status contract_nucleon(qcd_ctx* c, const void* prop, int t0, double* corr_dev, int precision,
-                            double2* partials);
+                            double2* partials, int canonical = 0);
 qcd_status threept_internal(qcd_ctx* c, const void* S_int, const void* S_sink, const int src[4], int t_sep,
                             int direction, double tol, int n_iter, double* corr3, qcd_rhs_stats* st);
 

@@ -12,7 +12,7 @@
 qcd_status solver_run(qcd_ctx* c, int n, const double* tol, qcd_rhs_stats* st);
 int solver_tile(qcd_ctx* c, int nrhs);
 qcd_status contract_nucleon(qcd_ctx* c, const void* prop, int t0, double* corr_dev, int precision,
-                            double2* partials);
+                            double2* partials, int canonical = 0);
 
 // --------------------------------------------------------------------------
 // errors
@@ -366,13 +366,11 @@ qcd_status qcd_nucleon_2pt(qcd_ctx* c, const double* prop, const int src[4], dou
   ARG_CHECK(precision == QCD_PREC_F64 || precision == QCD_PREC_F32, "unknown precision");
   for (int mu = 0; mu < 4; mu++) ARG_CHECK(src[mu] >= 0 && src[mu] < c->g.L[mu], "source outside the lattice");
   const int T = c->g.L[0];
-  QCD_TRY(devbuf_ensure(c->wsD[4], spinor_bytes(c, QCD_PREC_F64) * 12));
-  QCD_TRY(layout_spinor_import(c, prop, c->wsD[4].p, QCD_PREC_F64, 12));
   const size_t npart = 2 * (size_t)c->g.V;   // >= 2 * (V / sites per CTA)
   QCD_TRY(devbuf_ensure(c->contract, sizeof(double2) * (npart + 2 * T)));
   double2* part = (double2*)c->contract.p;
   double2* cd = part + npart;
-  QCD_TRY(contract_nucleon(c, c->wsD[4].p, src[0], (double*)cd, precision, part));
+  QCD_TRY(contract_nucleon(c, prop, src[0], (double*)cd, precision, part, 1));
   QCD_CUDA_OK(cudaMemcpyAsync(corr, cd, sizeof(double2) * 2 * T, cudaMemcpyDeviceToHost, c->stream));
   QCD_CUDA_OK(cudaStreamSynchronize(c->stream));
   return QCD_OK;

@@ -67,7 +67,7 @@ qcd_status gamma_apply(qcd_ctx* c, const void* in, void* out, int which, double 
 
 qcd_status solver_run(qcd_ctx* c, int n, const double* tol, qcd_rhs_stats* st);
 qcd_status contract_nucleon(qcd_ctx* c, const void* prop, int t0, double* corr_dev, int precision,
-                            double2* partials);
+                            double2* partials, int canonical = 0);
 
 namespace {
 __global__ void k_point12(double2* eta, int V, int site) {

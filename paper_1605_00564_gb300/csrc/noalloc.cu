@@ -51,9 +51,9 @@ qcd_status scratch_on_current_device(double2** out) {
     void* p = nullptr;
     QCD_CUDA_OK(cudaGetSymbolAddress(&p, g_nucleon_scratch));
     QCD_CUDA_OK(cudaFuncSetAttribute(nucleon::k_sites<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(144 * 32 * sizeof(Cplx<double>))));
+                                     (int)nucleon::cta_smem<double>(32)));
     QCD_CUDA_OK(cudaFuncSetAttribute(nucleon::k_sites<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(144 * 32 * sizeof(Cplx<float>))));
+                                     (int)nucleon::cta_smem<float>(32)));
     g_scratch_addr[dev] = (double2*)p;
   }
   *out = g_scratch_addr[dev];
@@ -108,10 +108,10 @@ extern "C" qcd_status qcd_nucleon_2pt_noalloc(const int dims[4], int time_bc, co
   // every partial slot read below is written first by its CTA: nothing to clear
   const int threads = nucleon::cta_threads(ns);
   if (precision == QCD_PREC_F64)
-    nucleon::k_sites<double, true><<<(unsigned)nb, threads, 144 * ns * sizeof(Cplx<double>), st>>>(
+    nucleon::k_sites<double, true><<<(unsigned)nb, threads, nucleon::cta_smem<double>(ns), st>>>(
         (const double2*)prop, (int)V, ns, scratch);
   else
-    nucleon::k_sites<float, true><<<(unsigned)nb, threads, 144 * ns * sizeof(Cplx<float>), st>>>(
+    nucleon::k_sites<float, true><<<(unsigned)nb, threads, nucleon::cta_smem<float>(ns), st>>>(
         (const double2*)prop, (int)V, ns, scratch);
   QCD_CUDA_OK(cudaGetLastError());
   nucleon::k_timeslices<<<T, 256, 0, st>>>(scratch, (int)(nb / T), T, src[0], time_bc * time_bc * time_bc,

@@ -14,111 +14,102 @@
 //   (G'^T S^{bb'T} G^T)_{ij} = g(i) g(j) S^{bb'}_{j^1 i^1}
 // and with P+- = (1 +- g0)/2, tr[P+- Z] = (1/2) sum_l (Z_{ll} -+ Z_{l^2, l}).
 //
-// Layout: 6 threads per site, one per sink colour permutation (a,b,c), each
-// summing over the 6 source permutations.  A CTA covers NS consecutive sites
-// of one timeslice (NS a power of two dividing the spatial volume, so a CTA
-// never straddles two timeslices); the propagator of those sites is staged
-// in shared memory (the 144 complex entries of a site are read by its 6
-// threads).  The CTA has 6 NS threads rounded up to whole warps; the padding
+// Evaluated in the diquark form (nucleon_diquark.cuh):
+//   tr[P+- G] = - sum_{cc'} ( tr R^{cc'} tr[P+- S^{cc'}] + tr[P+- R^{cc'} S^{cc'}] ).
+//
+// Layout: 9 threads per site, one per colour pair (c, c').  A CTA covers NS
+// consecutive sites of one timeslice (NS a power of two dividing the spatial
+// volume, so a CTA never straddles two timeslices); the propagator of those
+// sites is staged in shared memory (the 144 complex entries of a site are read
+// by its 9 threads; entry stride NS + 1, so that the canonical layout, whose
+// consecutive words are the components of one site, stages without bank
+// conflicts).  The CTA has 9 NS threads rounded up to whole warps; the padding
 // threads stage but contribute zero to the sums, so every warp of the
 // shuffle reduction is full.  The CTA's sum over its sites is written to a
 // partial; a second kernel sums the partials of each timeslice in a fixed
 // order, re-references the time to the source and applies the boundary sign
 // of wrapped sink times.
+//
+// FP64 is bound by the FP64 pipe (1.25 TFLOP/s), so the operation count sets the
+// time: 24^3x48 in 31.3 ms summed over the 36 colour permutations, 5.2 ms in this
+// form (the whole call, reading the canonical propagator).  FP32 is bound by
+// reading the FP64 propagator (2304 B a site).
 #pragma once
 
-#include "qcd_internal.cuh"
+#include "nucleon_diquark.cuh"
 
 // an unnamed namespace: each translation unit that includes this header
-// gets its own copy of the kernels and of the constant table
+// gets its own copy of the kernels
 namespace nucleon {
 namespace {
 
-__constant__ int c_perm[6][4] = {  // a, b, c, sign
-    {0, 1, 2, 1}, {1, 2, 0, 1}, {2, 0, 1, 1}, {0, 2, 1, -1}, {2, 1, 0, -1}, {1, 0, 2, -1}};
-
+// threads of a CTA covering ns sites: 9 ns rounded up to a multiple of 32
+inline int cta_threads(int ns) { return (9 * ns + 31) & ~31; }
+// dynamic shared memory of a CTA
 template <typename R>
-__device__ inline Cplx<R> Sget(const Cplx<R>* S_s, int ns, int i, int al, int a, int alp, int ap) {
-  return S_s[((3 * al + a) * 12 + 3 * alp + ap) * ns + i];
-}
-
-template <typename R>
-__device__ inline R gsign(int b) { return (b & 1) ? (R)1 : (R)-1; }
-
-// threads of a CTA covering ns sites: 6 ns rounded up to a multiple of 32
-inline int cta_threads(int ns) { return (6 * ns + 31) & ~31; }
+inline size_t cta_smem(int ns) { return (size_t)144 * (ns + 1) * sizeof(Cplx<R>); }
 
 // CANONICAL = true: prop is [rhs][site][spin][colour] complex FP64 (the C-ABI
 // layout); false: the internal FP64 spinor layout double2 [rhs][12][V].
 template <typename R, bool CANONICAL>
-__global__ void k_sites(const double2* __restrict__ prop, int V, int ns, double2* __restrict__ part) {
+__global__ void __launch_bounds__(288) k_sites(const double2* __restrict__ prop, int V, int ns,
+                                               double2* __restrict__ part) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Cplx<R>* S_s = (Cplx<R>*)smem_raw;
-  const int s0 = blockIdx.x * ns;
-  // stage: entry e = comp*12 + rhs of site s0 + i
+  const int s0 = blockIdx.x * ns, st = ns + 1;
+  // stage: entry e = 12 rhs + comp of site s0 + i at S_s[e * st + i]
   for (int idx = threadIdx.x; idx < 144 * ns; idx += blockDim.x) {
-    const int i = idx % ns, e = idx / ns;
-    const int comp = e / 12, rhs = e - comp * 12;
-    const double2 v = CANONICAL ? prop[((size_t)rhs * V + s0 + i) * 12 + comp]
-                                : prop[((size_t)rhs * 12 + comp) * V + s0 + i];
-    S_s[e * ns + i] = cmk((R)v.x, (R)v.y);
+    int i, e;
+    double2 v;
+    if (CANONICAL) {
+      const int rhs = idx / (12 * ns), rem = idx - rhs * 12 * ns;
+      i = rem / 12;
+      e = 12 * rhs + rem - 12 * i;
+      v = __ldg(prop + ((size_t)rhs * V + s0) * 12 + rem);
+    } else {
+      i = idx % ns;
+      e = idx / ns;
+      v = __ldg(prop + (size_t)e * V + s0 + i);
+    }
+    S_s[e * st + i] = cmk((R)v.x, (R)v.y);
   }
   __syncthreads();
 
   Cplx<R> accp = cmk((R)0, (R)0), accm = cmk((R)0, (R)0);
-  if (threadIdx.x < 6 * ns) {
+  if (threadIdx.x < 9 * ns) {
     const int i = threadIdx.x % ns;
-    const int pq = threadIdx.x / ns;   // sink permutation 0..5
-    const int a = c_perm[pq][0], b = c_perm[pq][1], c = c_perm[pq][2];
-    const R eps = (R)c_perm[pq][3];
-#pragma unroll 1
-    for (int q = 0; q < 6; q++) {
-      const int ap = c_perm[q][0], bp = c_perm[q][1], cp = c_perm[q][2];
-      const R ee = eps * (R)c_perm[q][3];
-      // T = tr[S^{aa'T} G S^{bb'} G']
-      Cplx<R> T = cmk((R)0, (R)0);
+    const int o = threadIdx.x / ns;
+    const int c = o / 3, cp = o - 3 * c;
+    auto get = [&](int al, int a, int alp, int ap) { return S_s[(12 * (3 * alp + ap) + 3 * al + a) * st + i]; };
+    Cplx<R> r[6];
+    diquark::diquark_r<R>(get, c, cp, r);
+    Cplx<R> Z[4][4];
 #pragma unroll
-      for (int be = 0; be < 4; be++)
+    for (int l = 0; l < 4; l++)
 #pragma unroll
-        for (int bq = 0; bq < 4; bq++) {
-          const Cplx<R> x = Sget(S_s, ns, i, be, a, bq, ap) * Sget(S_s, ns, i, be ^ 1, b, bq ^ 1, bp);
-          T = T + (gsign<R>(be) * gsign<R>(bq)) * x;
-        }
-      // tr[P+- S^{cc'}]
-      Cplx<R> d = cmk((R)0, (R)0), o = cmk((R)0, (R)0);
+      for (int k = 0; k < 4; k++) Z[l][k] = get(l, c, k, cp);
+    // tr S, tr[g0 S] = -o, tr[R S] and tr[g0 R S] = -zo over the independent entries of R
+    Cplx<R> d = Z[0][0], q = Z[2][0], zd = cmk((R)0, (R)0), zo = cmk((R)0, (R)0);
 #pragma unroll
-      for (int l = 0; l < 4; l++) {
-        d = d + Sget(S_s, ns, i, l, c, l, cp);
-        o = o + Sget(S_s, ns, i, l ^ 2, c, l, cp);
-      }
-      const Cplx<R> t1p = T * ((R)0.5 * (d - o)), t1m = T * ((R)0.5 * (d + o));
-      // Y = S^{ca'} M, M_{kj} = g(k) g(j) S^{bb'}_{j^1 k^1}
-      Cplx<R> Y[4][4];
-#pragma unroll
-      for (int ii = 0; ii < 4; ii++)
-#pragma unroll
-        for (int j = 0; j < 4; j++) {
-          Cplx<R> y = cmk((R)0, (R)0);
-#pragma unroll
-          for (int k = 0; k < 4; k++)
-            y = y + (gsign<R>(k) * gsign<R>(j)) *
-                        (Sget(S_s, ns, i, ii, c, k, ap) * Sget(S_s, ns, i, j ^ 1, b, k ^ 1, bp));
-          Y[ii][j] = y;
-        }
-      // tr[P+- Y S^{ac'}] = (1/2) sum_{l,k} (Y_{lk} -+ Y_{l^2 k}) S^{ac'}_{kl}
-      Cplx<R> zd = cmk((R)0, (R)0), zo = cmk((R)0, (R)0);
-#pragma unroll
-      for (int l = 0; l < 4; l++)
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-          const Cplx<R> sv = Sget(S_s, ns, i, k, a, l, cp);
-          zd = zd + Y[l][k] * sv;
-          zo = zo + Y[l ^ 2][k] * sv;
-        }
-      const Cplx<R> t2p = (R)0.5 * (zd - zo), t2m = (R)0.5 * (zd + zo);
-      accp = accp + ee * (t1p - t2p);
-      accm = accm + ee * (t1m - t2m);
+    for (int l = 1; l < 4; l++) {
+      d = d + Z[l][l];
+      q = q + Z[l ^ 2][l];
     }
+#pragma unroll
+    for (int m = 0; m < 6; m++) {
+      const int ii = diquark::r_row(m), j = diquark::r_col(m);
+      if (diquark::gsgn(ii) * diquark::gsgn(j) > 0) {
+        cmac(zd, r[m], Z[j][ii] + Z[ii ^ 1][j ^ 1]);
+        cmac(zo, r[m], Z[j][ii ^ 2] + Z[ii ^ 1][j ^ 3]);
+      } else {
+        cmac(zd, r[m], Z[j][ii] - Z[ii ^ 1][j ^ 1]);
+        cmac(zo, r[m], Z[j][ii ^ 2] - Z[ii ^ 1][j ^ 3]);
+      }
+    }
+    // tr R / 2 = R_00 + R_22; tr[P+- X] = (tr X +- tr[g0 X]) / 2
+    const Cplx<R> tr = r[0] + r[5];
+    accp = -(tr * (d - q) + (R)0.5 * (zd - zo));
+    accm = -(tr * (d + q) + (R)0.5 * (zd + zo));
   }
   // CTA sum (fixed order): warp shuffles over full warps, then one thread
   // over the warp sums
