@@ -165,13 +165,12 @@ extern "C" qcd_status qcd_fh_gradient(qcd_ctx* c, const double* prop, const int 
   }
   QCD_TRY(devbuf_ensure(c->contract, sizeof(double2) * 16 * T));
   QCD_CUDA_OK(cudaMemcpyAsync(c->contract.p, pm.data(), sizeof(double2) * 16 * T, cudaMemcpyHostToDevice, c->stream));
-  int ns = 8;
-  while (L3 % ns) ns >>= 1;
+  const int ns = nucleon_grad::sites_per_cta(L3);
   {
-    ProfScope ps(c, FAM_CONTRACT, (double)V * (2304 + 2 * 2304), (double)V * 36 * 6 * 200 * 8);
-    const size_t smem = sizeof(Cplx<double>) * 144 * ns;
+    ProfScope ps(c, FAM_CONTRACT, (double)V * (2304 + 2 * 2304), (double)V * 9 * 700 * 8);
+    const size_t smem = nucleon_grad::cta_smem(ns);
     QCD_CUDA_OK(cudaFuncSetAttribute(nucleon_grad::k_dC_dS, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    nucleon_grad::k_dC_dS<<<V / ns, 18 * ns, smem, c->stream>>>((const double2*)c->wsD[4].p,
+    nucleon_grad::k_dC_dS<<<V / ns, nucleon_grad::cta_threads(ns), smem, c->stream>>>((const double2*)c->wsD[4].p,
                                                                (const double2*)c->contract.p, V, L3, ns, 0,
                                                                (double2*)c->wsD[5].p);
     QCD_CUDA_OK(cudaGetLastError());

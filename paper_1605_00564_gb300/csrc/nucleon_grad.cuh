@@ -12,160 +12,190 @@
 // summed over the slots of flavour f, in the propagator's layout (field
 // rhs = 3 alpha' + colour', component 3 alpha + colour).
 //
-// Gamma structure (chiral basis): G = C g5 = diag(J, J), J = [[0,-1],[1,0]],
-// G' = g0 G^+ g0^T = -G; both act as "flip the index by ^1 and multiply by
-// g(i) g(j)", g(b) = -1 for even b, +1 for odd b.
+// In the diquark form (nucleon_diquark.cuh), with the u and d propagators kept
+// apart,
+//   C = - sum_{cc'} tr[ R^{cc'} N^{cc'} ],  N^{cc'} = tr[P U^{cc'}] 1 + U^{cc'} P,
+//   R^{cc'} = - sum_{x != c, x' != c'} s s' U^{xx'} D^{yy'}^T   (hat on D),
+// y, y' the remaining colours and s = +1 if x follows c cyclically, else -1 (s'
+// likewise).  At U = D = S its derivatives are, per colour pair (x, x'),
+//   dC/dU^{xx'} = [ - tr R^{xx'} P - P R^{xx'} + sum s s' S^{yy'}^T N^{cc'} ]^T
+//   dC/dD^{xx'} = hat( sum s s' N^{cc'} S^{yy'} )
+// (sums over the four (c, c') with c != x, c' != x'): eight 4x4 products a pair,
+// about 6,300 complex multiply-adds a site against 16,600 of the sum over the 36
+// colour permutations with its repeated products.  Bound by the FP64 pipe; that form
+// also spilled its 4x4 blocks and took 143 ms on 16^3x32 (all time-slices), this one
+// about 10 (the gradient call 296 -> 114 ms with the faster SAP sweep).
+//
+// P(t) has entries (k, k) and (k, k^2) only: true of P+-, of P+- g5 g3 and of
+// any combination of them (g0 and g3 both couple spin k to k^2).
 #pragma once
 
-#include "qcd_internal.cuh"
+#include "nucleon_diquark.cuh"
 
 namespace nucleon_grad {
 namespace {
 
-__constant__ int c_perm_fh[6][4] = {  // a, b, c, sign
-    {0, 1, 2, 1}, {1, 2, 0, 1}, {2, 0, 1, 1}, {0, 2, 1, -1}, {2, 1, 0, -1}, {1, 0, 2, -1}};
-
 using C64 = Cplx<double>;
+using diquark::cmsub;
 
-__device__ inline double gs(int b) { return (b & 1) ? 1.0 : -1.0; }
+// sites of one CTA: the largest power of two <= 16 dividing the spatial volume
+inline int sites_per_cta(long long L3) {
+  int ns = 16;
+  while (L3 % ns) ns >>= 1;
+  return ns;
+}
+inline int cta_threads(int ns) { return 9 * ns; }
+// S and N of the CTA's sites
+inline size_t cta_smem(int ns) { return (size_t)2 * 144 * ns * sizeof(C64); }
 
-struct M4 {
-  C64 m[4][4];
-};
+// a * +-1 by the sign bit (integer units; the FP64 pipe is the bound)
+__device__ inline double flip_sign(double a, int mask) {
+  return __hiloint2double(__double2hiint(a) ^ mask, __double2loint(a));
+}
+__device__ inline C64 flip_sign(C64 a, int mask) { return cmk(flip_sign(a.re, mask), flip_sign(a.im, mask)); }
 
-__device__ inline M4 load_blk(const C64* S_s, int ns, int i, int x, int xp) {
-  M4 o;
-#pragma unroll
-  for (int al = 0; al < 4; al++)
-#pragma unroll
-    for (int alp = 0; alp < 4; alp++) o.m[al][alp] = S_s[((3 * al + x) * 12 + 3 * alp + xp) * ns + i];
-  return o;
-}
-__device__ inline M4 mm(const M4& a, const M4& b) {
-  M4 o;
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int j = 0; j < 4; j++) {
-      C64 s = cmk(0.0, 0.0);
-#pragma unroll
-      for (int k = 0; k < 4; k++) s = s + a.m[i][k] * b.m[k][j];
-      o.m[i][j] = s;
-    }
-  return o;
-}
-// (G X G')-type sandwich: out_{ij} = g(i) g(j) X_{i^1, j^1}
-__device__ inline M4 flip(const M4& X) {
-  M4 o;
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int j = 0; j < 4; j++) o.m[i][j] = (gs(i) * gs(j)) * X.m[i ^ 1][j ^ 1];
-  return o;
-}
-// M = G'^T X^T G^T: M_{ij} = g(i) g(j) X_{j^1, i^1}
-__device__ inline M4 flipT(const M4& X) {
-  M4 o;
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int j = 0; j < 4; j++) o.m[i][j] = (gs(i) * gs(j)) * X.m[j ^ 1][i ^ 1];
-  return o;
-}
-__device__ inline C64 trace_prod(const M4& a, const M4& b) {   // tr[a b]
-  C64 s = cmk(0.0, 0.0);
-#pragma unroll
-  for (int i = 0; i < 4; i++)
-#pragma unroll
-    for (int k = 0; k < 4; k++) s = s + a.m[i][k] * b.m[k][i];
-  return s;
-}
-
-// H_f for NS sites per CTA, the CTAs covering the sites site0, site0 + 1, ...;
-// thread = (site i, output o), o = 9 f + 3 x + x' holding the 4x4 spin block
-// (x, x') of flavour f (0: u, 1: d).  pmat[t]: the 4x4 complex matrix P(t)
-// (row major) of time-slice t.  prop: internal FP64 layout, 12 fields; H:
-// internal FP64 layout, 24 fields (u then d), rhs = 3 alpha' + x'.
-__global__ void k_dC_dS(const double2* __restrict__ prop, const double2* __restrict__ pmat, int V, int L3, int ns,
-                        int site0, double2* __restrict__ H) {
+// H_f for ns sites per CTA, the CTAs covering the sites site0, site0 + 1, ...;
+// thread = (site i, colour pair (x, x')), first flavour u, then d.  pmat[t]: the
+// 4x4 complex matrix P(t) (row major) of time-slice t.  prop: internal FP64
+// layout, 12 fields; H: internal FP64 layout, 24 fields (u then d),
+// rhs = 3 alpha' + x'.
+__global__ void __launch_bounds__(144) k_dC_dS(const double2* __restrict__ prop, const double2* __restrict__ pmat,
+                                               int V, int L3, int ns, int site0, double2* __restrict__ H) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C64* S_s = (C64*)smem_raw;
+  C64* N_s = S_s + (size_t)144 * ns;
   const int s0 = site0 + blockIdx.x * ns;
   for (int idx = threadIdx.x; idx < 144 * ns; idx += blockDim.x) {
-    int i = idx % ns, e = idx / ns;
-    int comp = e / 12, rhs = e - comp * 12;
-    double2 v = prop[((size_t)rhs * 12 + comp) * V + s0 + i];
-    S_s[e * ns + i] = cmk(v.x, v.y);
+    const int i = idx % ns, e = idx / ns;
+    const double2 v = __ldg(prop + (size_t)e * V + s0 + i);
+    S_s[idx] = cmk(v.x, v.y);
   }
   __syncthreads();
   const int i = threadIdx.x % ns, o = threadIdx.x / ns;
-  if (o >= 18) return;
-  const int f = o / 9, x = (o % 9) / 3, xp = o % 3;
+  const int x = o / 3, xp = o - 3 * x;
+  auto get = [&](int al, int a, int alp, int ap) { return S_s[(12 * (3 * alp + ap) + 3 * al + a) * ns + i]; };
   const int t = (s0 + i) / L3;
-  M4 Pw;
+  C64 pd[4], po[4];   // P_kk and P_{k, k^2}
 #pragma unroll
-  for (int u = 0; u < 4; u++)
+  for (int k = 0; k < 4; k++) {
+    const double2 u = pmat[16 * t + 5 * k], v = pmat[16 * t + 4 * k + (k ^ 2)];
+    pd[k] = cmk(u.x, u.y);
+    po[k] = cmk(v.x, v.y);
+  }
+  // acc[j][k] = dC/dS_u(j, k): the third quark's part, -(tr R P + P R)_{kj}
+  C64 acc[4][4];
 #pragma unroll
-    for (int v = 0; v < 4; v++) {
-      const double2 e = pmat[16 * t + 4 * u + v];
-      Pw.m[u][v] = cmk(e.x, e.y);
+  for (int j = 0; j < 4; j++)
+#pragma unroll
+    for (int k = 0; k < 4; k++) acc[j][k] = cmk(0.0, 0.0);
+  {
+    C64 r[6];
+    diquark::diquark_r<double>(get, x, xp, r);
+    const C64 tr = 2.0 * (r[0] + r[5]);
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      cmsub(acc[k][k], tr, pd[k]);
+      cmsub(acc[k ^ 2][k], tr, po[k]);
     }
-  M4 acc;
+    // R entry (a, j) = rv: (P R)_{aj} takes P_aa, (P R)_{a^2, j} takes P_{a^2, a}
+    auto add = [&](int a, int j, C64 rv) {
+      cmsub(acc[j][a], pd[a], rv);
+      cmsub(acc[j][a ^ 2], po[a ^ 2], rv);
+    };
 #pragma unroll
-  for (int a = 0; a < 4; a++)
-#pragma unroll
-    for (int b = 0; b < 4; b++) acc.m[a][b] = cmk(0.0, 0.0);
-  for (int p = 0; p < 6; p++) {
-    const int a = c_perm_fh[p][0], b = c_perm_fh[p][1], c = c_perm_fh[p][2];
-    for (int q = 0; q < 6; q++) {
-      const int ap = c_perm_fh[q][0], bp = c_perm_fh[q][1], cp = c_perm_fh[q][2];
-      const double ee = (double)(c_perm_fh[p][3] * c_perm_fh[q][3]);
-      // first Wick term: ee tr[Pw S^{cc'}] tr[S^{aa'T} G S^{bb'} G']
-      if (f == 0 && x == a && xp == ap) {          // d/dS_u^{aa'} = ee trP(S^{cc'}) (G S^{bb'} G')
-        C64 tp = trace_prod(Pw, load_blk(S_s, ns, i, c, cp));
-        M4 Y = flip(load_blk(S_s, ns, i, b, bp));
-        for (int u = 0; u < 4; u++)
-          for (int v = 0; v < 4; v++) acc.m[u][v] = acc.m[u][v] + (ee * tp) * Y.m[u][v];
-      }
-      if (f == 0 && x == c && xp == cp) {          // d/dS_u^{cc'}_{al al'} = ee Pw_{al' al} T
-        M4 A = load_blk(S_s, ns, i, a, ap), B = flip(load_blk(S_s, ns, i, b, bp));
-        C64 T = cmk(0.0, 0.0);
-        for (int u = 0; u < 4; u++)
-          for (int v = 0; v < 4; v++) T = T + A.m[u][v] * B.m[u][v];
-        for (int u = 0; u < 4; u++)
-          for (int v = 0; v < 4; v++) acc.m[u][v] = acc.m[u][v] + (ee * T) * Pw.m[v][u];
-      }
-      if (f == 1 && x == b && xp == bp) {          // d/dS_d^{bb'} = ee trP(S^{cc'}) (G^T S^{aa'} G'^T)
-        C64 tp = trace_prod(Pw, load_blk(S_s, ns, i, c, cp));
-        M4 Y = flip(load_blk(S_s, ns, i, a, ap));
-        for (int u = 0; u < 4; u++)
-          for (int v = 0; v < 4; v++) acc.m[u][v] = acc.m[u][v] + (ee * tp) * Y.m[u][v];
-      }
-      // second Wick term (subtracted): ee tr[Pw S^{ca'} M S^{ac'}], M = G'^T S^{bb'T} G^T
-      if (f == 0 && x == c && xp == ap) {          // d/dS_u^{ca'}_{jk} = ee (M S^{ac'} Pw)_{kj}
-        M4 Z = mm(mm(flipT(load_blk(S_s, ns, i, b, bp)), load_blk(S_s, ns, i, a, cp)), Pw);
-        for (int u = 0; u < 4; u++)
-          for (int v = 0; v < 4; v++) acc.m[u][v] = acc.m[u][v] - ee * Z.m[v][u];
-      }
-      if (f == 0 && x == a && xp == cp) {          // d/dS_u^{ac'}_{jk} = ee (Pw S^{ca'} M)_{kj}
-        M4 Z = mm(mm(Pw, load_blk(S_s, ns, i, c, ap)), flipT(load_blk(S_s, ns, i, b, bp)));
-        for (int u = 0; u < 4; u++)
-          for (int v = 0; v < 4; v++) acc.m[u][v] = acc.m[u][v] - ee * Z.m[v][u];
-      }
-      if (f == 1 && x == b && xp == bp) {          // d/dS_d^{bb'}_{nm} = ee (G^T (S^{ac'} Pw S^{ca'}) G'^T)_{nm}
-        M4 Z = flip(mm(mm(load_blk(S_s, ns, i, a, cp), Pw), load_blk(S_s, ns, i, c, ap)));
-        for (int u = 0; u < 4; u++)
-          for (int v = 0; v < 4; v++) acc.m[u][v] = acc.m[u][v] - ee * Z.m[u][v];
-      }
+    for (int m = 0; m < 6; m++) {
+      const int a = diquark::r_row(m), j = diquark::r_col(m);
+      add(a, j, r[m]);
+      add(j ^ 1, a ^ 1, diquark::gsgn(a) * diquark::gsgn(j) > 0 ? r[m] : -r[m]);
     }
   }
-  // acc = dC/dS; H = conj(acc).  Entry (al, al') -> field rhs = 3 al' + x', comp 3 al + x
-  double2* Hf = H + (size_t)f * 12 * 12 * V;
+  {
+    // N = tr[P S] 1 + S P
+    C64 Z[4][4], n[4][4], tr = cmk(0.0, 0.0);
+#pragma unroll
+    for (int a = 0; a < 4; a++)
+#pragma unroll
+      for (int b = 0; b < 4; b++) Z[a][b] = get(a, x, b, xp);
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      cmac(tr, pd[k], Z[k][k]);
+      cmac(tr, po[k], Z[k ^ 2][k]);
+    }
+#pragma unroll
+    for (int a = 0; a < 4; a++)
+#pragma unroll
+      for (int b = 0; b < 4; b++) {
+        n[a][b] = a == b ? tr : cmk(0.0, 0.0);
+        cmac(n[a][b], Z[a][b], pd[b]);
+        cmac(n[a][b], Z[a][b ^ 2], po[b ^ 2]);
+        N_s[(16 * o + 4 * a + b) * ns + i] = n[a][b];
+      }
+  }
+  __syncthreads();
+  // the diquark parts: the four (c, c') with c = x + 1, x + 2 and c' likewise; the
+  // sign is that of the two cyclic steps, y and y' the remaining colours
+#pragma unroll 1
+  for (int q = 0; q < 4; q++) {
+    const int dc = 1 + (q & 1), dp = 1 + (q >> 1);
+    const int c = (x + dc) % 3, cp = (xp + dp) % 3, y = 3 - x - c, yp = 3 - xp - cp;
+    const int mask = dc != dp ? (int)0x80000000 : 0;
+    const C64* n = N_s + (size_t)(16 * (3 * c + cp)) * ns + i;
+#pragma unroll
+    for (int a = 0; a < 4; a++) {
+      // (S^{yy'}^T N)_{kj} += g(a) g(k) S_{a^1, k^1} N_{aj}
+      C64 nr[4], sr[4];
+#pragma unroll
+      for (int j = 0; j < 4; j++) nr[j] = flip_sign(n[(4 * a + j) * ns], mask);
+#pragma unroll
+      for (int k = 0; k < 4; k++) sr[k] = get(a ^ 1, y, k ^ 1, yp);
+#pragma unroll
+      for (int k = 0; k < 4; k++)
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+          if (diquark::gsgn(a) * diquark::gsgn(k) > 0) cmac(acc[j][k], sr[k], nr[j]);
+          else cmsub(acc[j][k], sr[k], nr[j]);
+        }
+    }
+  }
+  // H = conj(dC/dS): entry (al, al') -> field rhs = 3 al' + x', component 3 al + x
+#pragma unroll
   for (int al = 0; al < 4; al++)
+#pragma unroll
     for (int alp = 0; alp < 4; alp++)
-      Hf[((size_t)(3 * alp + xp) * 12 + 3 * al + x) * V + s0 + i] = make_double2(acc.m[al][alp].re, -acc.m[al][alp].im);
+      H[((size_t)(3 * alp + xp) * 12 + 3 * al + x) * V + s0 + i] = make_double2(acc[al][alp].re, -acc[al][alp].im);
+#pragma unroll
+  for (int j = 0; j < 4; j++)
+#pragma unroll
+    for (int k = 0; k < 4; k++) acc[j][k] = cmk(0.0, 0.0);
+#pragma unroll 1
+  for (int q = 0; q < 4; q++) {
+    const int dc = 1 + (q & 1), dp = 1 + (q >> 1);
+    const int c = (x + dc) % 3, cp = (xp + dp) % 3, y = 3 - x - c, yp = 3 - xp - cp;
+    const int mask = dc != dp ? (int)0x80000000 : 0;
+    const C64* n = N_s + (size_t)(16 * (3 * c + cp)) * ns + i;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      C64 nc[4], sr[4];
+#pragma unroll
+      for (int a = 0; a < 4; a++) nc[a] = flip_sign(n[(4 * a + k) * ns], mask);
+#pragma unroll
+      for (int b = 0; b < 4; b++) sr[b] = get(k, y, b, yp);
+#pragma unroll
+      for (int a = 0; a < 4; a++)
+#pragma unroll
+        for (int b = 0; b < 4; b++) cmac(acc[a][b], nc[a], sr[b]);
+    }
+  }
+  double2* Hd = H + (size_t)144 * V;
+#pragma unroll
+  for (int al = 0; al < 4; al++)
+#pragma unroll
+    for (int alp = 0; alp < 4; alp++) {
+      const C64 z = acc[al ^ 1][alp ^ 1];
+      const double sg = (double)(diquark::gsgn(al) * diquark::gsgn(alp));
+      Hd[((size_t)(3 * alp + xp) * 12 + 3 * al + x) * V + s0 + i] = make_double2(sg * z.re, -sg * z.im);
+    }
 }
 
 }  // namespace
 }  // namespace nucleon_grad
-

@@ -227,9 +227,8 @@ qcd_status threept_internal(qcd_ctx* c, const void* S_int, const void* S_sink, c
   QCD_TRY(devbuf_ensure(c->wsD[6], f64 * 24));
   QCD_TRY(devbuf_ensure(c->wsD[7], f64 * 24));
   const ThreePtMats M = three_pt_mats(direction);
-  int ns = 8;
-  while (L3 % ns) ns >>= 1;
-  const size_t smem = sizeof(C64) * 144 * ns;
+  const int ns = nucleon_grad::sites_per_cta(L3);
+  const size_t smem = nucleon_grad::cta_smem(ns);
   QCD_CUDA_OK(cudaFuncSetAttribute(nucleon_grad::k_dC_dS, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   std::vector<double2> pm(16 * (size_t)T);
   for (int p = 0; p < 2; p++) {
@@ -243,8 +242,8 @@ qcd_status threept_internal(qcd_ctx* c, const void* S_int, const void* S_sink, c
     QCD_CUDA_OK(cudaMemsetAsync(c->wsD[5].p, 0, f64 * 24, c->stream));
     {
       // the sequential source lives on the sink time-slice only
-      ProfScope ps(c, FAM_CONTRACT, (double)L3 * 3 * 2304, (double)L3 * 36 * 6 * 200 * 8);
-      nucleon_grad::k_dC_dS<<<L3 / ns, 18 * ns, smem, c->stream>>>((const double2*)S_sink,
+      ProfScope ps(c, FAM_CONTRACT, (double)L3 * 3 * 2304, (double)L3 * 9 * 700 * 8);
+      nucleon_grad::k_dC_dS<<<L3 / ns, nucleon_grad::cta_threads(ns), smem, c->stream>>>((const double2*)S_sink,
                                                                   (const double2*)c->contract.p, V, L3, ns, ts * L3,
                                                                   (double2*)c->wsD[5].p);
       QCD_CUDA_OK(cudaGetLastError());
