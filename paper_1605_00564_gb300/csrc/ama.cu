@@ -110,7 +110,7 @@ extern "C" qcd_status qcd_ama_nucleon(qcd_ctx* c, const int* src, int n_src, con
       rc = QCD_ERR_CUDA;
       break;
     }
-    if ((rc = smear_fields(c, c->wsD[0].p, 12)) != QCD_OK) break;      // smeared source
+    if ((rc = smear_fields(c, c->wsD[0].p, 12, s[0])) != QCD_OK) break;   // smeared source
     const bool fixed = !exact && p->n_iter_2pt > 0;
     std::vector<double> tols(12, exact ? p->exact_tol : (fixed ? 1e-300 : p->sloppy_tol));
     if (exact) c->params.basis_half = 0;      // an FP16 Krylov basis serves the sloppy solves only

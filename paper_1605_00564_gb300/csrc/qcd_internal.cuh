@@ -545,5 +545,6 @@ void* dfl_little(qcd_ctx* c);
 size_t spinor_bytes(const qcd_ctx* c, int prec);
 
 // Gaussian smearing (smear.cu) of nrhs FP64 internal spinors in place with
-// the context's smeared links and parameters (a no-op when smear_n is 0)
-qcd_status smear_fields(qcd_ctx* c, void* fields, int nrhs);
+// the context's smeared links and parameters (a no-op when smear_n is 0);
+// t >= 0: fields that vanish outside time-slice t
+qcd_status smear_fields(qcd_ctx* c, void* fields, int nrhs, int t = -1);

@@ -252,7 +252,7 @@ qcd_status threept_internal(qcd_ctx* c, const void* S_int, const void* S_sink, c
           (const double2*)c->wsD[5].p, (double2*)((char*)c->wsD[6].p + f64 * 12 * p), V);
       QCD_CUDA_OK(cudaGetLastError());
     }
-    if (S_sink != S_int) QCD_TRY(smear_fields(c, (char*)c->wsD[6].p + f64 * 12 * p, 12));
+    if (S_sink != S_int) QCD_TRY(smear_fields(c, (char*)c->wsD[6].p + f64 * 12 * p, 12, ts));
   }
   // the 24 sequential propagators, 12 at a time: W = D^-1 eta
   std::vector<double> tols(12, n_iter > 0 ? 1e-300 : tol);
