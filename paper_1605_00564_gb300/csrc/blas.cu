@@ -182,8 +182,14 @@ __global__ void __launch_bounds__(RED_TPB) k_reduce_final(const double2* __restr
   }
 }
 
+// CTAs per right-hand side of the reducing passes (a function of the volume alone:
+// a right-hand side gives the same bits in any batch).  A CTA ends in FP64 sums over
+// its threads, and a warp's FP64 addition takes the SM 16 cycles (1/64 of the FP32
+// rate): with one site per thread these sums took as long as the loads.  So
+// larger lattices give every thread at least four sites.
 int red_grid(const qcd_ctx* c) {
-  int g = (c->g.V + RED_TPB - 1) / RED_TPB;
+  const int per = RED_TPB * (c->g.V >= 131072 ? 4 : c->g.V >= 65536 ? 2 : 1);
+  int g = (c->g.V + per - 1) / per;
   return g < 4 * 152 ? g : 4 * 152;
 }
 
@@ -308,74 +314,39 @@ inline dim3 grid2(const qcd_ctx* c, int nrhs) { return dim3((c->g.V + 255) / 256
 // ---------------------------------------------------------------------------
 constexpr int GS_TPB = 256;
 
-// block sum of NV doubles; thread 0 holds the result in out[]
-template <int NV>
-__device__ inline void block_sum_n(double (&v)[NV], double* sh /* [NV][32] */) {
+// CTA sums of NV values per thread (GS_TPB threads, fixed order) in FP64: every warp
+// sums whole values from shared memory, 8 additions per lane and 5 across lanes,
+// instead of 5 across the lanes of each of the 8 warps and 8 more (with four sites per
+// thread the Gram-Schmidt passes of 12 RHS on 16^3x32 went from 4.0 to 5.5 TB/s).
+// Lane 0 of warp v % 8 passes the sum of value v to out(v, sum).
+template <int NV, typename R, typename Out>
+__device__ inline void cta_sums(const R (&v)[NV], R* sh /* [NV][GS_TPB] */, Out out) {
+  constexpr int NW = GS_TPB / 32;
+  __syncthreads();   // the previous use of sh is over
 #pragma unroll
-  for (int k = 0; k < NV; k++)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_xor_sync(0xffffffffu, v[k], o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
+  for (int k = 0; k < NV; k++) sh[k * GS_TPB + threadIdx.x] = v[k];
   __syncthreads();
-  if (l == 0)
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  for (int k = w; k < NV; k += NW) {
+    double t = 0;
 #pragma unroll
-    for (int k = 0; k < NV; k++) sh[k * 32 + w] = v[k];
-  __syncthreads();
-  if (threadIdx.x == 0)
+    for (int i = 0; i < NW; i++) t += (double)sh[k * GS_TPB + 32 * i + l];
 #pragma unroll
-    for (int k = 0; k < NV; k++) {
-      double t = 0;
-      for (int ww = 0; ww < nw; ww++) t += sh[k * 32 + ww];
-      v[k] = t;
-    }
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (l == 0) out(k, t);
+  }
 }
 
 // dots[j][r] = (chi_j, chi_k) for j < k: chi_k is read once, each chi_j once.
-// One thread per site; per-j CTA sums go to part[r][j][cta].
-template <typename X>
-__global__ void __launch_bounds__(GS_TPB) k_multi_dot(const char* __restrict__ chi, size_t jstride, int k, int V,
-                                                       double2* __restrict__ part, const int* mask) {
-  __shared__ double sh[2 * 32];
-  const int rhs = blockIdx.y;
-  if (mask && !mask[rhs]) return;
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t roff = (size_t)rhs * X::bytes * V;
-  using R = typename X::R;
-  Cplx<R> ck[12];
-  if (s < V) {
-#pragma unroll
-    for (int q = 0; q < 6; q++) X::ld(chi + k * jstride + roff, V, q, s, ck[2 * q], ck[2 * q + 1]);
-  } else {
-#pragma unroll
-    for (int q = 0; q < 12; q++) ck[q] = cmk((R)0, (R)0);
-  }
-  for (int j = 0; j < k; j++) {
-    R sr = 0, si = 0;
-    if (s < V) {
-#pragma unroll
-      for (int q = 0; q < 6; q++) {
-        Cplx<R> a, b;
-        X::ld(chi + j * jstride + roff, V, q, s, a, b);
-        sr += a.re * ck[2 * q].re + a.im * ck[2 * q].im + b.re * ck[2 * q + 1].re + b.im * ck[2 * q + 1].im;
-        si += a.re * ck[2 * q].im - a.im * ck[2 * q].re + b.re * ck[2 * q + 1].im - b.im * ck[2 * q + 1].re;
-      }
-    }
-    double v[2] = {(double)sr, (double)si};
-    block_sum_n<2>(v, sh);
-    if (threadIdx.x == 0) part[((size_t)rhs * k + j) * gridDim.x + blockIdx.x] = make_double2(v[0], v[1]);
-  }
-}
-
-// Same result with per-thread register accumulators: each thread walks its
-// sites (grid-stride) keeping one accumulator per j, so the CTA reduction
-// happens once per j per CTA instead of once per j per 256 sites.
+// Each thread walks its sites (grid-stride) keeping one accumulator per j;
+// per-j CTA sums go to part[r][j][cta].
 template <typename X, int KMAX>
 __global__ void __launch_bounds__(GS_TPB) k_multi_dot_acc(const char* __restrict__ chi, size_t jstride, int k, int V,
                                                            double2* __restrict__ part, const int* mask) {
-  __shared__ double sh[2 * 32];
+  using R = typename X::R;
+  __shared__ R sh[16 * GS_TPB];
   const int rhs = blockIdx.y;
   if (mask && !mask[rhs]) return;
-  using R = typename X::R;
   const size_t roff = (size_t)rhs * X::bytes * V;
   R ar[KMAX], ai[KMAX];
 #pragma unroll
@@ -396,12 +367,20 @@ __global__ void __launch_bounds__(GS_TPB) k_multi_dot_acc(const char* __restrict
       }
     }
   }
+  // eight j at a time
 #pragma unroll
-  for (int j = 0; j < KMAX; j++) {
-    if (j < k) {
-      double v[2] = {(double)ar[j], (double)ai[j]};
-      block_sum_n<2>(v, sh);
-      if (threadIdx.x == 0) part[((size_t)rhs * k + j) * gridDim.x + blockIdx.x] = make_double2(v[0], v[1]);
+  for (int j0 = 0; j0 < KMAX; j0 += 8) {
+    if (j0 < k) {
+      R v[16];
+#pragma unroll
+      for (int j = 0; j < 8; j++) {
+        v[2 * j] = ar[j0 + j];
+        v[2 * j + 1] = ai[j0 + j];
+      }
+      cta_sums<16>(v, sh, [&](int q, double t) {
+        const int j = j0 + (q >> 1);
+        if (j < k) ((double*)(part + ((size_t)rhs * k + j) * gridDim.x + blockIdx.x))[q & 1] = t;
+      });
     }
   }
 }
@@ -421,12 +400,21 @@ __global__ void __launch_bounds__(RED_TPB) k_sum_parts(const double2* __restrict
   if (threadIdx.x == 0) out[(size_t)j * nrhs + rhs] = t;
 }
 
+// the CTA's |chi_k|^2 and (chi_k, rho) to part[0][cta] and part[1][cta]
+template <typename R>
+__device__ inline void store_orth_sums(const R (&v)[3], R* sh, double2* part) {
+  cta_sums<3>(v, sh, [&](int q, double t) {
+    if (q == 0) part[blockIdx.x] = make_double2(t, 0.0);
+    else ((double*)(part + gridDim.x + blockIdx.x))[q - 1] = t;
+  });
+}
+
 // chi_k -= sum_{j<k} dots[j] chi_j; then partial sums of |chi_k|^2 and (chi_k, rho)
 template <typename X>
 __global__ void __launch_bounds__(GS_TPB) k_gs_orth(char* __restrict__ chi, size_t jstride, int k,
                                                      const double2* __restrict__ dots, const char* __restrict__ rho,
                                                      int V, int nrhs, double2* __restrict__ part, const int* mask) {
-  __shared__ double sh[3 * 32];
+  __shared__ double sh[3 * GS_TPB];
   const int rhs = blockIdx.y;
   if (mask && !mask[rhs]) return;
   using R = typename X::R;
@@ -454,13 +442,8 @@ __global__ void __launch_bounds__(GS_TPB) k_gs_orth(char* __restrict__ chi, size
       ci += (double)a.re * x.im - (double)a.im * x.re + (double)b.re * y.im - (double)b.im * y.re;
     }
   }
-  double v[3] = {n2, cr, ci};
-  block_sum_n<3>(v, sh);
-  if (threadIdx.x == 0) {
-    double2* p = part + (size_t)rhs * 2 * gridDim.x;
-    p[blockIdx.x] = make_double2(v[0], 0.0);
-    p[gridDim.x + blockIdx.x] = make_double2(v[1], v[2]);
-  }
+  const double v[3] = {n2, cr, ci};
+  store_orth_sums(v, sh, part + (size_t)rhs * 2 * gridDim.x);
 }
 
 // Site-major form of k_gs_orth: a thread holds all 12 components of chi_k
@@ -470,7 +453,8 @@ template <typename X, typename RH, int KMAX>
 __global__ void __launch_bounds__(GS_TPB) k_gs_orth_sm(char* __restrict__ chi, size_t jstride, int k,
                                                         const double2* __restrict__ dots, const char* __restrict__ rho,
                                                         int V, int nrhs, double2* __restrict__ part, const int* mask) {
-  __shared__ double sh[3 * 32];
+  using A = typename Acc<X, RH>::R;
+  __shared__ A sh[3 * GS_TPB];
   __shared__ float2 w_s[KMAX];
   const int rhs = blockIdx.y;
   if (mask && !mask[rhs]) return;
@@ -486,7 +470,6 @@ __global__ void __launch_bounds__(GS_TPB) k_gs_orth_sm(char* __restrict__ chi, s
   // per-thread sums in the arithmetic type of the pair (FP32 unless FP64 is
   // involved), widened to FP64 once per thread: FP64 arithmetic per site
   // would make the pass ALU-bound on this GPU
-  using A = typename Acc<X, RH>::R;
   A n2 = 0, cr = 0, ci = 0;
   for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < V; s += gridDim.x * blockDim.x) {
     Cplx<R> a[12];
@@ -515,13 +498,8 @@ __global__ void __launch_bounds__(GS_TPB) k_gs_orth_sm(char* __restrict__ chi, s
       ci = rfma(-ai, xr, ci);
     }
   }
-  double v[3] = {(double)n2, (double)cr, (double)ci};
-  block_sum_n<3>(v, sh);
-  if (threadIdx.x == 0) {
-    double2* pp = part + (size_t)rhs * 2 * gridDim.x;
-    pp[blockIdx.x] = make_double2(v[0], 0.0);
-    pp[gridDim.x + blockIdx.x] = make_double2(v[1], v[2]);
-  }
+  const A v[3] = {n2, cr, ci};
+  store_orth_sums(v, sh, part + (size_t)rhs * 2 * gridDim.x);
 }
 
 // Site-major y (FP64) += sign sum_{j<nx} coef_j x_j (FP32)
@@ -573,10 +551,10 @@ template <typename XC, typename XR>
 __global__ void __launch_bounds__(GS_TPB) k_gs_finish_inner(char* __restrict__ chik, const double* __restrict__ inv,
                                                              const double2* __restrict__ ck, char* __restrict__ rho,
                                                              int V, double2* __restrict__ part, const int* mask) {
-  __shared__ double sh[32];
+  using R = typename XR::R;
+  __shared__ R sh[GS_TPB];
   const int rhs = blockIdx.y;
   if (mask && !mask[rhs]) return;
-  using R = typename XR::R;
   char* cp = chik + (size_t)rhs * XC::bytes * V;
   char* rp = rho + (size_t)rhs * XR::bytes * V;
   const R f = (R)inv[rhs];
@@ -610,9 +588,8 @@ __global__ void __launch_bounds__(GS_TPB) k_gs_finish_inner(char* __restrict__ c
     st_site<XR>(rp, V, s, x);
     n2 += acc;
   }
-  double v[1] = {(double)n2};
-  block_sum_n<1>(v, sh);
-  if (threadIdx.x == 0) part[(size_t)rhs * gridDim.x + blockIdx.x] = make_double2(v[0], 0.0);
+  const R v[1] = {n2};
+  cta_sums<1>(v, sh, [&](int, double t) { part[(size_t)rhs * gridDim.x + blockIdx.x] = make_double2(t, 0.0); });
 }
 
 }  // namespace
