@@ -64,13 +64,6 @@ __device__ inline int blk_site(const BlkGeom& bg, const Geom& g, int blk, int l,
   for (int mu = 0; mu < 4; mu++) c[mu] = bc[mu] * bg.b[mu] + lc[mu];
   return ((c[0] * g.L[3] + c[3]) * g.L[2] + c[2]) * g.L[1] + c[1];
 }
-// block number of site with coordinates c
-__device__ inline int blk_of_site(const BlkGeom& bg, const int c[4]) {
-  int bc[4];
-  for (int mu = 0; mu < 4; mu++) bc[mu] = c[mu] / bg.b[mu];
-  return blk_index(bg, bc);
-}
-
 __device__ inline double2 dwarp_sum2(double2 v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -185,103 +178,157 @@ __global__ void __launch_bounds__(128) k_dfl_ypart(const char* __restrict__ phi,
 
 // ---------------------------------------------------------------------------
 // Per-block projection c[r][b][k] = sum_{y in b, comp} conj(Phi_k(y)) rho_r(y)
-// of the right-hand sides on the deflation fields.  One CTA per block; tiles
-// of TS sites of both operands are staged in shared memory.  (The little
-// Dirac operator itself is built on the tensor cores, dfl_tc.cu.)
+// of the unmasked right-hand sides on the deflation fields.  (The little Dirac
+// operator itself is built on the tensor cores, dfl_tc.cu.)
+//
+// One CTA per block.  Chunks of PTS sites of both operands are staged entry-major
+// (Pt[e][k], Rt[e][r], e = component * PTS + site; rows two words longer than the
+// tiles, so that consecutive sites fall into different banks).  A thread owns a tile of
+// 4 fields x 4 right-hand sides on one of the slices of the entries: four 128-bit
+// shared-memory reads for 16 complex products (one output per thread took two
+// reads a product, which bound the kernel).  The slices are summed in a fixed order
+// at the end.
 // ---------------------------------------------------------------------------
-constexpr int TS = 8;
+constexpr int PTS = 16;
 constexpr int GEMM_TPB = 256;
+constexpr int TK = 4, TR = 4;
 
-// Projection c[r][b][k] = (phi_k^b, rho_r) for the unmasked right-hand sides.
-// One CTA per block, tiles of TS sites: staging tasks of one field (phi_k or
-// rho_r) at one site, six 16-byte loads for its 12 components, stored entry-
-// major (Pt[e][k], Rt[e][r], e = site * 12 + component) so that the threads of
-// one RHS read consecutive words of Pt and one broadcast word of Rt.
+struct ProjectShape {
+  int tiles_k, tiles_r, slices, ldp, ldr;
+  size_t smem;
+};
+ProjectShape project_shape(int ns, int nrhs) {
+  ProjectShape s;
+  s.tiles_k = (ns + TK - 1) / TK;
+  s.tiles_r = (nrhs + TR - 1) / TR;
+  s.slices = GEMM_TPB / (s.tiles_k * s.tiles_r);   // ns <= 32, nrhs <= 24: at most 64 tiles
+  s.ldp = s.tiles_k * TK + 2;
+  s.ldr = s.tiles_r * TR + 2;
+  const size_t stage = (size_t)12 * PTS * (s.ldp + s.ldr);
+  const size_t red = (size_t)s.slices * s.tiles_k * s.tiles_r * TK * TR;
+  s.smem = sizeof(float2) * (stage > red ? stage : red);
+  return s;
+}
+
 __global__ void __launch_bounds__(GEMM_TPB) k_dfl_project(const char* __restrict__ phi, const char* __restrict__ rho,
                                                            float2* __restrict__ cout, Geom g, BlkGeom bg, int ns,
-                                                           int nrhs, const int* mask) {
+                                                           int nrhs, ProjectShape sh, const int* mask) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* Pt = (float2*)smem_raw;                // [12 TS][ns]
-  float2* Rt = Pt + (size_t)12 * TS * ns;        // [12 TS][nrhs]
+  float2* Pt = (float2*)smem_raw;                          // [12 PTS][ldp]
+  float2* Rt = Pt + (size_t)12 * PTS * sh.ldp;             // [12 PTS][ldr]
   const int blk = blockIdx.x;
   const size_t fb = FieldsF::spinor_bytes * (size_t)g.V;
-  const int nout = ns * nrhs;
-  const int nf = ns + nrhs;
-  Cplx<float> acc[4];
-  for (int o = 0; o < 4; o++) acc[o] = cmk(0.f, 0.f);
-  for (int t0 = 0; t0 < bg.vb; t0 += TS) {
+  const int kp = sh.tiles_k * TK, rp = sh.tiles_r * TR;    // padded rows (zeros beyond ns and nrhs)
+  const int ntile = sh.tiles_k * sh.tiles_r;
+  const int tile = threadIdx.x % ntile, slice = threadIdx.x / ntile;
+  const int k0 = (tile / sh.tiles_r) * TK, r0 = (tile % sh.tiles_r) * TR;
+  Cplx<float> acc[TK][TR];
+#pragma unroll
+  for (int i = 0; i < TK; i++)
+#pragma unroll
+    for (int j = 0; j < TR; j++) acc[i][j] = cmk(0.f, 0.f);
+  __shared__ int site[PTS];
+  for (int t0 = 0; t0 < bg.vb; t0 += PTS) {
     __syncthreads();
-    for (int task = threadIdx.x; task < nf * TS; task += blockDim.x) {
-      const int i = task % TS, f = task / TS;
+    if (threadIdx.x < PTS) {
       int lc[4], c[4];
-      const int s = blk_site(bg, g, blk, t0 + i, lc, c);
-      const bool isphi = f < ns;
-      const int r = f - ns;
-      const bool on = isphi || !mask || mask[r];
+      site[threadIdx.x] = blk_site(bg, g, blk, t0 + threadIdx.x, lc, c);
+    }
+    __syncthreads();
+    for (int task = threadIdx.x; task < (kp + rp) * PTS; task += blockDim.x) {
+      const int i = task % PTS, f = task / PTS;
+      const int s = site[i];
+      const bool isphi = f < kp;
+      const int r = f - kp;
+      const bool on = isphi ? f < ns : (r < nrhs && (!mask || mask[r]));
       const float4* src = (const float4*)(isphi ? phi + (size_t)f * fb : rho + (size_t)r * fb);
       float2* dst = isphi ? Pt + f : Rt + r;
-      const int st = isphi ? ns : nrhs;
+      const int ld = isphi ? sh.ldp : sh.ldr;
 #pragma unroll
       for (int q = 0; q < 6; q++) {
         const float4 v = on ? __ldg(src + (size_t)q * g.V + s) : make_float4(0.f, 0.f, 0.f, 0.f);
-        dst[(size_t)(i * 12 + 2 * q) * st] = make_float2(v.x, v.y);
-        dst[(size_t)(i * 12 + 2 * q + 1) * st] = make_float2(v.z, v.w);
+        dst[(2 * q * PTS + i) * ld] = make_float2(v.x, v.y);
+        dst[((2 * q + 1) * PTS + i) * ld] = make_float2(v.z, v.w);
       }
     }
     __syncthreads();
-    for (int o = 0; o < 4; o++) {
-      const int idx = threadIdx.x + o * GEMM_TPB;
-      if (idx >= nout) break;
-      const int r = idx / ns, k = idx - r * ns;
-      for (int e = 0; e < 12 * TS; e++) {
-        const float2 a = Pt[(size_t)e * ns + k], b = Rt[(size_t)e * nrhs + r];
-        cmac_conj(acc[o], cmk(a.x, a.y), cmk(b.x, b.y));
+    if (slice < sh.slices)
+      for (int e = slice; e < 12 * PTS; e += sh.slices) {
+        const float4* xp = (const float4*)(Pt + e * sh.ldp + k0);
+        const float4* yp = (const float4*)(Rt + e * sh.ldr + r0);
+        const float4 x0 = xp[0], x1 = xp[1], y0 = yp[0], y1 = yp[1];
+        const Cplx<float> x[TK] = {cmk(x0.x, x0.y), cmk(x0.z, x0.w), cmk(x1.x, x1.y), cmk(x1.z, x1.w)};
+        const Cplx<float> y[TR] = {cmk(y0.x, y0.y), cmk(y0.z, y0.w), cmk(y1.x, y1.y), cmk(y1.z, y1.w)};
+#pragma unroll
+        for (int i = 0; i < TK; i++)
+#pragma unroll
+          for (int j = 0; j < TR; j++) cmac_conj(acc[i][j], x[i], y[j]);
       }
-    }
   }
-  for (int o = 0; o < 4; o++) {
-    const int idx = threadIdx.x + o * GEMM_TPB;
-    if (idx >= nout) break;
-    const int r = idx / ns, k = idx - r * ns;
-    cout[((size_t)r * bg.nblk + blk) * ns + k] = make_float2(acc[o].re, acc[o].im);
+  __syncthreads();
+  float2* red = (float2*)smem_raw;   // [slice][r][k] over the padded rows
+  if (slice < sh.slices)
+#pragma unroll
+    for (int i = 0; i < TK; i++)
+#pragma unroll
+      for (int j = 0; j < TR; j++)
+        red[((size_t)slice * rp + r0 + j) * kp + k0 + i] = make_float2(acc[i][j].re, acc[i][j].im);
+  __syncthreads();
+  for (int o = threadIdx.x; o < ns * nrhs; o += blockDim.x) {
+    const int r = o / ns, k = o - r * ns;
+    float2 t = make_float2(0.f, 0.f);
+    for (int q = 0; q < sh.slices; q++) {
+      const float2 v = red[((size_t)q * rp + r) * kp + k];
+      t.x += v.x;
+      t.y += v.y;
+    }
+    cout[((size_t)r * bg.nblk + blk) * ns + k] = t;
   }
 }
 
-// Prolongation x_r(y) = sum_k e[r][b(y)][k] phi_k(y); one thread per (site, group of RG rhs)
-constexpr int RG = 4;
-__global__ void __launch_bounds__(128) k_dfl_prolong(const char* __restrict__ phi, const float2* __restrict__ e,
-                                                     char* __restrict__ x, Geom g, BlkGeom bg, int ns, int nrhs,
-                                                     const int* mask) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  const int r0 = blockIdx.y * RG;
-  if (s >= g.V) return;
-  const size_t fb = FieldsF::spinor_bytes * (size_t)g.V;
-  int c[4];
-  site_coords(g, s, c);
-  const int blk = blk_of_site(bg, c);
-  Spinor<float> acc[RG];
-#pragma unroll
-  for (int i = 0; i < RG; i++)
-#pragma unroll
-    for (int q = 0; q < 12; q++) acc[i].c[q] = cmk(0.f, 0.f);
-  for (int k = 0; k < ns; k++) {
-    Spinor<float> p = FieldsF::load_spinor(phi + k * fb, g.V, s);
-#pragma unroll
-    for (int i = 0; i < RG; i++) {
-      int r = r0 + i;
-      if (r >= nrhs) break;
-      float2 cf = __ldg(e + ((size_t)r * bg.nblk + blk) * ns + k);
-      Cplx<float> w = cmk(cf.x, cf.y);
-#pragma unroll
-      for (int q = 0; q < 12; q++) acc[i].c[q] = acc[i].c[q] + w * p.c[q];
-    }
+// Prolongation x_r(y) = sum_k e[r][b(y)][k] phi_k(y).  One CTA per block, threads
+// over its sites; the block's coefficients in shared memory; a thread takes two
+// components of up to 12 right-hand sides at a time, so phi is read once per 12.
+constexpr int PRG = 12;
+__global__ void __launch_bounds__(256) k_dfl_prolong(const char* __restrict__ phi, const float2* __restrict__ e, char* __restrict__ x, Geom g,
+                              BlkGeom bg, int ns, int nrhs, const int* mask) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* cf = (float2*)smem_raw;   // [k][nrhs rounded up to PRG], zeros beyond nrhs
+  const int blk = blockIdx.x, ld = (nrhs + PRG - 1) / PRG * PRG;
+  for (int o = threadIdx.x; o < ns * ld; o += blockDim.x) {
+    const int r = o / ns, k = o - r * ns;
+    cf[k * ld + r] = r < nrhs ? e[((size_t)r * bg.nblk + blk) * ns + k] : make_float2(0.f, 0.f);
   }
+  __syncthreads();
+  const size_t fb = FieldsF::spinor_bytes * (size_t)g.V;
+  for (int l = threadIdx.x; l < bg.vb; l += blockDim.x) {
+    int lc[4], c[4];
+    const int s = blk_site(bg, g, blk, l, lc, c);
+    for (int r0 = 0; r0 < nrhs; r0 += PRG)
+#pragma unroll 1
+      for (int q = 0; q < 6; q++) {
+        Cplx<float> a0[PRG], a1[PRG];
 #pragma unroll
-  for (int i = 0; i < RG; i++) {
-    int r = r0 + i;
-    if (r >= nrhs) break;
-    if (mask && !mask[r]) continue;
-    FieldsF::store_spinor(x + r * fb, g.V, s, acc[i]);
+        for (int i = 0; i < PRG; i++) a0[i] = a1[i] = cmk(0.f, 0.f);
+#pragma unroll 4
+        for (int k = 0; k < ns; k++) {
+          const float4 v = __ldg((const float4*)(phi + k * fb) + (size_t)q * g.V + s);
+          const float4* w = (const float4*)(cf + k * ld + r0);
+#pragma unroll
+          for (int i = 0; i < PRG; i += 2) {
+            const float4 u = w[i >> 1];
+            cmac(a0[i], cmk(u.x, u.y), cmk(v.x, v.y));
+            cmac(a1[i], cmk(u.x, u.y), cmk(v.z, v.w));
+            cmac(a0[i + 1], cmk(u.z, u.w), cmk(v.x, v.y));
+            cmac(a1[i + 1], cmk(u.z, u.w), cmk(v.z, v.w));
+          }
+        }
+#pragma unroll
+        for (int i = 0; i < PRG; i++)
+          if (r0 + i < nrhs && (!mask || mask[r0 + i]))
+            ((float4*)(x + (size_t)(r0 + i) * fb))[(size_t)q * g.V + s] =
+                make_float4(a0[i].re, a0[i].im, a1[i].re, a1[i].im);
+      }
   }
 }
 
@@ -372,35 +419,36 @@ __device__ inline void little_mac(float& ar, float& ai, float2 a, float2 v) {
   ai = fmaf(a.y, v.x, ai);
 }
 
-// y = A x (nparts = 9) or y = Ainv x (nparts = 1, diagonal blocks only).  One
-// CTA per block, thread (k, rr) = row k for the RHS rr, rr + rb, ...: the rb
-// threads of a row read the same matrix row (L1 broadcast), the ns threads of
-// an RHS the same neighbour vector.  MT = double2: FP64 products and sums;
-// float2: FP32.
-template <typename MT>
-__global__ void k_little_apply(const MT* __restrict__ M, int nparts, const float2* __restrict__ x,
-                               float2* __restrict__ y, BlkGeom bg, int ns, int nrhs, const int* mask) {
-  using RT = decltype(MT::x);
+// the blocks the nine parts of A couple a block to
+__device__ inline void little_neighbours(const BlkGeom& bg, int blk, int nbr[9]) {
+  int bc[4];
+  blk_coords(bg, blk, bc);
+  nbr[0] = blk;
+#pragma unroll
+  for (int mu = 0; mu < 4; mu++) {
+    int cc[4] = {bc[0], bc[1], bc[2], bc[3]};
+    cc[mu] = bc[mu] + 1 == bg.nb[mu] ? 0 : bc[mu] + 1;
+    nbr[1 + 2 * mu] = blk_index(bg, cc);
+    cc[mu] = bc[mu] == 0 ? bg.nb[mu] - 1 : bc[mu] - 1;
+    nbr[2 + 2 * mu] = blk_index(bg, cc);
+  }
+}
+
+// y = A x with the FP64 matrix (the test entry point).  One CTA per block, thread
+// (k, rr) = row k for the RHS rr, rr + rb, ...: the rb threads of a row read the same
+// matrix row (L1 broadcast), the ns threads of an RHS the same neighbour vector.
+__global__ void k_little_apply(const double2* __restrict__ M, const float2* __restrict__ x, float2* __restrict__ y,
+                               BlkGeom bg, int ns, int nrhs) {
   const int blk = blockIdx.x;
   const int k = threadIdx.x % ns, rr = threadIdx.x / ns;
   const int rb = blockDim.x / ns;
   if (rr >= rb) return;
-  int bc[4];
-  blk_coords(bg, blk, bc);
   int nbr[9];
-  nbr[0] = blk;
-  for (int mu = 0; mu < 4; mu++) {
-    int cc[4] = {bc[0], bc[1], bc[2], bc[3]};
-    cc[mu] = (bc[mu] + 1) % bg.nb[mu];
-    nbr[1 + 2 * mu] = blk_index(bg, cc);
-    cc[mu] = (bc[mu] - 1 + bg.nb[mu]) % bg.nb[mu];
-    nbr[2 + 2 * mu] = blk_index(bg, cc);
-  }
+  little_neighbours(bg, blk, nbr);
   for (int r = rr; r < nrhs; r += rb) {
-    if (mask && !mask[r]) continue;
-    RT ar = 0, ai = 0;
-    for (int p = 0; p < nparts; p++) {
-      const MT* row = M + (((size_t)blk * nparts + p) * ns + k) * ns;
+    double ar = 0, ai = 0;
+    for (int p = 0; p < 9; p++) {
+      const double2* row = M + (((size_t)blk * 9 + p) * ns + k) * ns;
       const float2* xv = x + ((size_t)r * bg.nblk + nbr[p]) * ns;
       for (int l = 0; l < ns; l++) little_mac(ar, ai, __ldg(row + l), __ldg(xv + l));
     }
@@ -414,94 +462,216 @@ __global__ void k_to_float2(const double2* __restrict__ in, float2* __restrict__
     out[i] = make_float2((float)in[i].x, (float)in[i].y);
 }
 
-// per-rhs dots d[j][r] = (q_j, v) for j < nj (q_j at qbase + j*stride): CTA
-// (g, j, r) sums chunk g of the product of q_j and v for RHS r into part
-// [r][j][g].  Products and the per-thread sums in FP32 (the vectors are FP32),
-// widened to FP64 once per thread for the sum across threads.
-__global__ void k_little_dots(const float2* __restrict__ qbase, size_t stride, int nj, const float2* __restrict__ v,
-                              int n, double2* __restrict__ part, const int* mask) {
-  __shared__ double2 sh[32];
-  const int g = blockIdx.x, j = blockIdx.y, r = blockIdx.z;
-  if (mask && !mask[r]) return;
-  const float2* q = qbase + j * stride + (size_t)r * n;
-  const float2* vv = v + (size_t)r * n;
-  float ar = 0.f, ai = 0.f;
-  for (int i = g * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const float2 a = q[i], b = vv[i];
-    ar = fmaf(a.x, b.x, ar);
-    ar = fmaf(a.y, b.y, ar);
-    ai = fmaf(a.x, b.y, ai);
-    ai = fmaf(-a.y, b.x, ai);
+// ---------------------------------------------------------------------------
+// The little GCR step in five launches (twelve before: product with the diagonal
+// inverses, product with A, dots, their sums, orthogonalisation, norm, its sum,
+// scaling, overlap, its sum, update).  The vectors of a 16^3x32 lattice are 1 MB
+// for 12 RHS, so a launch takes microseconds and their number counts.  Sums over
+// threads are FP64 in a fixed order; a CTA of the summing kernels is one warp (an FP64
+// addition of a warp takes the SM 16 cycles: the shuffle sums of 256 threads were
+// most of the time of the dots).  Masked right-hand sides have a zero residual and
+// stay zero.  A deflated 16^3x32 solve, 12 RHS, N_s 20, 24 steps: all deflation
+// kernels of an outer iteration 3.5 -> 1.75 ms.
+// ---------------------------------------------------------------------------
+constexpr int LTPB = 256;
+constexpr int LITTLE_G = 608;    // CTAs of the kernels that leave partial sums
+constexpr int LITTLE_RHS = 24;   // right-hand sides of one little solve
+constexpr int LITTLE_JR = 6;     // (j, r) sums per thread: 64 steps x 24 RHS / 256
+
+// q = A p on the CTA's blocks, and the CTA's partial sums of (q_j, q), j < nj, to
+// part[(r nj + j) gridDim + cta].  Per block the nine neighbours' p and the matrix
+// rows are staged in shared memory; thread (k, r), right-hand side fastest.
+__global__ void __launch_bounds__(LTPB) k_little_q(const float2* __restrict__ A, const float2* __restrict__ p,
+                                                   float2* __restrict__ q, const float2* __restrict__ qbase,
+                                                   size_t stride, int nj, double2* __restrict__ part, BlkGeom bg,
+                                                   int ns, int n) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* xs = (float2*)smem_raw;                 // [9 ns][n]
+  float2* As = xs + (size_t)9 * ns * n;           // [ns][9 ns]
+  float2* qs = As + (size_t)9 * ns * ns;          // [ns][n]
+  float2 acc[LITTLE_JR];
+#pragma unroll
+  for (int i = 0; i < LITTLE_JR; i++) acc[i] = make_float2(0.f, 0.f);
+  for (int blk = blockIdx.x; blk < bg.nblk; blk += gridDim.x) {
+    int nbr[9];
+    little_neighbours(bg, blk, nbr);
+    __syncthreads();
+    const float2* a = A + (size_t)blk * 9 * ns * ns;
+    for (int i = threadIdx.x; i < 9 * ns * ns; i += LTPB) {
+      const int mk = i / ns, m = mk / ns;
+      As[((mk - m * ns) * 9 + m) * ns + i - mk * ns] = __ldg(a + i);
+    }
+#pragma unroll
+    for (int m = 0; m < 9; m++)
+      for (int i = threadIdx.x; i < ns * n; i += LTPB) {
+        const int r = i / ns, k = i - r * ns;
+        xs[(m * ns + k) * n + r] = p[((size_t)r * bg.nblk + nbr[m]) * ns + k];
+      }
+    __syncthreads();
+    for (int o = threadIdx.x; o < ns * n; o += LTPB) {
+      const int k = o / n, r = o - k * n;
+      float ar = 0.f, ai = 0.f;
+      const float2* row = As + k * 9 * ns;
+#pragma unroll 9
+      for (int l = 0; l < 9 * ns; l++) little_mac(ar, ai, row[l], xs[l * n + r]);
+      qs[o] = make_float2(ar, ai);
+      q[((size_t)r * bg.nblk + blk) * ns + k] = qs[o];
+    }
+    if (nj == 0) continue;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < LITTLE_JR; i++) {
+      const int o = threadIdx.x + i * LTPB;
+      if (o < nj * n) {
+        const int j = o / n, r = o - j * n;
+        const float2* qj = qbase + j * stride + ((size_t)r * bg.nblk + blk) * ns;
+#pragma unroll 4
+        for (int k = 0; k < ns; k++) {
+          const float2 u = __ldg(qj + k), v = qs[k * n + r];
+          acc[i].x = fmaf(u.x, v.x, acc[i].x);
+          acc[i].x = fmaf(u.y, v.y, acc[i].x);
+          acc[i].y = fmaf(u.x, v.y, acc[i].y);
+          acc[i].y = fmaf(-u.y, v.x, acc[i].y);
+        }
+      }
+    }
   }
-  const double2 t = cta_sum2(make_double2(ar, ai), sh);
-  if (threadIdx.x == 0) part[((size_t)r * nj + j) * gridDim.x + g] = t;
+#pragma unroll
+  for (int i = 0; i < LITTLE_JR; i++) {
+    const int o = threadIdx.x + i * LTPB;
+    if (o < nj * n) {
+      const int j = o / n, r = o - j * n;
+      part[((size_t)r * nj + j) * gridDim.x + blockIdx.x] = make_double2((double)acc[i].x, (double)acc[i].y);
+    }
+  }
 }
 
-__global__ void k_little_sum(const double2* __restrict__ part, int nj, int G, double2* __restrict__ out, int nrhs,
-                             const int* mask) {
-  __shared__ double2 sh[32];
+// out[j][r] = sum over g of part[(r nj + j) G + g]: one warp per (j, r)
+__global__ void k_little_sum(const double2* __restrict__ part, int nj, int G, double2* __restrict__ out, int n) {
   const int j = blockIdx.x, r = blockIdx.y;
-  if (mask && !mask[r]) return;
-  double2 acc = make_double2(0, 0);
-  for (int i = threadIdx.x; i < G; i += blockDim.x) {
-    double2 v = part[((size_t)r * nj + j) * G + i];
-    acc.x += v.x;
-    acc.y += v.y;
+  double2 t = make_double2(0, 0);
+  for (int i = threadIdx.x; i < G; i += 32) {
+    const double2 v = part[((size_t)r * nj + j) * G + i];
+    t.x += v.x;
+    t.y += v.y;
   }
-  double2 t = cta_sum2(acc, sh);
-  if (threadIdx.x == 0) out[(size_t)j * nrhs + r] = t;
+  t = dwarp_sum2(t);
+  if (threadIdx.x == 0) out[(size_t)j * n + r] = t;
 }
 
-// y_r -= sum_{j<nj} d[j][r] q_j for two vector families at once (q and p)
-__global__ void k_little_orth(float2* __restrict__ qi, float2* __restrict__ pi, const float2* __restrict__ qbase,
-                              const float2* __restrict__ pbase, size_t stride, int nj, const double2* __restrict__ d,
-                              int n, int nrhs, const int* mask) {
+// q -= sum_j d_j q_j, p -= sum_j d_j p_j; CTA partial sums of |q|^2 (part[r][0])
+// and (q, res) (part[r][1])
+__global__ void __launch_bounds__(LTPB) k_little_orth(float2* __restrict__ qi, float2* __restrict__ pi,
+                                                      const float2* __restrict__ qbase,
+                                                      const float2* __restrict__ pbase, size_t stride, int nj,
+                                                      const double2* __restrict__ d, const float2* __restrict__ res,
+                                                      int N, int n, double2* __restrict__ part) {
+  __shared__ float2 ds[64];
+  __shared__ float sh[3][LTPB];
   const int r = blockIdx.y;
-  if (mask && !mask[r]) return;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    size_t o = (size_t)r * n + i;
+  if ((int)threadIdx.x < nj) {
+    const double2 v = d[(size_t)threadIdx.x * n + r];
+    ds[threadIdx.x] = make_float2((float)v.x, (float)v.y);
+  }
+  __syncthreads();
+  float n2 = 0.f, cr = 0.f, ci = 0.f;
+  for (int i = blockIdx.x * LTPB + threadIdx.x; i < N; i += gridDim.x * LTPB) {
+    const size_t o = (size_t)r * N + i;
     float2 q = qi[o], p = pi[o];
+#pragma unroll 4
     for (int j = 0; j < nj; j++) {
-      double2 dj = d[(size_t)j * nrhs + r];
-      float dr = (float)dj.x, di = (float)dj.y;
-      float2 a = qbase[j * stride + o], b = pbase[j * stride + o];
-      q.x -= dr * a.x - di * a.y; q.y -= dr * a.y + di * a.x;
-      p.x -= dr * b.x - di * b.y; p.y -= dr * b.y + di * b.x;
+      const float2 w = ds[j], a = __ldg(qbase + j * stride + o), b = __ldg(pbase + j * stride + o);
+      q.x -= w.x * a.x - w.y * a.y; q.y -= w.x * a.y + w.y * a.x;
+      p.x -= w.x * b.x - w.y * b.y; p.y -= w.x * b.y + w.y * b.x;
     }
     qi[o] = q;
     pi[o] = p;
+    const float2 v = res[o];
+    n2 = fmaf(q.x, q.x, n2);
+    n2 = fmaf(q.y, q.y, n2);
+    cr = fmaf(q.x, v.x, cr);
+    cr = fmaf(q.y, v.y, cr);
+    ci = fmaf(q.x, v.y, ci);
+    ci = fmaf(-q.y, v.x, ci);
+  }
+  sh[0][threadIdx.x] = n2;
+  sh[1][threadIdx.x] = cr;
+  sh[2][threadIdx.x] = ci;
+  __syncthreads();
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  if (w < 3) {
+    double t = 0;
+#pragma unroll
+    for (int i = 0; i < LTPB / 32; i++) t += (double)sh[w][32 * i + l];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (l == 0) {
+      double* out = (double*)(part + (size_t)r * 2 * gridDim.x);
+      if (w == 0) out[2 * blockIdx.x] = t;
+      else out[2 * (gridDim.x + blockIdx.x) + w - 1] = t;
+    }
   }
 }
 
-// q /= |q|, p /= |q| (nrm2 from the dots kernel), then alpha = (q, res):
-// done in two steps; here the scaling
-__global__ void k_little_scale2(float2* __restrict__ q, float2* __restrict__ p, const double2* __restrict__ n2, int n,
-                                const int* mask) {
-  const int r = blockIdx.y;
-  if (mask && !mask[r]) return;
-  double v = n2[r].x;
-  float f = v > 0 ? (float)(1.0 / sqrt(v)) : 0.f;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    size_t o = (size_t)r * n + i;
-    q[o].x *= f; q[o].y *= f;
-    p[o].x *= f; p[o].y *= f;
+// from the partial sums of k_little_orth: f = 1/|q| and alpha = (q, res)/|q|^2 (the
+// step along the normalised q is alpha |q|), per right-hand side {f, alpha |q|}
+__global__ void k_little_scalars(const double2* __restrict__ part, int G, float4* __restrict__ out) {
+  const int r = blockIdx.x;
+  double2 a = make_double2(0, 0), c = make_double2(0, 0);
+  for (int i = threadIdx.x; i < G; i += 32) {
+    a.x += part[(size_t)r * 2 * G + i].x;
+    const double2 v = part[((size_t)r * 2 + 1) * G + i];
+    c.x += v.x;
+    c.y += v.y;
+  }
+  a = dwarp_sum2(a);
+  c = dwarp_sum2(c);
+  if (threadIdx.x == 0) {
+    const double f = a.x > 0 ? 1.0 / sqrt(a.x) : 0.0;
+    out[r] = make_float4((float)f, (float)(c.x * f), (float)(c.y * f), 0.f);
   }
 }
 
-// x += alpha p, res -= alpha q
-__global__ void k_little_update(float2* __restrict__ x, float2* __restrict__ res, const float2* __restrict__ p,
-                                const float2* __restrict__ q, const double2* __restrict__ alpha, int n,
-                                const int* mask) {
-  const int r = blockIdx.y;
-  if (mask && !mask[r]) return;
-  float ar = (float)alpha[r].x, ai = (float)alpha[r].y;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    size_t o = (size_t)r * n + i;
-    float2 pp = p[o], qq = q[o], xx = x[o], rr = res[o];
-    xx.x += ar * pp.x - ai * pp.y; xx.y += ar * pp.y + ai * pp.x;
-    rr.x -= ar * qq.x - ai * qq.y; rr.y -= ar * qq.y + ai * qq.x;
-    x[o] = xx;
-    res[o] = rr;
+// q, p normalised; x += alpha p, res -= alpha q (first: x = alpha p); pnext = the
+// diagonal-block inverses times the new residual.  start: only that product.
+__global__ void __launch_bounds__(LTPB) k_little_step(float2* __restrict__ x, float2* __restrict__ res,
+                                                      float2* __restrict__ p, float2* __restrict__ q,
+                                                      float2* __restrict__ pnext, const float2* __restrict__ Ainv,
+                                                      const float4* __restrict__ sc, int first, int start, BlkGeom bg,
+                                                      int ns, int n) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* rs = (float2*)smem_raw;                 // [ns][n]
+  float2* As = rs + (size_t)ns * n;               // [ns][ns]
+  for (int blk = blockIdx.x; blk < bg.nblk; blk += gridDim.x) {
+    __syncthreads();
+    if (pnext)
+      for (int i = threadIdx.x; i < ns * ns; i += LTPB) As[i] = __ldg(Ainv + (size_t)blk * ns * ns + i);
+    for (int i = threadIdx.x; i < ns * n; i += LTPB) {
+      const int r = i / ns, k = i - r * ns;
+      const size_t o = ((size_t)r * bg.nblk + blk) * ns + k;
+      float2 v = res[o];
+      if (!start) {
+        const float4 c = sc[r];
+        float2 pp = p[o], qq = q[o], xx = first ? make_float2(0.f, 0.f) : x[o];
+        pp.x *= c.x; pp.y *= c.x;
+        qq.x *= c.x; qq.y *= c.x;
+        xx.x += c.y * pp.x - c.z * pp.y; xx.y += c.y * pp.y + c.z * pp.x;
+        v.x -= c.y * qq.x - c.z * qq.y; v.y -= c.y * qq.y + c.z * qq.x;
+        p[o] = pp;
+        q[o] = qq;
+        x[o] = xx;
+        res[o] = v;
+      }
+      rs[k * n + r] = v;
+    }
+    if (!pnext) continue;
+    __syncthreads();
+    for (int i = threadIdx.x; i < ns * n; i += LTPB) {
+      const int k = i / n, r = i - k * n;
+      float ar = 0.f, ai = 0.f;
+      for (int l = 0; l < ns; l++) little_mac(ar, ai, As[k * ns + l], rs[l * n + r]);
+      pnext[((size_t)r * bg.nblk + blk) * ns + k] = make_float2(ar, ai);
+    }
   }
 }
 
@@ -606,39 +776,55 @@ static int little_threads(int ns, int n) {
   return ns * rb;
 }
 
-// m steps of block-Jacobi preconditioned GCR on the little vectors from x = 0:
-// res holds the right-hand side on entry and the residual on exit, xl the
-// approximate solution; P, Q: m (p, q) pairs of vlen float2 each.
-static qcd_status little_gcr(qcd_ctx* c, DflState* d, float2* res, float2* xl, float2* P, float2* Q, double2* part,
-                             double2* dots, int n, int m, const int* mask) {
+// scratch of little_gcr in d->part: partial sums, dots, scalars
+static size_t little_part_count(int n, int m) { return (size_t)n * (m + 2) * LITTLE_G; }
+static size_t little_part_bytes(int n, int m) {
+  if (n > LITTLE_RHS) n = LITTLE_RHS;
+  return sizeof(double2) * (little_part_count(n, m) + (size_t)(m + 2) * n) + sizeof(float4) * n;
+}
+
+// little_gcr for at most LITTLE_RHS right-hand sides; vlen: distance of P's and Q's vectors
+static qcd_status little_gcr_tile(qcd_ctx* c, DflState* d, float2* res, float2* xl, float2* P, float2* Q, size_t vlen,
+                                  int n, int m) {
   const BlkGeom& bg = d->bg;
   const int ns = d->ns;
   const int N = bg.nblk * ns;
-  const size_t vlen = (size_t)N * n;
-  const int G = 64;
-  const dim3 gv(G, n);
-  // dot chunks of about 8 elements per thread (at most G)
-  const int Gd = (N + 2047) / 2048 < G ? (N + 2047) / 2048 : G;
-  const int nt = little_threads(ns, n);
-  QCD_CUDA_OK(cudaMemsetAsync(xl, 0, sizeof(float2) * vlen, c->stream));
+  double2* part = (double2*)d->part.p;
+  double2* dots = part + little_part_count(n, m);
+  float4* sc = (float4*)(dots + (size_t)(m + 2) * n);
+  const int Gq = bg.nblk < LITTLE_G ? bg.nblk : LITTLE_G;
+  // one element per thread of the orthogonalisation (its time is the latency of the
+  // loads along j), at most LITTLE_G CTAs per RHS
+  const int Go = (N + LTPB - 1) / LTPB < LITTLE_G ? (N + LTPB - 1) / LTPB : LITTLE_G;
+  const size_t sm_q = sizeof(float2) * ((size_t)9 * ns * n + (size_t)9 * ns * ns + (size_t)ns * n);
+  const size_t sm_s = sizeof(float2) * ((size_t)ns * n + (size_t)ns * ns);
+  QCD_CUDA_OK(cudaFuncSetAttribute(k_little_q, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_q));
+  const float2* Ainv = (const float2*)d->Ainvf.p;
+  const unsigned Gs = (unsigned)bg.nblk;
+  k_little_step<<<Gs, LTPB, sm_s, c->stream>>>(xl, res, nullptr, nullptr, P, Ainv, sc, 0, 1, bg, ns, n);
   for (int i = 0; i < m; i++) {
     float2* pi = P + vlen * i;
     float2* qi = Q + vlen * i;
-    k_little_apply<float2><<<bg.nblk, nt, 0, c->stream>>>((const float2*)d->Ainvf.p, 1, res, pi, bg, ns, n, mask);
-    k_little_apply<float2><<<bg.nblk, nt, 0, c->stream>>>((const float2*)d->Af.p, 9, pi, qi, bg, ns, n, mask);
-    if (i > 0) {
-      k_little_dots<<<dim3(Gd, i, n), 256, 0, c->stream>>>(Q, vlen, i, qi, N, part, mask);
-      k_little_sum<<<dim3(i, n), 256, 0, c->stream>>>(part, i, Gd, dots, n, mask);
-      k_little_orth<<<gv, 256, 0, c->stream>>>(qi, pi, Q, P, vlen, i, dots, N, n, mask);
-    }
-    k_little_dots<<<dim3(Gd, 1, n), 256, 0, c->stream>>>(qi, 0, 1, qi, N, part, mask);
-    k_little_sum<<<dim3(1, n), 256, 0, c->stream>>>(part, 1, Gd, dots, n, mask);
-    k_little_scale2<<<gv, 256, 0, c->stream>>>(qi, pi, dots, N, mask);
-    k_little_dots<<<dim3(Gd, 1, n), 256, 0, c->stream>>>(qi, 0, 1, res, N, part, mask);
-    k_little_sum<<<dim3(1, n), 256, 0, c->stream>>>(part, 1, Gd, dots, n, mask);
-    k_little_update<<<gv, 256, 0, c->stream>>>(xl, res, pi, qi, dots, N, mask);
+    k_little_q<<<Gq, LTPB, sm_q, c->stream>>>((const float2*)d->Af.p, pi, qi, Q, vlen, i, part, bg, ns, n);
+    if (i > 0) k_little_sum<<<dim3(i, n), 32, 0, c->stream>>>(part, i, Gq, dots, n);
+    k_little_orth<<<dim3(Go, n), LTPB, 0, c->stream>>>(qi, pi, Q, P, vlen, i, dots, res, N, n, part);
+    k_little_scalars<<<n, 32, 0, c->stream>>>(part, Go, sc);
+    k_little_step<<<Gs, LTPB, sm_s, c->stream>>>(xl, res, pi, qi, i + 1 < m ? pi + vlen : nullptr, Ainv, sc, i == 0, 0,
+                                                 bg, ns, n);
   }
   QCD_CUDA_OK(cudaGetLastError());
+  return QCD_OK;
+}
+
+// m steps of block-Jacobi preconditioned GCR on the little vectors from x = 0:
+// res holds the right-hand side on entry and the residual on exit, xl the
+// approximate solution; P, Q: m (p, q) pairs of n little vectors each.  Every
+// right-hand side is a problem of its own; they are taken LITTLE_RHS at a time.
+static qcd_status little_gcr(qcd_ctx* c, DflState* d, float2* res, float2* xl, float2* P, float2* Q, int n, int m) {
+  const size_t N = (size_t)d->bg.nblk * d->ns;
+  for (int r0 = 0; r0 < n; r0 += LITTLE_RHS)
+    QCD_TRY(little_gcr_tile(c, d, res + N * r0, xl + N * r0, P + N * r0, Q + N * r0, N * n,
+                            n - r0 < LITTLE_RHS ? n - r0 : LITTLE_RHS, m));
   return QCD_OK;
 }
 
@@ -724,35 +910,35 @@ qcd_status dfl_low_mode(qcd_ctx* c, const void* rho, void* x, int n, const int* 
   }
   const int N = bg.nblk * ns;                     // little vector length per rhs
   const size_t vlen = (size_t)N * n;              // float2 per little vector (all rhs)
-  // little workspace: rhs c, residual, x, then m (p, q) pairs
-  QCD_TRY(devbuf_ensure(d->little, sizeof(float2) * vlen * (3 + 2 * (size_t)m)));
-  float2* cl = (float2*)d->little.p;
-  float2* res = cl + vlen;
+  // little workspace: residual (the projection on entry), x, then m (p, q) pairs
+  QCD_TRY(devbuf_ensure(d->little, sizeof(float2) * vlen * (2 + 2 * (size_t)m)));
+  float2* res = (float2*)d->little.p;
   float2* xl = res + vlen;
   float2* P = xl + vlen;
   float2* Q = P + vlen * m;
-  const int G = 64;
-  QCD_TRY(devbuf_ensure(d->part, sizeof(double2) * ((size_t)n * (m + 2) * G + (size_t)(m + 2) * n)));
-  double2* part = (double2*)d->part.p;
-  double2* dots = part + (size_t)n * (m + 2) * G;
+  QCD_TRY(devbuf_ensure(d->part, little_part_bytes(n, m)));
   {
-    const size_t smem = sizeof(Cplx<float>) * (size_t)(ns + n) * 12 * TS;
     ProfScope ps(c, FAM_DFL, (double)spinor_bytes(c, QCD_PREC_F32) * (ns + nactive), 8.0 * c->g.V * 12 * ns * nactive);
-    QCD_CUDA_OK(cudaFuncSetAttribute(k_dfl_project, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    k_dfl_project<<<bg.nblk, GEMM_TPB, smem, c->stream>>>((const char*)d->phi.p, (const char*)rho, cl, c->g, bg, ns, n,
-                                                           mask);
-    QCD_CUDA_OK(cudaGetLastError());
+    for (int r0 = 0; r0 < n; r0 += LITTLE_RHS) {   // at most 64 tiles of outputs
+      const int nr = n - r0 < LITTLE_RHS ? n - r0 : LITTLE_RHS;
+      const ProjectShape sh = project_shape(ns, nr);
+      QCD_CUDA_OK(cudaFuncSetAttribute(k_dfl_project, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem));
+      k_dfl_project<<<bg.nblk, GEMM_TPB, sh.smem, c->stream>>>(
+          (const char*)d->phi.p, (const char*)rho + spinor_bytes(c, QCD_PREC_F32) * r0, res + (size_t)N * r0, c->g, bg,
+          ns, nr, sh, mask ? mask + r0 : nullptr);
+      QCD_CUDA_OK(cudaGetLastError());
+    }
   }
   // little GCR with block-Jacobi preconditioning, x = 0 start, m steps
   {
-    ProfScope ps(c, FAM_DFL, 8.0 * vlen * (6.0 + 3.0 * m) * m, 0.0, 4 + 8 * m);
-    QCD_CUDA_OK(cudaMemcpyAsync(res, cl, sizeof(float2) * vlen, cudaMemcpyDeviceToDevice, c->stream));
-    QCD_TRY(little_gcr(c, d, res, xl, P, Q, part, dots, n, m, mask));
+    ProfScope ps(c, FAM_DFL, 8.0 * vlen * (6.0 + 3.0 * m) * m, 0.0, 5 * m);
+    QCD_TRY(little_gcr(c, d, res, xl, P, Q, n, m));
   }
   {
     ProfScope ps(c, FAM_DFL, (double)spinor_bytes(c, QCD_PREC_F32) * (ns + nactive), 8.0 * c->g.V * 12 * ns * nactive);
-    dim3 grid((c->g.V + 127) / 128, (n + RG - 1) / RG);
-    k_dfl_prolong<<<grid, 128, 0, c->stream>>>((const char*)d->phi.p, xl, (char*)x, c->g, bg, ns, n, mask);
+    k_dfl_prolong<<<bg.nblk, bg.vb < 256 ? bg.vb : 256, sizeof(float2) * ns * ((n + PRG - 1) / PRG * PRG), c->stream>>>(
+        (const char*)d->phi.p, xl, (char*)x, c->g, bg,
+                                                                         ns, n, mask);
     QCD_CUDA_OK(cudaGetLastError());
   }
   return QCD_OK;
@@ -772,21 +958,17 @@ qcd_status dfl_little_host(qcd_ctx* c, const double* in, double* out, int n, int
   float2* y = x + vlen;
   QCD_CUDA_OK(cudaMemcpyAsync(x, h.data(), sizeof(float2) * vlen, cudaMemcpyHostToDevice, c->stream));
   if (mode == 0) {
-    k_little_apply<double2><<<d->bg.nblk, little_threads(d->ns, n), 0, c->stream>>>((const double2*)d->A.p, 9, x, y,
-                                                                                    d->bg, d->ns, n, nullptr);
+    k_little_apply<<<d->bg.nblk, little_threads(d->ns, n), 0, c->stream>>>((const double2*)d->A.p, x, y, d->bg, d->ns, n);
   } else {
-    // reuse the solver on little vectors: the projection is skipped by copying x into the rhs slot
-    QCD_TRY(devbuf_ensure(d->little, sizeof(float2) * vlen * (3 + 2 * (size_t)m)));
-    const int G = 64;
-    QCD_TRY(devbuf_ensure(d->part, sizeof(double2) * ((size_t)n * (m + 2) * G + (size_t)(m + 2) * n)));
-    float2* res = (float2*)d->little.p + vlen;
+    // the solver on little vectors, without projection and prolongation
+    QCD_TRY(devbuf_ensure(d->little, sizeof(float2) * vlen * (2 + 2 * (size_t)m)));
+    QCD_TRY(devbuf_ensure(d->part, little_part_bytes(n, m)));
+    float2* res = (float2*)d->little.p;
     float2* xl = res + vlen;
     float2* P = xl + vlen;
     float2* Q = P + vlen * m;
-    double2* part = (double2*)d->part.p;
-    double2* dots = part + (size_t)n * (m + 2) * G;
     QCD_CUDA_OK(cudaMemcpyAsync(res, x, sizeof(float2) * vlen, cudaMemcpyDeviceToDevice, c->stream));
-    QCD_TRY(little_gcr(c, d, res, xl, P, Q, part, dots, n, m, nullptr));
+    QCD_TRY(little_gcr(c, d, res, xl, P, Q, n, m));
     QCD_CUDA_OK(cudaMemcpyAsync(y, xl, sizeof(float2) * vlen, cudaMemcpyDeviceToDevice, c->stream));
   }
   QCD_CUDA_OK(cudaGetLastError());
