@@ -1,5 +1,7 @@
 // Field layouts: canonical FP64 <-> internal structure-of-arrays copies, and
 // the clover term built from plaquette leaves on the device.
+#include <type_traits>
+
 #include "qcd_internal.cuh"
 
 namespace {
@@ -184,61 +186,74 @@ __global__ void k_clover_export(const double2* __restrict__ clD, int V, double2*
   }
 }
 
-// canonical [rhs][V][12] complex -> internal (prec 0: double2[rhs][12][V]; 1: float4[rhs][6][V])
-template <typename T>
-__global__ void k_spinor_import(const double2* __restrict__ in, T* __restrict__ out, int V, int nrhs);
+// canonical [rhs][V][12] complex <-> internal (double2 [rhs][12][V] or float4
+// [rhs][6][V]).  A CTA moves LNS sites of one right-hand side through shared memory:
+// the canonical side is one contiguous run, the internal side a run per plane, both
+// read and written with consecutive threads on consecutive words.  (One thread per
+// site, 192 bytes apart on the canonical side, reached 3.6 TB/s, this 6.7.)
+constexpr int LNS = 64;          // sites per CTA
+constexpr int LLD = LNS + 1;     // words of a component's row in shared memory
 
-template <>
-__global__ void k_spinor_import<double2>(const double2* __restrict__ in, double2* __restrict__ out, int V, int nrhs) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)V * nrhs) return;
-  int s = (int)(i % V);
-  size_t r = i / V;
-  const double2* p = in + i * 12;
+template <typename T>
+__global__ void __launch_bounds__(TPB) k_spinor_import(const double2* __restrict__ in, T* __restrict__ out, int V) {
+  __shared__ double2 sm[12 * LLD];
+  const int nch = (V + LNS - 1) / LNS;
+  const size_t r = blockIdx.x / nch;
+  const int s0 = (blockIdx.x - (unsigned)r * nch) * LNS, ns = V - s0 < LNS ? V - s0 : LNS;
+  const double2* p = in + (r * V + s0) * 12;
 #pragma unroll
-  for (int c = 0; c < 12; c++) out[(r * 12 + c) * V + s] = p[c];
-}
-template <>
-__global__ void k_spinor_import<float4>(const double2* __restrict__ in, float4* __restrict__ out, int V, int nrhs) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)V * nrhs) return;
-  int s = (int)(i % V);
-  size_t r = i / V;
-  const double2* p = in + i * 12;
+  for (int k = 0; k < 12 * LNS / TPB; k++) {
+    const int i = k * TPB + threadIdx.x;
+    if (i < 12 * ns) sm[(i % 12) * LLD + i / 12] = __ldg(p + i);
+  }
+  __syncthreads();
+  if constexpr (std::is_same<T, double2>::value) {
 #pragma unroll
-  for (int k = 0; k < 6; k++) {
-    double2 a = p[2 * k], b = p[2 * k + 1];
-    out[(r * 6 + k) * V + s] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+    for (int k = 0; k < 12 * LNS / TPB; k++) {
+      const int i = k * TPB + threadIdx.x, c = i / LNS, s = i % LNS;
+      if (s < ns) out[(r * 12 + c) * V + s0 + s] = sm[c * LLD + s];
+    }
+  } else {
+    for (int i = threadIdx.x; i < 6 * LNS; i += TPB) {
+      const int k = i / LNS, s = i % LNS;
+      const double2 a = sm[2 * k * LLD + s], b = sm[(2 * k + 1) * LLD + s];
+      if (s < ns) out[(r * 6 + k) * V + s0 + s] = make_float4((float)a.x, (float)a.y, (float)b.x, (float)b.y);
+    }
   }
 }
 
 template <typename T>
-__global__ void k_spinor_export(const T* __restrict__ in, double2* __restrict__ out, int V, int nrhs);
-
-template <>
-__global__ void k_spinor_export<double2>(const double2* __restrict__ in, double2* __restrict__ out, int V, int nrhs) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)V * nrhs) return;
-  int s = (int)(i % V);
-  size_t r = i / V;
-  double2* p = out + i * 12;
+__global__ void __launch_bounds__(TPB) k_spinor_export(const T* __restrict__ in, double2* __restrict__ out, int V) {
+  __shared__ double2 sm[12 * LLD];
+  const int nch = (V + LNS - 1) / LNS;
+  const size_t r = blockIdx.x / nch;
+  const int s0 = (blockIdx.x - (unsigned)r * nch) * LNS, ns = V - s0 < LNS ? V - s0 : LNS;
+  if constexpr (std::is_same<T, double2>::value) {
 #pragma unroll
-  for (int c = 0; c < 12; c++) p[c] = in[(r * 12 + c) * V + s];
-}
-template <>
-__global__ void k_spinor_export<float4>(const float4* __restrict__ in, double2* __restrict__ out, int V, int nrhs) {
-  size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)V * nrhs) return;
-  int s = (int)(i % V);
-  size_t r = i / V;
-  double2* p = out + i * 12;
+    for (int k = 0; k < 12 * LNS / TPB; k++) {
+      const int i = k * TPB + threadIdx.x, c = i / LNS, s = i % LNS;
+      if (s < ns) sm[c * LLD + s] = __ldg(in + (r * 12 + c) * V + s0 + s);
+    }
+  } else {
+    for (int i = threadIdx.x; i < 6 * LNS; i += TPB) {
+      const int k = i / LNS, s = i % LNS;
+      if (s < ns) {
+        const float4 v = __ldg(in + (r * 6 + k) * V + s0 + s);
+        sm[2 * k * LLD + s] = make_double2(v.x, v.y);
+        sm[(2 * k + 1) * LLD + s] = make_double2(v.z, v.w);
+      }
+    }
+  }
+  __syncthreads();
+  double2* p = out + (r * V + s0) * 12;
 #pragma unroll
-  for (int k = 0; k < 6; k++) {
-    float4 v = in[(r * 6 + k) * V + s];
-    p[2 * k] = make_double2(v.x, v.y);
-    p[2 * k + 1] = make_double2(v.z, v.w);
+  for (int k = 0; k < 12 * LNS / TPB; k++) {
+    const int i = k * TPB + threadIdx.x;
+    if (i < 12 * ns) p[i] = sm[(i % 12) * LLD + i / 12];
   }
 }
+
+inline unsigned spinor_grid(int V, int nrhs) { return (unsigned)((V + LNS - 1) / LNS) * nrhs; }
 
 }  // namespace
 
@@ -271,23 +286,25 @@ qcd_status clover_export(qcd_ctx* c, double* out_dev) {
 }
 
 qcd_status layout_spinor_import(qcd_ctx* c, const double* in, void* out, int prec, int nrhs) {
-  size_t n = (size_t)c->g.V * nrhs;
+  const size_t n = (size_t)c->g.V * nrhs;
+  const unsigned grid = spinor_grid(c->g.V, nrhs);
   ProfScope ps(c, FAM_LAYOUT, (double)n * (192 + (prec == QCD_PREC_F64 ? 192 : 96)), 0.0);
   if (prec == QCD_PREC_F64)
-    k_spinor_import<double2><<<nblk(n), TPB, 0, c->stream>>>((const double2*)in, (double2*)out, c->g.V, nrhs);
+    k_spinor_import<double2><<<grid, TPB, 0, c->stream>>>((const double2*)in, (double2*)out, c->g.V);
   else
-    k_spinor_import<float4><<<nblk(n), TPB, 0, c->stream>>>((const double2*)in, (float4*)out, c->g.V, nrhs);
+    k_spinor_import<float4><<<grid, TPB, 0, c->stream>>>((const double2*)in, (float4*)out, c->g.V);
   QCD_CUDA_OK(cudaGetLastError());
   return QCD_OK;
 }
 
 qcd_status layout_spinor_export(qcd_ctx* c, const void* in, double* out, int prec, int nrhs) {
-  size_t n = (size_t)c->g.V * nrhs;
+  const size_t n = (size_t)c->g.V * nrhs;
+  const unsigned grid = spinor_grid(c->g.V, nrhs);
   ProfScope ps(c, FAM_LAYOUT, (double)n * (192 + (prec == QCD_PREC_F64 ? 192 : 96)), 0.0);
   if (prec == QCD_PREC_F64)
-    k_spinor_export<double2><<<nblk(n), TPB, 0, c->stream>>>((const double2*)in, (double2*)out, c->g.V, nrhs);
+    k_spinor_export<double2><<<grid, TPB, 0, c->stream>>>((const double2*)in, (double2*)out, c->g.V);
   else
-    k_spinor_export<float4><<<nblk(n), TPB, 0, c->stream>>>((const float4*)in, (double2*)out, c->g.V, nrhs);
+    k_spinor_export<float4><<<grid, TPB, 0, c->stream>>>((const float4*)in, (double2*)out, c->g.V);
   QCD_CUDA_OK(cudaGetLastError());
   return QCD_OK;
 }
