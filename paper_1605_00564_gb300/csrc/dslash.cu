@@ -18,7 +18,7 @@
 
 namespace {
 
-constexpr int DSLASH_TPB = 128;
+constexpr int DSLASH_TPB = 128;   // sites of a run; CTAs of 128 threads, or 32 on small problems (launch)
 
 // cp: runs of DSLASH_TPB sites per (t, z) plane (0: plain lexicographic
 // order); zw: z planes per slab

@@ -24,6 +24,7 @@
 
 #include <type_traits>
 
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -37,6 +38,22 @@ struct SapGeom {
   int lst[4];   // local stride of direction mu inside a block
   int vb;       // block volume
 };
+
+// the blk-th block of a colour
+__device__ __forceinline__ void block_of(const SapGeom& sg, int colour, int blk, int bc[4]) {
+  const int nbx2 = sg.nb[1] >> 1;
+  int q = blk / nbx2;
+  const int j = blk - q * nbx2;
+  bc[2] = q % sg.nb[2];
+  q /= sg.nb[2];
+  bc[3] = q % sg.nb[3];
+  bc[0] = q / sg.nb[3];
+  bc[1] = 2 * j + ((colour + bc[0] + bc[3] + bc[2]) & 1);
+}
+// its number within its colour
+__device__ __forceinline__ int block_number(const SapGeom& sg, const int bc[4]) {
+  return ((bc[0] * sg.nb[3] + bc[3]) * sg.nb[2] + bc[2]) * (sg.nb[1] >> 1) + (bc[1] >> 1);
+}
 
 template <typename R>
 __device__ inline Spinor<R> smem_load(const Cplx<R>* r_s, int vb, int l) {
@@ -213,6 +230,255 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sap_sweep(const char* __restrict
   }
   F::store_spinor(rho, g.V, s, r);
   F::store_spinor(delta, g.V, s, x);
+}
+
+// ---------------------------------------------------------------------------
+// FP64, 4^4 blocks.  The FP64 pipe is the bound (a warp instruction takes the SM 16
+// cycles, with however few lanes active), so no warp runs with idle lanes: hops are
+// tasks, numbered over the sites that have a neighbour in the block (3/4 of them
+// in every direction) or over the sites of a face (boundary term), and their
+// results are added to the site's sum in shared memory, one direction and sign
+// per round.  Per MR step and block 48 hops of a warp instead of 60 with one
+// thread per site, in the boundary term 16 instead of 64.
+//
+// C = 2 spreads a block over a cluster of two CTAs (time-slices 0-1 and 2-3) that
+// read each other's residual through distributed shared memory: with few blocks
+// the units of work are coarse (8^3x16 with 12 RHS: 192 on 152 SMs).
+// ---------------------------------------------------------------------------
+using CD = Cplx<double>;
+
+__device__ __forceinline__ Spinor<double> sm_ld(const CD* b, int n, int l) {
+  Spinor<double> o;
+#pragma unroll
+  for (int k = 0; k < 12; k++) {
+    const double2 v = *(const double2*)(b + k * n + l);
+    o.c[k] = cmk(v.x, v.y);
+  }
+  return o;
+}
+__device__ __forceinline__ void sm_st(CD* b, int n, int l, const Spinor<double>& v) {
+#pragma unroll
+  for (int k = 0; k < 12; k++) *(double2*)(b + k * n + l) = make_double2(v.c[k].re, v.c[k].im);
+}
+
+// o += scale * hop of r over link MU at site sl
+template <int MU, bool FWD>
+__device__ __forceinline__ void hop_d(Spinor<double>& o, const Spinor<double>& r, const void* gauge, int V, int sl,
+                                      double scale) {
+  HalfSpinor<double> h = project<MU, FWD ? -1 : +1>(r);
+  if (FWD) h = su3_mul(FieldsD::load_link(gauge, V, MU, sl), h);
+  else h = su3_dag_mul(FieldsD::load_link(gauge, V, MU, sl), h);
+  accum_recon<MU, FWD ? -1 : +1>(o, h, scale);
+}
+
+template <int C>
+struct BlockD {   // what the tasks need to know about the CTA's part of a block
+  static constexpr int N = 256 / C, NT = 4 / C;   // sites, time-slices
+  CD *r_s, *p_s;          // [12][N] residual and operator sum
+  const CD* other;        // the other CTA's r_s (C = 2)
+  const void* gauge;
+  int co[4], t0, rank;    // first site of the block, first local time-slice
+};
+template <int C>
+__device__ __forceinline__ int site_of(const BlockD<C>& B, const Geom& g, int t, int x, int y, int z) {
+  return (((B.co[0] + t) * g.L[3] + B.co[3] + z) * g.L[2] + B.co[2] + y) * g.L[1] + B.co[1] + x;
+}
+
+// one round of the block operator: p_s += scale * (hops in direction MU, one sign)
+template <int C, int MU, bool FWD>
+__device__ __forceinline__ void hop_round(const BlockD<C>& B, const Geom& g, int i, double scale) {
+  constexpr int N = BlockD<C>::N, NT = BlockD<C>::NT;
+  // sites with a neighbour: x, y, z: three of four coordinates; t: those whose
+  // neighbour is in the block (for C = 2 also in the other CTA)
+  int x, y, z, t;   // t local to the CTA
+  if (MU == 0) {
+    const bool edge = C == 1 || (FWD ? B.rank == C - 1 : B.rank == 0);   // the block ends on this side
+    if (i >= 64 * (edge ? NT - 1 : NT)) return;
+    x = i & 3; y = (i >> 2) & 3; z = (i >> 4) & 3; t = (i >> 6) + (!FWD && edge ? 1 : 0);
+  } else {
+    if (i >= N / 4 * 3) return;
+    const int d = i / (N / 4), e = i % (N / 4), v = d + (FWD ? 0 : 1);   // the coordinate in MU, the others
+    const int a = e & 3, b = (e >> 2) & 3;
+    t = e >> 4;
+    x = MU == 1 ? v : a;
+    y = MU == 2 ? v : MU == 1 ? a : b;
+    z = MU == 3 ? v : b;
+  }
+  const int l = ((t * 4 + z) * 4 + y) * 4 + x;
+  constexpr int st = MU == 0 ? 64 : MU == 1 ? 1 : MU == 2 ? 4 : 16;
+  int ln = l + (FWD ? st : -st);
+  const CD* rb = B.r_s;
+  if (MU == 0 && C > 1 && (ln < 0 || ln >= N)) {
+    rb = B.other;
+    ln += ln < 0 ? N : -N;
+  }
+  const int s = site_of(B, g, B.t0 + t, x, y, z);
+  Spinor<double> p = sm_ld(B.p_s, N, l);
+  hop_d<MU, FWD>(p, sm_ld(rb, N, ln), B.gauge, g.V, FWD ? s : s - g.stride[MU], scale);
+  sm_st(B.p_s, N, l, p);
+}
+
+// boundary term of one direction: the hops from delta across the two MU faces
+template <int C, int MU>
+__device__ __forceinline__ void gather_round(const BlockD<C>& B, const Geom& g, const char* delta, int i,
+                                             double kappa) {
+  constexpr int N = BlockD<C>::N, NT = BlockD<C>::NT;
+  constexpr int nf = MU == 0 ? 64 : N / 4;   // sites of one face in this CTA
+  if (i >= 2 * nf) return;
+  const bool fwd = i >= nf;
+  const int e = fwd ? i - nf : i, a = e & 3, b = (e >> 2) & 3, d = e >> 4;
+  int t, x, y, z;
+  if (MU == 0) {
+    if (C > 1 && (fwd ? B.rank != C - 1 : B.rank != 0)) return;
+    x = a; y = b; z = d; t = fwd ? NT - 1 : 0;
+  } else {
+    const int v = fwd ? 3 : 0;
+    t = d;
+    x = MU == 1 ? v : a;
+    y = MU == 2 ? v : MU == 1 ? a : b;
+    z = MU == 3 ? v : b;
+  }
+  const int l = ((t * 4 + z) * 4 + y) * 4 + x, s = site_of(B, g, B.t0 + t, x, y, z);
+  const int c[4] = {B.co[0] + B.t0 + t, B.co[1] + x, B.co[2] + y, B.co[3] + z};
+  Spinor<double> r = sm_ld(B.r_s, N, l);
+  if (fwd) {
+    const double sc = (MU == 0 && c[0] == g.L[0] - 1) ? g.bc_t * kappa : kappa;
+    hop_d<MU, true>(r, FieldsD::load_spinor(delta, g.V, site_fwd(g, s, c, MU)), B.gauge, g.V, s, sc);
+  } else {
+    const int sb = site_bwd(g, s, c, MU);
+    const double sc = (MU == 0 && c[0] == 0) ? g.bc_t * kappa : kappa;
+    hop_d<MU, false>(r, FieldsD::load_spinor(delta, g.V, sb), B.gauge, g.V, sb, sc);
+  }
+  sm_st(B.r_s, N, l, r);
+}
+
+template <int C>
+__device__ __forceinline__ void sync_block() {
+  if (C == 1) __syncthreads();
+  else cooperative_groups::this_cluster().sync();
+}
+
+template <int C>
+__global__ void __launch_bounds__(256 / C, C)
+    k_sap_sweep_d4(const char* __restrict__ rho_src, char* __restrict__ rho, char* __restrict__ psi,
+                   char* __restrict__ delta, const void* __restrict__ gauge, const void* __restrict__ clover, Geom g,
+                   SapGeom sg, int colour, int gather, int psi_init, int last, double kappa, int nmr, int nrhs,
+                   const int* mask) {
+  constexpr int N = 256 / C, NW = N / 32;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double red[2][3][NW];
+  const int unit = blockIdx.x / C;
+  const int rhs = unit % nrhs;   // RHS fastest, as in k_sap_sweep
+  const int blk = unit / nrhs;
+  if (mask && !mask[rhs]) return;   // all CTAs of a cluster
+  const size_t off = (size_t)rhs * FieldsD::spinor_bytes * g.V;
+  rho_src += off;
+  rho += off;
+  psi += off;
+  delta += off;
+  int bc[4];
+  block_of(sg, colour, blk, bc);
+  BlockD<C> B;
+  B.r_s = (CD*)smem_raw;
+  B.p_s = B.r_s + 12 * N;
+  B.gauge = gauge;
+  B.rank = C == 1 ? 0 : (int)(blockIdx.x % C);
+  B.other = B.r_s;
+  if constexpr (C > 1) B.other = cooperative_groups::this_cluster().map_shared_rank(B.r_s, 1 - B.rank);
+#pragma unroll
+  for (int mu = 0; mu < 4; mu++) B.co[mu] = 4 * bc[mu];
+  B.t0 = B.rank * (4 / C);
+  const int l = threadIdx.x;
+  const int s = site_of(B, g, B.t0 + (l >> 6), l & 3, (l >> 2) & 3, (l >> 4) & 3);
+
+  Spinor<double> r = FieldsD::load_spinor(rho_src, g.V, s);
+  sm_st(B.r_s, N, l, r);
+  if (gather) {
+    __syncthreads();
+    gather_round<C, 0>(B, g, delta, l, kappa);
+    __syncthreads();
+    gather_round<C, 1>(B, g, delta, l, kappa);
+    __syncthreads();
+    gather_round<C, 2>(B, g, delta, l, kappa);
+    __syncthreads();
+    gather_round<C, 3>(B, g, delta, l, kappa);
+    __syncthreads();
+    r = sm_ld(B.r_s, N, l);
+  }
+  Spinor<double> x;
+#pragma unroll
+  for (int k = 0; k < 12; k++) x.c[k] = cmk(0.0, 0.0);
+  const int warp = l >> 5, lane = l & 31;
+  for (int step = 0; step < nmr; step++) {
+    sm_st(B.p_s, N, l, clover_apply<FieldsD>(clover, g.V, s, r));
+    sync_block<C>();   // the residual and the sums of all CTAs are in place
+    hop_round<C, 0, true>(B, g, l, -kappa);
+    __syncthreads();
+    hop_round<C, 0, false>(B, g, l, -kappa);
+    __syncthreads();
+    hop_round<C, 1, true>(B, g, l, -kappa);
+    __syncthreads();
+    hop_round<C, 1, false>(B, g, l, -kappa);
+    __syncthreads();
+    hop_round<C, 2, true>(B, g, l, -kappa);
+    __syncthreads();
+    hop_round<C, 2, false>(B, g, l, -kappa);
+    __syncthreads();
+    hop_round<C, 3, true>(B, g, l, -kappa);
+    __syncthreads();
+    hop_round<C, 3, false>(B, g, l, -kappa);
+    __syncthreads();
+    const Spinor<double> p = sm_ld(B.p_s, N, l);
+    CD pr = cmk(0.0, 0.0);
+    double pp = 0;
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+      cmac_conj(pr, p.c[k], r.c[k]);
+      pp = fma(p.c[k].re, p.c[k].re, pp);
+      pp = fma(p.c[k].im, p.c[k].im, pp);
+    }
+    pr.re = warp_sum(pr.re);
+    pr.im = warp_sum(pr.im);
+    pp = warp_sum(pp);
+    // two buffers: the other CTA may still read the last step's sums
+    double(*rd)[NW] = red[step & 1];
+    if (lane == 0) {
+      rd[0][warp] = pr.re;
+      rd[1][warp] = pr.im;
+      rd[2][warp] = pp;
+    }
+    sync_block<C>();   // also: every CTA has read its neighbour's residual
+    double a[3] = {0, 0, 0};
+#pragma unroll
+    for (int q = 0; q < C; q++) {   // CTA 0's sums first, for every CTA
+      const double* src = &rd[0][0];
+      if constexpr (C > 1) src = cooperative_groups::this_cluster().map_shared_rank(&rd[0][0], q);
+#pragma unroll
+      for (int k = 0; k < 3; k++)
+#pragma unroll
+        for (int w = 0; w < NW; w++) a[k] += src[k * NW + w];
+    }
+    const CD alpha = a[2] > 0 ? cmk(a[0] / a[2], a[1] / a[2]) : cmk(0.0, 0.0);
+    const CD malpha = -alpha;
+#pragma unroll
+    for (int k = 0; k < 12; k++) {
+      cmac(x.c[k], alpha, r.c[k]);
+      cmac(r.c[k], malpha, p.c[k]);
+    }
+    sm_st(B.r_s, N, l, r);
+  }
+  if (psi_init) {
+    FieldsD::store_spinor(psi, g.V, s, x);
+  } else {
+    Spinor<double> y = FieldsD::load_spinor(psi, g.V, s);
+#pragma unroll
+    for (int k = 0; k < 12; k++) y.c[k] = y.c[k] + x.c[k];
+    FieldsD::store_spinor(psi, g.V, s, y);
+  }
+  // the last cycle's residuals and the last half-cycle's delta have no reader
+  if (last < 1) FieldsD::store_spinor(rho, g.V, s, r);
+  if (last < 2) FieldsD::store_spinor(delta, g.V, s, x);
+  if constexpr (C > 1) sync_block<C>();   // the other CTA's last reads of this shared memory
 }
 
 // ---------------------------------------------------------------------------
@@ -504,22 +770,6 @@ __device__ inline void smem_gather_dir(void* r_s, const SapGeom& sg, const Geom&
     delta_hop<MU, +1, true>(r, delta, gauge, g.V, sb, sb, (MU == 0 && c[0] == 0) ? (float)g.bc_t * kappa : kappa);
   }
   rs_store<false>(r_s, sg.vb, ls, r);
-}
-
-// the blk-th block of a colour
-__device__ __forceinline__ void block_of(const SapGeom& sg, int colour, int blk, int bc[4]) {
-  const int nbx2 = sg.nb[1] >> 1;
-  int q = blk / nbx2;
-  const int j = blk - q * nbx2;
-  bc[2] = q % sg.nb[2];
-  q /= sg.nb[2];
-  bc[3] = q % sg.nb[3];
-  bc[0] = q / sg.nb[3];
-  bc[1] = 2 * j + ((colour + bc[0] + bc[3] + bc[2]) & 1);
-}
-// its number within its colour
-__device__ __forceinline__ int block_number(const SapGeom& sg, const int bc[4]) {
-  return ((bc[0] * sg.nb[3] + bc[3]) * sg.nb[2] + bc[2]) * (sg.nb[1] >> 1) + (bc[1] >> 1);
 }
 
 // Any block shape: rho, psi and delta in the lexicographic layout.  img: the
@@ -1069,6 +1319,13 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
                        : cudaFuncSetAttribute(kernF, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   else
     QCD_CUDA_OK(cudaFuncSetAttribute(kernD, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // FP64 4^4 blocks: two CTAs per block while there are fewer than 8 blocks per SM
+  // (a coarse last wave otherwise); beyond that one CTA, without cluster barriers
+  const int split = (long long)(nblocks / 2) * nrhs < 8 * 152 ? 2 : 1;
+  const size_t smem_d4 = (size_t)2 * 12 * (256 / split) * sizeof(double2);
+  if (!f32 && b4)
+    QCD_CUDA_OK(split == 2 ? cudaFuncSetAttribute(k_sap_sweep_d4<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_d4)
+                           : cudaFuncSetAttribute(k_sap_sweep_d4<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_d4));
   auto issue = [&]() -> qcd_status {
     for (int cy = 0; cy < P.ncy; cy++)
       for (int col = 0; col < 2; col++) {
@@ -1092,7 +1349,21 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
                                                     nrhs, mask);
           }
         }
-        else
+        else if (b4) {
+          cudaLaunchConfig_t cfg = {};
+          cfg.gridDim = dim3(grid.x * split);
+          cfg.blockDim = dim3(256 / split);
+          cfg.dynamicSmemBytes = smem_d4;
+          cfg.stream = c->stream;
+          cudaLaunchAttribute at[1];
+          at[0].id = cudaLaunchAttributeClusterDimension;
+          at[0].val.clusterDim.x = split;
+          at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+          cfg.attrs = at;
+          cfg.numAttrs = 1;
+          QCD_CUDA_OK(cudaLaunchKernelEx(&cfg, split == 2 ? k_sap_sweep_d4<2> : k_sap_sweep_d4<1>, rin, rho, psi, delta,
+                                         gauge, clover, c->g, sg, col, gather, first, last, c->kappa, P.nmr, nrhs, mask));
+        } else
           kernD<<<grid, sg.vb, smem, c->stream>>>(rin, rho, psi, delta, gauge, clover, c->g, sg, col, gather, first,
                                                   c->kappa, P.nmr, nrhs, mask);
         QCD_CUDA_OK(cudaGetLastError());
