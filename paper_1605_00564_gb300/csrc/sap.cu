@@ -241,9 +241,12 @@ __global__ void __launch_bounds__(MAXT, MINB) k_sap_sweep(const char* __restrict
 // per round.  Per MR step and block 48 hops of a warp instead of 60 with one
 // thread per site, in the boundary term 16 instead of 64.
 //
-// C = 2 spreads a block over a cluster of two CTAs (time-slices 0-1 and 2-3) that
-// read each other's residual through distributed shared memory: with few blocks
-// the units of work are coarse (8^3x16 with 12 RHS: 192 on 152 SMs).
+// A block is spread over a cluster of two CTAs (time-slices 0-1 and 2-3) that read
+// each other's residual through distributed shared memory: the units of work are
+// coarse (8^3x16 with 12 RHS: 192 on 152 SMs).  Per half-cycle, one thread per site on
+// one CTA -> tasks on one CTA -> tasks on two: 8^3x16, 12 RHS 770 -> 669 -> 531 us, one
+// RHS 388 -> 337 -> 215; 16^3x32, 12 RHS 8.11 -> 7.12 -> 6.65 ms.  (Four CTAs of one
+// time-slice leave half-empty warps again: 598 us and 7.96 ms.)
 // ---------------------------------------------------------------------------
 using CD = Cplx<double>;
 
@@ -271,28 +274,26 @@ __device__ __forceinline__ void hop_d(Spinor<double>& o, const Spinor<double>& r
   accum_recon<MU, FWD ? -1 : +1>(o, h, scale);
 }
 
-template <int C>
-struct BlockD {   // what the tasks need to know about the CTA's part of a block
-  static constexpr int N = 256 / C, NT = 4 / C;   // sites, time-slices
+struct BlockD {   // what the tasks need to know about the CTA's half of a block
+  static constexpr int N = 128, NT = 2;   // sites, time-slices
   CD *r_s, *p_s;          // [12][N] residual and operator sum
-  const CD* other;        // the other CTA's r_s (C = 2)
+  const CD* other;        // the other CTA's r_s
   const void* gauge;
   int co[4], t0, rank;    // first site of the block, first local time-slice
 };
-template <int C>
-__device__ __forceinline__ int site_of(const BlockD<C>& B, const Geom& g, int t, int x, int y, int z) {
+__device__ __forceinline__ int site_of(const BlockD& B, const Geom& g, int t, int x, int y, int z) {
   return (((B.co[0] + t) * g.L[3] + B.co[3] + z) * g.L[2] + B.co[2] + y) * g.L[1] + B.co[1] + x;
 }
 
 // one round of the block operator: p_s += scale * (hops in direction MU, one sign)
-template <int C, int MU, bool FWD>
-__device__ __forceinline__ void hop_round(const BlockD<C>& B, const Geom& g, int i, double scale) {
-  constexpr int N = BlockD<C>::N, NT = BlockD<C>::NT;
+template <int MU, bool FWD>
+__device__ __forceinline__ void hop_round(const BlockD& B, const Geom& g, int i, double scale) {
+  constexpr int N = BlockD::N, NT = BlockD::NT;
   // sites with a neighbour: x, y, z: three of four coordinates; t: those whose
-  // neighbour is in the block (for C = 2 also in the other CTA)
+  // neighbour is in the block (here or in the other CTA)
   int x, y, z, t;   // t local to the CTA
   if (MU == 0) {
-    const bool edge = C == 1 || (FWD ? B.rank == C - 1 : B.rank == 0);   // the block ends on this side
+    const bool edge = FWD ? B.rank == 1 : B.rank == 0;   // the block ends on this side
     if (i >= 64 * (edge ? NT - 1 : NT)) return;
     x = i & 3; y = (i >> 2) & 3; z = (i >> 4) & 3; t = (i >> 6) + (!FWD && edge ? 1 : 0);
   } else {
@@ -308,7 +309,7 @@ __device__ __forceinline__ void hop_round(const BlockD<C>& B, const Geom& g, int
   constexpr int st = MU == 0 ? 64 : MU == 1 ? 1 : MU == 2 ? 4 : 16;
   int ln = l + (FWD ? st : -st);
   const CD* rb = B.r_s;
-  if (MU == 0 && C > 1 && (ln < 0 || ln >= N)) {
+  if (MU == 0 && (ln < 0 || ln >= N)) {
     rb = B.other;
     ln += ln < 0 ? N : -N;
   }
@@ -319,17 +320,17 @@ __device__ __forceinline__ void hop_round(const BlockD<C>& B, const Geom& g, int
 }
 
 // boundary term of one direction: the hops from delta across the two MU faces
-template <int C, int MU>
-__device__ __forceinline__ void gather_round(const BlockD<C>& B, const Geom& g, const char* delta, int i,
+template <int MU>
+__device__ __forceinline__ void gather_round(const BlockD& B, const Geom& g, const char* delta, int i,
                                              double kappa) {
-  constexpr int N = BlockD<C>::N, NT = BlockD<C>::NT;
+  constexpr int N = BlockD::N, NT = BlockD::NT;
   constexpr int nf = MU == 0 ? 64 : N / 4;   // sites of one face in this CTA
   if (i >= 2 * nf) return;
   const bool fwd = i >= nf;
   const int e = fwd ? i - nf : i, a = e & 3, b = (e >> 2) & 3, d = e >> 4;
   int t, x, y, z;
   if (MU == 0) {
-    if (C > 1 && (fwd ? B.rank != C - 1 : B.rank != 0)) return;
+    if (fwd ? B.rank != 1 : B.rank != 0) return;
     x = a; y = b; z = d; t = fwd ? NT - 1 : 0;
   } else {
     const int v = fwd ? 3 : 0;
@@ -352,25 +353,21 @@ __device__ __forceinline__ void gather_round(const BlockD<C>& B, const Geom& g, 
   sm_st(B.r_s, N, l, r);
 }
 
-template <int C>
-__device__ __forceinline__ void sync_block() {
-  if (C == 1) __syncthreads();
-  else cooperative_groups::this_cluster().sync();
-}
+// both CTAs of the block
+__device__ __forceinline__ void sync_block() { cooperative_groups::this_cluster().sync(); }
 
-template <int C>
-__global__ void __launch_bounds__(256 / C, C)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, 2)
     k_sap_sweep_d4(const char* __restrict__ rho_src, char* __restrict__ rho, char* __restrict__ psi,
                    char* __restrict__ delta, const void* __restrict__ gauge, const void* __restrict__ clover, Geom g,
                    SapGeom sg, int colour, int gather, int psi_init, int last, double kappa, int nmr, int nrhs,
                    const int* mask) {
-  constexpr int N = 256 / C, NW = N / 32;
+  constexpr int N = BlockD::N, NW = N / 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double red[2][3][NW];
-  const int unit = blockIdx.x / C;
+  const int unit = blockIdx.x / 2;
   const int rhs = unit % nrhs;   // RHS fastest, as in k_sap_sweep
   const int blk = unit / nrhs;
-  if (mask && !mask[rhs]) return;   // all CTAs of a cluster
+  if (mask && !mask[rhs]) return;   // both CTAs of a cluster
   const size_t off = (size_t)rhs * FieldsD::spinor_bytes * g.V;
   rho_src += off;
   rho += off;
@@ -378,16 +375,15 @@ __global__ void __launch_bounds__(256 / C, C)
   delta += off;
   int bc[4];
   block_of(sg, colour, blk, bc);
-  BlockD<C> B;
+  BlockD B;
   B.r_s = (CD*)smem_raw;
   B.p_s = B.r_s + 12 * N;
   B.gauge = gauge;
-  B.rank = C == 1 ? 0 : (int)(blockIdx.x % C);
-  B.other = B.r_s;
-  if constexpr (C > 1) B.other = cooperative_groups::this_cluster().map_shared_rank(B.r_s, 1 - B.rank);
+  B.rank = blockIdx.x % 2;
+  B.other = cooperative_groups::this_cluster().map_shared_rank(B.r_s, 1 - B.rank);
 #pragma unroll
   for (int mu = 0; mu < 4; mu++) B.co[mu] = 4 * bc[mu];
-  B.t0 = B.rank * (4 / C);
+  B.t0 = 2 * B.rank;
   const int l = threadIdx.x;
   const int s = site_of(B, g, B.t0 + (l >> 6), l & 3, (l >> 2) & 3, (l >> 4) & 3);
 
@@ -395,13 +391,13 @@ __global__ void __launch_bounds__(256 / C, C)
   sm_st(B.r_s, N, l, r);
   if (gather) {
     __syncthreads();
-    gather_round<C, 0>(B, g, delta, l, kappa);
+    gather_round<0>(B, g, delta, l, kappa);
     __syncthreads();
-    gather_round<C, 1>(B, g, delta, l, kappa);
+    gather_round<1>(B, g, delta, l, kappa);
     __syncthreads();
-    gather_round<C, 2>(B, g, delta, l, kappa);
+    gather_round<2>(B, g, delta, l, kappa);
     __syncthreads();
-    gather_round<C, 3>(B, g, delta, l, kappa);
+    gather_round<3>(B, g, delta, l, kappa);
     __syncthreads();
     r = sm_ld(B.r_s, N, l);
   }
@@ -411,22 +407,22 @@ __global__ void __launch_bounds__(256 / C, C)
   const int warp = l >> 5, lane = l & 31;
   for (int step = 0; step < nmr; step++) {
     sm_st(B.p_s, N, l, clover_apply<FieldsD>(clover, g.V, s, r));
-    sync_block<C>();   // the residual and the sums of all CTAs are in place
-    hop_round<C, 0, true>(B, g, l, -kappa);
+    sync_block();   // the residual of both CTAs and the sums are in place
+    hop_round<0, true>(B, g, l, -kappa);
     __syncthreads();
-    hop_round<C, 0, false>(B, g, l, -kappa);
+    hop_round<0, false>(B, g, l, -kappa);
     __syncthreads();
-    hop_round<C, 1, true>(B, g, l, -kappa);
+    hop_round<1, true>(B, g, l, -kappa);
     __syncthreads();
-    hop_round<C, 1, false>(B, g, l, -kappa);
+    hop_round<1, false>(B, g, l, -kappa);
     __syncthreads();
-    hop_round<C, 2, true>(B, g, l, -kappa);
+    hop_round<2, true>(B, g, l, -kappa);
     __syncthreads();
-    hop_round<C, 2, false>(B, g, l, -kappa);
+    hop_round<2, false>(B, g, l, -kappa);
     __syncthreads();
-    hop_round<C, 3, true>(B, g, l, -kappa);
+    hop_round<3, true>(B, g, l, -kappa);
     __syncthreads();
-    hop_round<C, 3, false>(B, g, l, -kappa);
+    hop_round<3, false>(B, g, l, -kappa);
     __syncthreads();
     const Spinor<double> p = sm_ld(B.p_s, N, l);
     CD pr = cmk(0.0, 0.0);
@@ -447,12 +443,11 @@ __global__ void __launch_bounds__(256 / C, C)
       rd[1][warp] = pr.im;
       rd[2][warp] = pp;
     }
-    sync_block<C>();   // also: every CTA has read its neighbour's residual
+    sync_block();   // also: both CTAs have read the other's residual
     double a[3] = {0, 0, 0};
 #pragma unroll
-    for (int q = 0; q < C; q++) {   // CTA 0's sums first, for every CTA
-      const double* src = &rd[0][0];
-      if constexpr (C > 1) src = cooperative_groups::this_cluster().map_shared_rank(&rd[0][0], q);
+    for (int q = 0; q < 2; q++) {   // CTA 0's sums first, for both
+      const double* src = cooperative_groups::this_cluster().map_shared_rank(&rd[0][0], q);
 #pragma unroll
       for (int k = 0; k < 3; k++)
 #pragma unroll
@@ -478,7 +473,7 @@ __global__ void __launch_bounds__(256 / C, C)
   // the last cycle's residuals and the last half-cycle's delta have no reader
   if (last < 1) FieldsD::store_spinor(rho, g.V, s, r);
   if (last < 2) FieldsD::store_spinor(delta, g.V, s, x);
-  if constexpr (C > 1) sync_block<C>();   // the other CTA's last reads of this shared memory
+  sync_block();   // the other CTA's last reads of this shared memory
 }
 
 // ---------------------------------------------------------------------------
@@ -1319,13 +1314,9 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
                        : cudaFuncSetAttribute(kernF, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   else
     QCD_CUDA_OK(cudaFuncSetAttribute(kernD, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  // FP64 4^4 blocks: two CTAs per block while there are fewer than 8 blocks per SM
-  // (a coarse last wave otherwise); beyond that one CTA, without cluster barriers
-  const int split = (long long)(nblocks / 2) * nrhs < 8 * 152 ? 2 : 1;
-  const size_t smem_d4 = (size_t)2 * 12 * (256 / split) * sizeof(double2);
+  const size_t smem_d4 = (size_t)2 * 12 * BlockD::N * sizeof(double2);
   if (!f32 && b4)
-    QCD_CUDA_OK(split == 2 ? cudaFuncSetAttribute(k_sap_sweep_d4<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_d4)
-                           : cudaFuncSetAttribute(k_sap_sweep_d4<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_d4));
+    QCD_CUDA_OK(cudaFuncSetAttribute(k_sap_sweep_d4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_d4));
   auto issue = [&]() -> qcd_status {
     for (int cy = 0; cy < P.ncy; cy++)
       for (int col = 0; col < 2; col++) {
@@ -1350,19 +1341,9 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
           }
         }
         else if (b4) {
-          cudaLaunchConfig_t cfg = {};
-          cfg.gridDim = dim3(grid.x * split);
-          cfg.blockDim = dim3(256 / split);
-          cfg.dynamicSmemBytes = smem_d4;
-          cfg.stream = c->stream;
-          cudaLaunchAttribute at[1];
-          at[0].id = cudaLaunchAttributeClusterDimension;
-          at[0].val.clusterDim.x = split;
-          at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-          cfg.attrs = at;
-          cfg.numAttrs = 1;
-          QCD_CUDA_OK(cudaLaunchKernelEx(&cfg, split == 2 ? k_sap_sweep_d4<2> : k_sap_sweep_d4<1>, rin, rho, psi, delta,
-                                         gauge, clover, c->g, sg, col, gather, first, last, c->kappa, P.nmr, nrhs, mask));
+          k_sap_sweep_d4<<<2 * grid.x, BlockD::N, smem_d4, c->stream>>>(rin, rho, psi, delta, gauge, clover, c->g, sg,
+                                                                        col, gather, first, last, c->kappa, P.nmr,
+                                                                        nrhs, mask);
         } else
           kernD<<<grid, sg.vb, smem, c->stream>>>(rin, rho, psi, delta, gauge, clover, c->g, sg, col, gather, first,
                                                   c->kappa, P.nmr, nrhs, mask);

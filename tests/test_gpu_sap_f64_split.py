@@ -1,7 +1,6 @@
-"""The FP64 4^4 sweep with a block on one CTA and on a cluster of two: the sums
-run over the same groups of sites in the same order, so a right-hand side gives
-the same bits either way (few right-hand sides: two CTAs per block, 24 on 8 x 16^3:
-one)."""
+"""The FP64 4^4 sweep (a block on a cluster of two CTAs): sums run over fixed groups of
+sites in a fixed order, so a right-hand side gives the same bits alone and in a
+batch of 24, for one and several cycles and MR steps."""
 import numpy as np
 import pytest
 
@@ -12,7 +11,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("ncy,nmr", [(1, 1), (2, 4), (3, 3)])
-def test_sap_f64_one_and_two_ctas(ncy, nmr):
+def test_sap_f64_batched_equals_single(ncy, nmr):
     lat, _, _ = make_lattice((8, 16, 16, 16), eps=0.3, csw=1.2, kappa=0.126, seed=80)
     lat.set_params(block=(4, 4, 4, 4), ncy=ncy, nmr=nmr, precision="f64")
     eta = synth.random_spinor(lat.dims, 31, nrhs=24)
