@@ -450,12 +450,13 @@ struct qcd_ctx {
   // fields
   DevBuf gaugeD, gaugeF, cloverD, cloverF;
   // SAP block images of the links and clover term (sap.cu), 16-bit and FP32,
-  // and the FP32 links across the faces of 4^4 blocks; rebuilt when gauge_id
+  // and the FP32 links across the faces of 4 or 8 x 4^3 blocks; rebuilt when gauge_id
   // (counted up by every qcd_load_gauge) or the block shape differs
   uint64_t gauge_id = 0, flinks_id = 0;
   SapImage sap_img16, sap_img32;
   DevBuf flinks;
-  DevBuf sap_vec;     // block-ordered working vectors of the 4^4 sweep
+  int flinks_nt = 0;   // time extent of the blocks they were built for
+  DevBuf sap_vec;     // block-ordered working vectors of the same blocks' sweep
   // workspaces (grown on demand, kept until destroy)
   DevBuf wsD[8];      // FP64 spinors (nrhs each)
   DevBuf wsF[8];      // FP32 spinors

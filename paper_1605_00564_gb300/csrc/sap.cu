@@ -497,7 +497,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, 2)
 //              block takes 172 KB and an SM holds one CTA, whose loads and
 //              barriers nothing hides;
 //   FromImage  the FP32 image read from L2 at every step (blocks of more than 256
-//              sites, whose copies exceed shared memory);
+//              sites, whose copies exceed shared memory; 8 x 4^3 blocks have the
+//              sweep of their own below);
 //   FromField  the same from the lexicographic fields, where there is no memory
 //              for an image.
 // Either staged form leaves room for two CTAs of a 4^4 block per SM.
@@ -673,6 +674,7 @@ __device__ __forceinline__ void mr_steps(PairSpinor& r, PairSpinor& x, void* r_s
     if (lane == 0) red[warp] = make_float4(pr_re, pr_im, pp, 0.f);
     __syncthreads();
     float a_re = 0, a_im = 0, n2 = 0;
+#pragma unroll 8   // (all 16 sums of a 512-site block at once would spill)
     for (int w = 0; w < nw; w++) {
       const float4 v = red[w];
       a_re += v.x;
@@ -877,20 +879,21 @@ __global__ void __launch_bounds__(MAXT, MINB)
   if (last < 2) pair_store(delta, g.V, s, x);
 }
 
-// 4^4 blocks.  Between the first and the last cycle everything a CTA reads and
-// writes is a contiguous run of its block:
-//   rho_b, psi_b  [rhs][block][record q][256] float4, the residual and the sum
+// Blocks of T x 4^3 sites, T = 4 or 8 in time.  Between the first and the last
+// cycle everything a CTA reads and writes is a contiguous run of its block:
+//   rho_b, psi_b  [rhs][block][record q][64 T] float4, the residual and the sum
 //                 of the increments (the first cycle reads the caller's
 //                 lexicographic residual, the last one writes its psi);
 //   faces         what the neighbours of the other colour need of delta: per
 //                 block of a colour, face f = 2 mu + side (side 0: the sites at
-//                 -mu, 1: at +mu) and colour a the half spinors of the 64 face
-//                 sites, [rhs][colour][block][8][3][64] float4, projected with
-//                 1 - gamma_mu (side 0, for the block at -mu) or 1 + gamma_mu;
+//                 -mu, 1: at +mu) and colour a the half spinors of the face
+//                 sites (64 in time, 16 T in space), [rhs][colour][block][face]
+//                 [3][site] float4, projected with 1 - gamma_mu (side 0, for the
+//                 block at -mu) or 1 + gamma_mu;
 //   flinks        the FP32 links across a block's own faces in the same order,
-//                 [block][8][link row word 3][64] float4.
-// Boundary term: 8 faces x 64 sites are 16 tasks of a warp, two per warp (warp
-// w: side (w >> 1) & 1, half w & 1, mu = w >> 2 and 2 + (w >> 2)): read the
+//                 [block][face][link row word 3][site] float4.
+// Boundary term: the face sites are 4 + 6 T / 2 tasks of a warp, at most two per
+// warp (task k of warp k mod 2 T, faces in order): read the
 // neighbour's half spinor and the link, multiply, leave the product in shared
 // memory; after a barrier every site adds those of the faces it lies on, in the
 // order t, x, y, z.  The products take the block residual's place before it is
@@ -902,7 +905,11 @@ __global__ void __launch_bounds__(MAXT, MINB)
 // scalar arithmetic: 32^3x64, 12 RHS, 16-bit copies 44.4 -> 33.7 ms per
 // application (5 cycles); 24^3x48, one RHS, FP32 copies 225 -> 119 us per
 // half-cycle.  (Two-lane arithmetic alone, still loading lexicographic pieces, gave
-// nothing: the loads were the bound.)
+// nothing: the loads were the bound.)  T = 8, one CTA of 512 threads per SM, against
+// the general sweep on FromImage: 24^3x48, 12 RHS 2050 -> 1375 us per half-cycle;
+// 48x24x8x16, 5 RHS 191 -> 141, one RHS 37 -> 30 (the 4^4 block: 1180, 123, 29).  A
+// block on a cluster of two CTAs, hops across the middle from the other's shared
+// memory: 1453, 155 and 35.
 struct SapB4 {
   const char* rho_src;
   float4 *rho_b, *psi_b, *faces;
@@ -916,15 +923,25 @@ template <int MU>
 __device__ __forceinline__ int face_site_of(int l) {   // index of site l on a mu face (the other three coordinates)
   return MU == 0 ? (l & 63) : MU == 1 ? (l >> 2) : MU == 2 ? ((l & 3) | ((l >> 4) << 2)) : ((l & 15) | ((l >> 6) << 4));
 }
-template <int MU>
+// sites of a mu face and the first site of face f = 2 mu + side in the order of
+// the faces; 128 + 96 T in all (at most 2 per site of the block)
+template <int NT>
+__host__ __device__ constexpr int face_sites(int mu) { return mu == 0 ? 64 : 16 * NT; }
+template <int NT>
+__host__ __device__ constexpr int face_first(int f) { return f < 2 ? 64 * f : 128 + (f - 2) * 16 * NT; }
+template <int NT>
+__host__ __device__ constexpr int all_face_sites() { return 128 + 96 * NT; }
+
+template <int NT, int MU>
 __device__ __forceinline__ void face_add(PairSpinor& r, const float4* buf, const Geom& g, int t, const int lc[4], int l,
                                          float kappa) {
   const int tf = face_site_of<MU>(l);
-  if (lc[MU] == 3) {
+  constexpr int n = face_sites<NT>(MU);
+  if (lc[MU] == (MU == 0 ? NT : 4) - 1) {
     const float s = (MU == 0 && t == g.L[0] - 1) ? (float)g.bc_t * kappa : kappa;
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-      const float4 v = buf[(3 * (2 * MU + 1) + a) * 64 + tf];
+      const float4 v = buf[3 * face_first<NT>(2 * MU + 1) + a * n + tf];
       pair_recon<MU, -1>(r, a, p2(v.x, v.y), p2(v.z, v.w), s);
     }
   }
@@ -932,33 +949,34 @@ __device__ __forceinline__ void face_add(PairSpinor& r, const float4* buf, const
     const float s = (MU == 0 && t == 0) ? (float)g.bc_t * kappa : kappa;
 #pragma unroll
     for (int a = 0; a < 3; a++) {
-      const float4 v = buf[(3 * (2 * MU) + a) * 64 + tf];
+      const float4 v = buf[3 * face_first<NT>(2 * MU) + a * n + tf];
       pair_recon<MU, +1>(r, a, p2(v.x, v.y), p2(v.z, v.w), s);
     }
   }
 }
 // the projections of delta = x the neighbours will read
-template <int MU>
+template <int NT, int MU>
 __device__ __forceinline__ void face_store(float4* out, const PairSpinor& x, const int lc[4], int l) {
   const int tf = face_site_of<MU>(l);
+  constexpr int n = face_sites<NT>(MU);
   float2 hr, hi;
   if (lc[MU] == 0) {
 #pragma unroll
     for (int a = 0; a < 3; a++) {
       pair_project<MU, -1>(x.re[0][a], x.im[0][a], x.re[1][a], x.im[1][a], hr, hi);
-      out[(3 * (2 * MU) + a) * 64 + tf] = make_float4(hr.x, hr.y, hi.x, hi.y);
+      out[3 * face_first<NT>(2 * MU) + a * n + tf] = make_float4(hr.x, hr.y, hi.x, hi.y);
     }
   }
-  if (lc[MU] == 3) {
+  if (lc[MU] == (MU == 0 ? NT : 4) - 1) {
 #pragma unroll
     for (int a = 0; a < 3; a++) {
       pair_project<MU, +1>(x.re[0][a], x.im[0][a], x.re[1][a], x.im[1][a], hr, hi);
-      out[(3 * (2 * MU + 1) + a) * 64 + tf] = make_float4(hr.x, hr.y, hi.x, hi.y);
+      out[3 * face_first<NT>(2 * MU + 1) + a * n + tf] = make_float4(hr.x, hr.y, hi.x, hi.y);
     }
   }
 }
-// U h (side 1) or U^+ h (side 0) of a half spinor in three records
-__device__ __forceinline__ void face_mul(const float4 (&h)[3], const float4 (&u)[3], int side, float4* out) {
+// U h (side 1) or U^+ h (side 0) of a half spinor in three records, n apart in out
+__device__ __forceinline__ void face_mul(const float4 (&h)[3], const float4 (&u)[3], int side, float4* out, int n) {
   const LinkRows U = link_rows(u[0], u[1], u[2]);
   auto mul = [&](auto link) {
 #pragma unroll
@@ -972,26 +990,28 @@ __device__ __forceinline__ void face_mul(const float4 (&h)[3], const float4 (&u)
         gi = pfma(pbc(w.x), hi, gi);
         gi = pfma(pbc(w.y), hr, gi);
       }
-      out[a * 64] = make_float4(gr.x, gr.y, gi.x, gi.y);
+      out[a * n] = make_float4(gr.x, gr.y, gi.x, gi.y);
     }
   };
   if (side) mul([&](int a, int b) { return U.m[3 * a + b]; });
   else mul([&](int a, int b) { return p2(U.m[3 * b + a].x, -U.m[3 * b + a].y); });
 }
 
-template <typename S, bool BF>
-__global__ void __launch_bounds__(256, 2)
+template <typename S, bool BF, int NT>
+__global__ void __launch_bounds__(64 * NT, 8 / NT)
     k_sap_sweep_b4(SapB4 A, Geom g, SapGeom sg, float kappa, int nmr, int nrhs, const int* mask) {
-  sg.b[0] = sg.b[1] = sg.b[2] = sg.b[3] = 4;
+  constexpr int VB = 64 * NT, NW = VB / 32, FS = all_face_sites<NT>();
+  sg.b[0] = NT;
+  sg.b[1] = sg.b[2] = sg.b[3] = 4;
   sg.lst[1] = 1;
   sg.lst[2] = 4;
   sg.lst[3] = 16;
   sg.lst[0] = 64;
-  sg.vb = 256;
+  sg.vb = VB;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  void* r_s = smem_raw;                          // 24 KB: boundary products, then the residual
-  unsigned char* lk_s = smem_raw + 96 * 256;
-  __shared__ float4 red[8];
+  void* r_s = smem_raw;                          // boundary products, then the residual
+  unsigned char* lk_s = smem_raw + 96 * VB;
+  __shared__ float4 red[NW];
 
   launch_dependents();
   const int rhs = blockIdx.x % nrhs;   // RHS fastest, as in k_sap_sweep
@@ -1001,21 +1021,21 @@ __global__ void __launch_bounds__(256, 2)
   const size_t bidx = (size_t)A.colour * nhalf + blk;
   const int l = threadIdx.x;
 
-  BlockFields f = {lk_s, lk_s + 144 * 256, nullptr, nullptr};
+  BlockFields f = {lk_s, lk_s + 144 * VB, nullptr, nullptr};
   {
-    const unsigned char* img = A.img + bidx * (size_t)((std::is_same<S, __half>::value ? 288 : 480) * 256);
+    const unsigned char* img = A.img + bidx * (size_t)((std::is_same<S, __half>::value ? 288 : 480) * VB);
 #pragma unroll
     for (int k = 0; k < (std::is_same<S, __half>::value ? 18 : 12); k++)
-      cp_async16(lk_s + 16 * (k * 256 + l), img + 16 * (k * 256 + l));
-    if (!std::is_same<S, __half>::value) f.cl = img + 192 * 256;
+      cp_async16(lk_s + 16 * (k * VB + l), img + 16 * (k * VB + l));
+    if (!std::is_same<S, __half>::value) f.cl = img + 192 * VB;
   }
   int bc[4];
   block_of(sg, A.colour, blk, bc);
   const int lc[4] = {l >> 6, l & 3, (l >> 2) & 3, (l >> 4) & 3};
-  const int t = 4 * bc[0] + lc[0];
+  const int t = NT * bc[0] + lc[0];
   const int s = ((t * g.L[3] + 4 * bc[3] + lc[3]) * g.L[2] + 4 * bc[2] + lc[2]) * g.L[1] + 4 * bc[1] + lc[1];
 
-  const size_t voff = ((size_t)rhs * 2 * nhalf + bidx) * 6 * 256 + l;   // block-ordered vectors
+  const size_t voff = ((size_t)rhs * 2 * nhalf + bidx) * 6 * VB + l;   // block-ordered vectors
   float4* rho_b = A.rho_b + voff;
   float4* psi_b = A.psi_b + voff;
   // above: the mask, the links and the clover term, which no half-cycle writes;
@@ -1023,7 +1043,7 @@ __global__ void __launch_bounds__(256, 2)
   dependency_wait();
   if (!A.first) {
 #pragma unroll
-    for (int q = 0; q < 6; q++) prefetch_l2(psi_b + q * 256);
+    for (int q = 0; q < 6; q++) prefetch_l2(psi_b + q * VB);
   }
 
   float4 rw[6];
@@ -1031,7 +1051,7 @@ __global__ void __launch_bounds__(256, 2)
     load_words(A.rho_src + (size_t)rhs * FieldsF::spinor_bytes * g.V, g.V, s, rw);
   } else {
 #pragma unroll
-    for (int q = 0; q < 6; q++) rw[q] = rho_b[q * 256];
+    for (int q = 0; q < 6; q++) rw[q] = rho_b[q * VB];
   }
   auto residual = [&]() {
     if (A.first) return pair_from_words(rw);
@@ -1046,58 +1066,72 @@ __global__ void __launch_bounds__(256, 2)
   PairSpinor r;
   if (A.gather) {
     float4* buf = (float4*)r_s;
-    const int w = l >> 5, side = (w >> 1) & 1, tf = ((w & 1) << 5) | (l & 31);
+    constexpr int NTASK = FS / 32;
+    // task i of this warp: its face 2 mu + side and its 32 sites of it, from tf on
+    auto task = [&](int i, int& mu, int& side, int& tf) {
+      const int k = i * NW + (l >> 5);
+      const bool time = i == 0 && k < 4;   // (2 T > 4 warps)
+      const int per_face = time ? 2 : NT / 2, j = time ? k : (k - 4) % NT;
+      mu = time ? 0 : 1 + (k - 4) / NT;
+      side = j / per_face;
+      tf = (j % per_face) * 32 + (l & 31);
+      return NTASK == 2 * NW || k < NTASK;
+    };
     float4 h[2][3], u[2][3];
+    int mu, side, tf;
 #pragma unroll
     for (int i = 0; i < 2; i++) {
-      const int mu = 2 * i + (w >> 2);
+      if (!task(i, mu, side, tf)) continue;
       int nbc[4] = {bc[0], bc[1], bc[2], bc[3]};
 #pragma unroll
       for (int m = 0; m < 4; m++)
         if (m == mu) nbc[m] = side ? (bc[m] == sg.nb[m] - 1 ? 0 : bc[m] + 1) : (bc[m] == 0 ? sg.nb[m] - 1 : bc[m] - 1);
-      const float4* hp =
-          A.faces + (((size_t)rhs * 2 + 1 - A.colour) * nhalf + block_number(sg, nbc)) * 1536 + (2 * mu + 1 - side) * 192 + tf;
-      const float4* up = A.flinks + bidx * 1536 + (2 * mu + side) * 192 + tf;
+      const int n = face_sites<NT>(mu);
+      const float4* hp = A.faces + (((size_t)rhs * 2 + 1 - A.colour) * nhalf + block_number(sg, nbc)) * (3 * FS) +
+                         3 * face_first<NT>(2 * mu + 1 - side) + tf;
+      const float4* up = A.flinks + bidx * (3 * FS) + 3 * face_first<NT>(2 * mu + side) + tf;
 #pragma unroll
       for (int a = 0; a < 3; a++) {
-        h[i][a] = hp[a * 64];
-        u[i][a] = __ldg(up + a * 64);
+        h[i][a] = hp[a * n];
+        u[i][a] = __ldg(up + a * n);
       }
     }
 #pragma unroll
-    for (int i = 0; i < 2; i++) face_mul(h[i], u[i], side, buf + (2 * (2 * i + (w >> 2)) + side) * 192 + tf);
+    for (int i = 0; i < 2; i++)
+      if (task(i, mu, side, tf))
+        face_mul(h[i], u[i], side, buf + 3 * face_first<NT>(2 * mu + side) + tf, face_sites<NT>(mu));
     __syncthreads();
     r = residual();
-    face_add<0>(r, buf, g, t, lc, l, kappa);
-    face_add<1>(r, buf, g, t, lc, l, kappa);
-    face_add<2>(r, buf, g, t, lc, l, kappa);
-    face_add<3>(r, buf, g, t, lc, l, kappa);
+    face_add<NT, 0>(r, buf, g, t, lc, l, kappa);
+    face_add<NT, 1>(r, buf, g, t, lc, l, kappa);
+    face_add<NT, 2>(r, buf, g, t, lc, l, kappa);
+    face_add<NT, 3>(r, buf, g, t, lc, l, kappa);
     __syncthreads();   // the products are read before the residual takes their place
   } else {
     r = residual();
   }
-  rs_store<BF>(r_s, 256, l, r);
+  rs_store<BF>(r_s, VB, l, r);
   cp_async_wait();   // this thread's copies; the barrier of the first MR step covers the others'
 
   PairSpinor x;
   mr_steps<S, BF>(r, x, r_s, f, sg, g, s, l, lc, kappa, nmr, red);
 
   if (A.last < 2) {
-    float4* out = A.faces + (((size_t)rhs * 2 + A.colour) * nhalf + blk) * 1536;
-    face_store<0>(out, x, lc, l);
-    face_store<1>(out, x, lc, l);
-    face_store<2>(out, x, lc, l);
-    face_store<3>(out, x, lc, l);
+    float4* out = A.faces + (((size_t)rhs * 2 + A.colour) * nhalf + blk) * (3 * FS);
+    face_store<NT, 0>(out, x, lc, l);
+    face_store<NT, 1>(out, x, lc, l);
+    face_store<NT, 2>(out, x, lc, l);
+    face_store<NT, 3>(out, x, lc, l);
   }
   if (A.last < 1) {
 #pragma unroll
-    for (int q = 0; q < 6; q++) rho_b[q * 256] = pair_rec(r, q);
+    for (int q = 0; q < 6; q++) rho_b[q * VB] = pair_rec(r, q);
   }
   if (!A.first) {
     PairSpinor y;
 #pragma unroll
     for (int q = 0; q < 6; q++) {
-      const float4 v = psi_b[q * 256];
+      const float4 v = psi_b[q * VB];
       y.re[q / 3][q % 3] = p2(v.x, v.y);
       y.im[q / 3][q % 3] = p2(v.z, v.w);
     }
@@ -1105,7 +1139,7 @@ __global__ void __launch_bounds__(256, 2)
   }
   if (A.last < 1) {
 #pragma unroll
-    for (int q = 0; q < 6; q++) psi_b[q * 256] = pair_rec(x, q);
+    for (int q = 0; q < 6; q++) psi_b[q * VB] = pair_rec(x, q);
   } else {
     char* psi = A.psi + (size_t)rhs * FieldsF::spinor_bytes * g.V;
     if (A.accumulate) pair_add(x, pair_load(psi, g.V, s));
@@ -1171,27 +1205,33 @@ __global__ void k_block_image(const float4* __restrict__ gauge, const float4* __
   }
 }
 
-// flinks of 4^4 blocks: one thread per (block, face, face site)
+// flinks: one thread per (block, face, face site)
+template <int NT>
 __global__ void k_face_links(const float4* __restrict__ gauge, Geom g, SapGeom sg, float4* __restrict__ out) {
+  constexpr int FS = all_face_sites<NT>();
+  const int nblocks = g.V / (64 * NT);
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (size_t)2 * g.V) return;   // 512 face sites per 256-site block
-  const int bidx = (int)(i >> 9), f = (int)(i >> 6) & 7, tf = (int)i & 63, nhalf = g.V / 512;
-  const int mu = f >> 1, side = f & 1, e = side ? 3 : 0;
+  if (i >= (size_t)nblocks * FS) return;
+  const int bidx = (int)(i / FS), j = (int)(i % FS), nhalf = nblocks / 2;
+  const int f = j < 128 ? j >> 6 : 2 + (j - 128) / (16 * NT), tf = j - face_first<NT>(f);
+  const int mu = f >> 1, side = f & 1, e = side ? (mu == 0 ? NT : 4) - 1 : 0;
   int bc[4], c[4];
   block_of(sg, bidx >= nhalf, bidx >= nhalf ? bidx - nhalf : bidx, bc);
   const int a = tf & 3, b = (tf >> 2) & 3, d = tf >> 4;
-  c[0] = 4 * bc[0] + (mu == 0 ? e : d);
+  c[0] = NT * bc[0] + (mu == 0 ? e : d);
   c[1] = 4 * bc[1] + (mu == 1 ? e : a);
   c[2] = 4 * bc[2] + (mu == 2 ? e : mu == 1 ? a : b);
   c[3] = 4 * bc[3] + (mu == 3 ? e : mu == 0 ? d : b);
   int s = ((c[0] * g.L[3] + c[3]) * g.L[2] + c[2]) * g.L[1] + c[1];
   if (!side) s = site_bwd(g, s, c, mu);
 #pragma unroll
-  for (int k = 0; k < 3; k++) out[((size_t)bidx * 24 + 3 * f + k) * 64 + tf] = gauge[(size_t)(3 * mu + k) * g.V + s];
+  for (int k = 0; k < 3; k++)
+    out[(size_t)bidx * (3 * FS) + 3 * face_first<NT>(f) + k * face_sites<NT>(mu) + tf] =
+        gauge[(size_t)(3 * mu + k) * g.V + s];
 }
 
 // Brings the context's block image for these blocks up to date; *img = nullptr
-// when there is no memory for it.  flinks only for 4^4 blocks.
+// when there is no memory for it.  flinks only for blocks of T x 4^3, T = 4 or 8.
 qcd_status block_image(qcd_ctx* c, const SapGeom& sg, bool half, bool faces, const unsigned char** img,
                        const float4** flinks) {
   SapImage& m = half ? c->sap_img16 : c->sap_img32;
@@ -1216,15 +1256,18 @@ qcd_status block_image(qcd_ctx* c, const SapGeom& sg, bool half, bool faces, con
     for (int mu = 0; mu < 4; mu++) m.block[mu] = sg.b[mu];
     m.gauge_id = c->gauge_id;
   }
-  if (faces && c->flinks_id != c->gauge_id) {
+  if (faces && (c->flinks_id != c->gauge_id || c->flinks_nt != sg.b[0])) {
     c->flinks_id = 0;
     const qcd_status st = devbuf_ensure(c->flinks, V * 96);
     if (st == QCD_ERR_OOM) return QCD_OK;
     QCD_TRY(st);
     ProfScope ps(c, FAM_LAYOUT, (double)V * 192, 0.0);
-    k_face_links<<<(unsigned)((2 * V + 255) / 256), 256, 0, c->stream>>>((const float4*)c->gaugeF.p, c->g, sg,
-                                                                         (float4*)c->flinks.p);
+    // (at most two face sites per site of a block)
+    auto kern = sg.b[0] == 4 ? k_face_links<4> : k_face_links<8>;
+    kern<<<(unsigned)((2 * V + 255) / 256), 256, 0, c->stream>>>((const float4*)c->gaugeF.p, c->g, sg,
+                                                                 (float4*)c->flinks.p);
     QCD_CUDA_OK(cudaGetLastError());
+    c->flinks_nt = sg.b[0];
     c->flinks_id = c->gauge_id;
   }
   *img = (const unsigned char*)m.buf.p;
@@ -1269,10 +1312,11 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   const double flops_site = P.nmr * (1320.0 * (1.0 - face / 8.0) + 504.0 + 192.0) + flops_gather;
   const int fam = sizeof(typename F::R) == 8 ? FAM_SAP_D : FAM_SAP_F;
   constexpr bool f32 = sizeof(typename F::R) == 4;
-  const bool b4 = sg.b[0] == 4 && sg.b[1] == 4 && sg.b[2] == 4 && sg.b[3] == 4;
+  const bool s4 = sg.b[1] == 4 && sg.b[2] == 4 && sg.b[3] == 4;
+  const bool b4 = s4 && (sg.b[0] == 4 || (f32 && sg.b[0] == 8));
   // FP32 blocks of at most 256 sites are staged in shared memory; without memory
-  // for the FP32 image (FromField), or for the block-ordered vectors of a 4^4
-  // block, the sweep runs on the lexicographic fields
+  // for the FP32 image (FromField), or for the block-ordered vectors of a block of
+  // 4 or 8 x 4^3, the sweep runs on the lexicographic fields
   const bool h16 = f32 && P.sap_half && sg.vb <= 256;
   const unsigned char* img = nullptr;
   SapB4 A = {};
@@ -1301,8 +1345,10 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   auto kernD = sg.vb <= 256   ? k_sap_sweep<FieldsD, 256, 1>
                : sg.vb <= 512 ? k_sap_sweep<FieldsD, 512, 1>
                               : k_sap_sweep<FieldsD, 1024, 1>;
-  auto kernB = !h16 ? k_sap_sweep_b4<float, false>
-                     : (P.sap_half == 2 ? k_sap_sweep_b4<__half, true> : k_sap_sweep_b4<__half, false>);
+  auto kernB = sg.b[0] == 8    ? k_sap_sweep_b4<float, false, 8>
+               : !h16            ? k_sap_sweep_b4<float, false, 4>
+               : P.sap_half == 2 ? k_sap_sweep_b4<__half, true, 4>
+                                 : k_sap_sweep_b4<__half, false, 4>;
   auto kernF = staged ? (!h16              ? k_sap_sweep_pair<float, false, 256, 2>
                          : P.sap_half == 2 ? k_sap_sweep_pair<__half, true, 256, 2>
                                            : k_sap_sweep_pair<__half, false, 256, 2>)
@@ -1310,10 +1356,10 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
                                       : k_sap_sweep_pair<FromImage, false, 1024, 1>)
                       : (sg.vb <= 512 ? k_sap_sweep_pair<FromField, false, 512, 1>
                                       : k_sap_sweep_pair<FromField, false, 1024, 1>);
-  const size_t smem = (size_t)sg.vb * (!f32      ? 192
-                                       : !staged ? 96
-                                       : !h16    ? 96 + Stage<float>::bytes
-                                                 : (P.sap_half == 2 && !use_b4 ? 48 : 96) + Stage<__half>::bytes);
+  const size_t smem = (size_t)sg.vb * (!f32                 ? 192
+                                       : !staged && !use_b4 ? 96
+                                       : !h16               ? 96 + Stage<float>::bytes
+                                              : (P.sap_half == 2 && !use_b4 ? 48 : 96) + Stage<__half>::bytes);
   // links and clover term read per active site and launch: their FP16 copies
   // (36 B per link, 144 B clover) for the 16-bit staged blocks, else FP32
   const double gcb = h16 ? 4 * 36.0 + 144.0 : 4 * lb + cb;
@@ -1347,7 +1393,7 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
             // 1095 -> 1093 and 229.5 -> 228.5.
             cudaLaunchConfig_t cfg = {};
             cfg.gridDim = grid;
-            cfg.blockDim = dim3(256);
+            cfg.blockDim = dim3(sg.vb);
             cfg.dynamicSmemBytes = smem;
             cfg.stream = c->stream;
             cudaLaunchAttribute at[1];
