@@ -278,10 +278,8 @@ qcd_status qcd_apply_dirac(qcd_ctx* c, const double* in, double* out, int nrhs, 
   const size_t b = spinor_bytes(c, precision) * nrhs;
   DevBuf* ws = precision == QCD_PREC_F64 ? c->wsD : c->wsF;
   QCD_TRY(devbuf_ensure(ws[4], b));
-  QCD_TRY(devbuf_ensure(ws[5], b));
   QCD_TRY(layout_spinor_import(c, in, ws[4].p, precision, nrhs));
-  QCD_TRY(dslash_apply(c, ws[4].p, ws[5].p, precision, nrhs, dagger ? 1 : 0, nullptr, nrhs));
-  QCD_TRY(layout_spinor_export(c, ws[5].p, out, precision, nrhs));
+  QCD_TRY(dslash_apply(c, ws[4].p, out, precision, nrhs, dagger ? 1 : 0, nullptr, nrhs, DSLASH_CANONICAL));
   QCD_CUDA_OK(cudaStreamSynchronize(c->stream));
   return QCD_OK;
 }

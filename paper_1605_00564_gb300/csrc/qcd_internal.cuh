@@ -501,7 +501,9 @@ qcd_status clover_export(qcd_ctx* c, double* out_dev);
 
 // out = D in (or D^+), internal layout, precision prec; mask may be null,
 // nactive = number of unmasked right-hand sides (for the timing records);
-// out_prec = QCD_PREC_H16 stores an FP32 operator's output as FP16 + scale
+// out_prec = QCD_PREC_H16 stores an FP32 operator's output as FP16 + scale,
+// DSLASH_CANONICAL the output of either precision in the caller's layout
+constexpr int DSLASH_CANONICAL = 100;
 qcd_status dslash_apply(qcd_ctx* c, const void* in, void* out, int prec, int nrhs, int dagger, const int* mask,
                         int nactive, int out_prec = -1);
 
