@@ -15,7 +15,7 @@
 
 #include <vector>
 
-#include "qcd_internal.cuh"
+#include "spin_pair.cuh"
 
 namespace {
 
@@ -210,6 +210,12 @@ ProjectShape project_shape(int ns, int nrhs) {
   return s;
 }
 
+// acc += conj(x) y in (re, im) lanes; miy = -i y
+__device__ __forceinline__ void cmac_conj2(float2& acc, float2 x, float2 y, float2 miy) {
+  acc = pfma(pbc(x.x), y, acc);
+  acc = pfma(pbc(x.y), miy, acc);
+}
+
 __global__ void __launch_bounds__(GEMM_TPB) k_dfl_project(const char* __restrict__ phi, const char* __restrict__ rho,
                                                            float2* __restrict__ cout, Geom g, BlkGeom bg, int ns,
                                                            int nrhs, ProjectShape sh, const int* mask) {
@@ -222,11 +228,11 @@ __global__ void __launch_bounds__(GEMM_TPB) k_dfl_project(const char* __restrict
   const int ntile = sh.tiles_k * sh.tiles_r;
   const int tile = threadIdx.x % ntile, slice = threadIdx.x / ntile;
   const int k0 = (tile / sh.tiles_r) * TK, r0 = (tile % sh.tiles_r) * TR;
-  Cplx<float> acc[TK][TR];
+  float2 acc[TK][TR];
 #pragma unroll
   for (int i = 0; i < TK; i++)
 #pragma unroll
-    for (int j = 0; j < TR; j++) acc[i][j] = cmk(0.f, 0.f);
+    for (int j = 0; j < TR; j++) acc[i][j] = p2(0.f, 0.f);
   __shared__ int site[PTS];
   for (int t0 = 0; t0 < bg.vb; t0 += PTS) {
     __syncthreads();
@@ -257,12 +263,14 @@ __global__ void __launch_bounds__(GEMM_TPB) k_dfl_project(const char* __restrict
         const float4* xp = (const float4*)(Pt + e * sh.ldp + k0);
         const float4* yp = (const float4*)(Rt + e * sh.ldr + r0);
         const float4 x0 = xp[0], x1 = xp[1], y0 = yp[0], y1 = yp[1];
-        const Cplx<float> x[TK] = {cmk(x0.x, x0.y), cmk(x0.z, x0.w), cmk(x1.x, x1.y), cmk(x1.z, x1.w)};
-        const Cplx<float> y[TR] = {cmk(y0.x, y0.y), cmk(y0.z, y0.w), cmk(y1.x, y1.y), cmk(y1.z, y1.w)};
+        const float2 x[TK] = {p2(x0.x, x0.y), p2(x0.z, x0.w), p2(x1.x, x1.y), p2(x1.z, x1.w)};
+        const float2 y[TR] = {p2(y0.x, y0.y), p2(y0.z, y0.w), p2(y1.x, y1.y), p2(y1.z, y1.w)};
 #pragma unroll
-        for (int i = 0; i < TK; i++)
+        for (int j = 0; j < TR; j++) {
+          const float2 miy = p2(y[j].y, -y[j].x);
 #pragma unroll
-          for (int j = 0; j < TR; j++) cmac_conj(acc[i][j], x[i], y[j]);
+          for (int i = 0; i < TK; i++) cmac_conj2(acc[i][j], x[i], y[j], miy);
+        }
       }
   }
   __syncthreads();
@@ -272,7 +280,7 @@ __global__ void __launch_bounds__(GEMM_TPB) k_dfl_project(const char* __restrict
     for (int i = 0; i < TK; i++)
 #pragma unroll
       for (int j = 0; j < TR; j++)
-        red[((size_t)slice * rp + r0 + j) * kp + k0 + i] = make_float2(acc[i][j].re, acc[i][j].im);
+        red[((size_t)slice * rp + r0 + j) * kp + k0 + i] = acc[i][j];
   __syncthreads();
   for (int o = threadIdx.x; o < ns * nrhs; o += blockDim.x) {
     const int r = o / ns, k = o - r * ns;
@@ -286,15 +294,21 @@ __global__ void __launch_bounds__(GEMM_TPB) k_dfl_project(const char* __restrict
   }
 }
 
-// Prolongation x_r(y) = sum_k e[r][b(y)][k] phi_k(y).  One CTA per block, threads
-// over its sites; the block's coefficients in shared memory; a thread takes two
-// components of up to 12 right-hand sides at a time, so phi is read once per 12.
-constexpr int PRG = 12;
-__global__ void __launch_bounds__(256) k_dfl_prolong(const char* __restrict__ phi, const float2* __restrict__ e, char* __restrict__ x, Geom g,
-                              BlkGeom bg, int ns, int nrhs, const int* mask) {
+// Prolongation x_r(y) = sum_k e[r][b(y)][k] phi_k(y).  Each of a block's three CTAs
+// takes PRW of the six words of its sites; the block's coefficients in shared memory;
+// a thread takes a word (two components) of up to 12 right-hand sides at a time, so
+// phi is read once per 12.  (16^3x32, 12 RHS, N_s 20: with two-lane arithmetic here and
+// in the projection, and three CTAs per block instead of one, which left the second of
+// two waves two thirds empty, 1.77 -> 1.61 ms of deflation per outer iteration.
+// Fields kept in block order: 1.58, not worth a second layout.)
+constexpr int PRG = 12, PRW = 2;
+__global__ void __launch_bounds__(256, 2) k_dfl_prolong(const char* __restrict__ phi, const float2* __restrict__ e,
+                                                        char* __restrict__ x, Geom g, BlkGeom bg, int ns, int nrhs,
+                                                        const int* mask) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* cf = (float2*)smem_raw;   // [k][nrhs rounded up to PRG], zeros beyond nrhs
-  const int blk = blockIdx.x, ld = (nrhs + PRG - 1) / PRG * PRG;
+  const int blk = blockIdx.x / (6 / PRW), ld = (nrhs + PRG - 1) / PRG * PRG;
+  const int q0 = blockIdx.x % (6 / PRW) * PRW;
   for (int o = threadIdx.x; o < ns * ld; o += blockDim.x) {
     const int r = o / ns, k = o - r * ns;
     cf[k * ld + r] = r < nrhs ? e[((size_t)r * bg.nblk + blk) * ns + k] : make_float2(0.f, 0.f);
@@ -306,28 +320,29 @@ __global__ void __launch_bounds__(256) k_dfl_prolong(const char* __restrict__ ph
     const int s = blk_site(bg, g, blk, l, lc, c);
     for (int r0 = 0; r0 < nrhs; r0 += PRG)
 #pragma unroll 1
-      for (int q = 0; q < 6; q++) {
-        Cplx<float> a0[PRG], a1[PRG];
+      for (int q = q0; q < q0 + PRW; q++) {
+        float2 a0[PRG], a1[PRG];
 #pragma unroll
-        for (int i = 0; i < PRG; i++) a0[i] = a1[i] = cmk(0.f, 0.f);
+        for (int i = 0; i < PRG; i++) a0[i] = a1[i] = p2(0.f, 0.f);
 #pragma unroll 4
         for (int k = 0; k < ns; k++) {
           const float4 v = __ldg((const float4*)(phi + k * fb) + (size_t)q * g.V + s);
+          const float2 v0 = p2(v.x, v.y), v1 = p2(v.z, v.w), iv0 = p2(-v.y, v.x), iv1 = p2(-v.w, v.z);
           const float4* w = (const float4*)(cf + k * ld + r0);
 #pragma unroll
           for (int i = 0; i < PRG; i += 2) {
             const float4 u = w[i >> 1];
-            cmac(a0[i], cmk(u.x, u.y), cmk(v.x, v.y));
-            cmac(a1[i], cmk(u.x, u.y), cmk(v.z, v.w));
-            cmac(a0[i + 1], cmk(u.z, u.w), cmk(v.x, v.y));
-            cmac(a1[i + 1], cmk(u.z, u.w), cmk(v.z, v.w));
+            a0[i] = pfma(pbc(u.y), iv0, pfma(pbc(u.x), v0, a0[i]));
+            a1[i] = pfma(pbc(u.y), iv1, pfma(pbc(u.x), v1, a1[i]));
+            a0[i + 1] = pfma(pbc(u.w), iv0, pfma(pbc(u.z), v0, a0[i + 1]));
+            a1[i + 1] = pfma(pbc(u.w), iv1, pfma(pbc(u.z), v1, a1[i + 1]));
           }
         }
 #pragma unroll
         for (int i = 0; i < PRG; i++)
           if (r0 + i < nrhs && (!mask || mask[r0 + i]))
             ((float4*)(x + (size_t)(r0 + i) * fb))[(size_t)q * g.V + s] =
-                make_float4(a0[i].re, a0[i].im, a1[i].re, a1[i].im);
+                make_float4(a0[i].x, a0[i].y, a1[i].x, a1[i].y);
       }
   }
 }
@@ -936,9 +951,9 @@ qcd_status dfl_low_mode(qcd_ctx* c, const void* rho, void* x, int n, const int* 
   }
   {
     ProfScope ps(c, FAM_DFL, (double)spinor_bytes(c, QCD_PREC_F32) * (ns + nactive), 8.0 * c->g.V * 12 * ns * nactive);
-    k_dfl_prolong<<<bg.nblk, bg.vb < 256 ? bg.vb : 256, sizeof(float2) * ns * ((n + PRG - 1) / PRG * PRG), c->stream>>>(
-        (const char*)d->phi.p, xl, (char*)x, c->g, bg,
-                                                                         ns, n, mask);
+    k_dfl_prolong<<<6 / PRW * bg.nblk, bg.vb < 256 ? bg.vb : 256,
+                    sizeof(float2) * ns * ((n + PRG - 1) / PRG * PRG), c->stream>>>((const char*)d->phi.p, xl, (char*)x,
+                                                                                    c->g, bg, ns, n, mask);
     QCD_CUDA_OK(cudaGetLastError());
   }
   return QCD_OK;
