@@ -471,6 +471,16 @@ __global__ void k_little_apply(const double2* __restrict__ M, const float2* __re
   }
 }
 
+// FP32 copy of na / (ns ns) matrices, transposed
+__global__ void k_little_transpose(const double2* __restrict__ in, float2* __restrict__ out, int ns, size_t na) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < na; i += (size_t)gridDim.x * blockDim.x) {
+    const size_t m = i / ns, b = m / ns;
+    const int l = (int)(m - b * ns), k = (int)(i - m * ns);
+    const double2 v = in[(b * ns + k) * ns + l];
+    out[i] = make_float2((float)v.x, (float)v.y);
+  }
+}
+
 // FP32 copy of an FP64 complex array
 __global__ void k_to_float2(const double2* __restrict__ in, float2* __restrict__ out, size_t n) {
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
@@ -494,43 +504,75 @@ constexpr int LITTLE_RHS = 24;   // right-hand sides of one little solve
 constexpr int LITTLE_JR = 6;     // (j, r) sums per thread: 64 steps x 24 RHS / 256
 
 // q = A p on the CTA's blocks, and the CTA's partial sums of (q_j, q), j < nj, to
-// part[(r nj + j) gridDim + cta].  Per block the nine neighbours' p and the matrix
-// rows are staged in shared memory; thread (k, r), right-hand side fastest.
-__global__ void __launch_bounds__(LTPB) k_little_q(const float2* __restrict__ A, const float2* __restrict__ p,
+// part[(r nj + j) gridDim + cta].  At: the matrix with the row index of each of its
+// nine parts fastest.  A thread takes row k of one of the nine parts for up to LQR right-hand
+// sides: the matrix is read once, consecutive rows by consecutive threads, from
+// global memory, and the neighbours' p are broadcast reads from shared memory, six
+// 128-bit words for 12 products.  (One output per thread took two shared-memory words
+// per product, 86,000 per block and step, and staged the matrix.)  Bound by the latency
+// of its loads: four CTAs of 64 registers per SM hold all 512 blocks of a 16^3x32
+// lattice at once (three, in two waves, are no faster than the old form); the dots read
+// 128-bit words, the orthogonalisation below keeps 24 loads in flight: deflation 1.61
+// -> 1.41 ms per outer iteration (12 RHS, N_s 20, 24 steps).  The nine parts are summed in a fixed order.
+constexpr int LQR = 12;
+__global__ void __launch_bounds__(LTPB, 4) k_little_q(const float2* __restrict__ At, const float2* __restrict__ p,
                                                    float2* __restrict__ q, const float2* __restrict__ qbase,
                                                    size_t stride, int nj, double2* __restrict__ part, BlkGeom bg,
                                                    int ns, int n) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2* xs = (float2*)smem_raw;                 // [9 ns][n]
-  float2* As = xs + (size_t)9 * ns * n;           // [ns][9 ns]
-  float2* qs = As + (size_t)9 * ns * ns;          // [ns][n]
+  float2* xs = (float2*)smem_raw;                 // [9 ns][LQR]
+  float2* red = xs + (size_t)9 * ns * LQR;        // [9][LQR][ns]
+  float2* qs = red + (size_t)9 * ns * LQR;        // [ns][n]
   float2 acc[LITTLE_JR];
 #pragma unroll
   for (int i = 0; i < LITTLE_JR; i++) acc[i] = make_float2(0.f, 0.f);
   for (int blk = blockIdx.x; blk < bg.nblk; blk += gridDim.x) {
     int nbr[9];
     little_neighbours(bg, blk, nbr);
-    __syncthreads();
-    const float2* a = A + (size_t)blk * 9 * ns * ns;
-    for (int i = threadIdx.x; i < 9 * ns * ns; i += LTPB) {
-      const int mk = i / ns, m = mk / ns;
-      As[((mk - m * ns) * 9 + m) * ns + i - mk * ns] = __ldg(a + i);
-    }
+    for (int c0 = 0; c0 < n; c0 += LQR) {
+      __syncthreads();
 #pragma unroll
-    for (int m = 0; m < 9; m++)
-      for (int i = threadIdx.x; i < ns * n; i += LTPB) {
-        const int r = i / ns, k = i - r * ns;
-        xs[(m * ns + k) * n + r] = p[((size_t)r * bg.nblk + nbr[m]) * ns + k];
+      for (int m = 0; m < 9; m++)
+        for (int i = threadIdx.x; i < ns * LQR; i += LTPB) {
+          const int r = i / ns, k = i - r * ns;
+          xs[(m * ns + k) * LQR + r] =
+              c0 + r < n ? p[((size_t)(c0 + r) * bg.nblk + nbr[m]) * ns + k] : make_float2(0.f, 0.f);
+        }
+      __syncthreads();
+      for (int t = threadIdx.x; t < 9 * ns; t += LTPB) {
+        const int m = t / ns, k = t - m * ns;
+        const float2* a = At + ((size_t)blk * 9 + m) * ns * ns + k;
+        const float4* xv = (const float4*)(xs + (size_t)m * ns * LQR);
+        float2 u[LQR];
+#pragma unroll
+        for (int r = 0; r < LQR; r++) u[r] = p2(0.f, 0.f);
+#pragma unroll 10
+        for (int l = 0; l < ns; l++) {
+          const float2 w = __ldg(a + l * ns), wi = p2(-w.y, w.y);
+#pragma unroll
+          for (int r = 0; r < LQR; r += 2) {
+            const float4 x = xv[(l * LQR + r) >> 1];
+            u[r] = pfma(wi, p2(x.y, x.x), pfma(pbc(w.x), p2(x.x, x.y), u[r]));
+            u[r + 1] = pfma(wi, p2(x.w, x.z), pfma(pbc(w.x), p2(x.z, x.w), u[r + 1]));
+          }
+        }
+#pragma unroll
+        for (int r = 0; r < LQR; r++) red[(m * LQR + r) * ns + k] = u[r];
       }
-    __syncthreads();
-    for (int o = threadIdx.x; o < ns * n; o += LTPB) {
-      const int k = o / n, r = o - k * n;
-      float ar = 0.f, ai = 0.f;
-      const float2* row = As + k * 9 * ns;
-#pragma unroll 9
-      for (int l = 0; l < 9 * ns; l++) little_mac(ar, ai, row[l], xs[l * n + r]);
-      qs[o] = make_float2(ar, ai);
-      q[((size_t)r * bg.nblk + blk) * ns + k] = qs[o];
+      __syncthreads();
+      for (int o = threadIdx.x; o < ns * LQR; o += LTPB) {
+        const int r = o / ns, k = o - r * ns;
+        if (c0 + r >= n) continue;
+        float2 t = red[o];
+#pragma unroll
+        for (int m = 1; m < 9; m++) {
+          const float2 w = red[m * LQR * ns + o];
+          t.x += w.x;
+          t.y += w.y;
+        }
+        qs[k * n + c0 + r] = t;
+        q[((size_t)(c0 + r) * bg.nblk + blk) * ns + k] = t;
+      }
     }
     if (nj == 0) continue;
     __syncthreads();
@@ -540,13 +582,22 @@ __global__ void __launch_bounds__(LTPB) k_little_q(const float2* __restrict__ A,
       if (o < nj * n) {
         const int j = o / n, r = o - j * n;
         const float2* qj = qbase + j * stride + ((size_t)r * bg.nblk + blk) * ns;
-#pragma unroll 4
-        for (int k = 0; k < ns; k++) {
-          const float2 u = __ldg(qj + k), v = qs[k * n + r];
+        auto mac = [&](float2 u, float2 v) {
           acc[i].x = fmaf(u.x, v.x, acc[i].x);
           acc[i].x = fmaf(u.y, v.y, acc[i].x);
           acc[i].y = fmaf(u.x, v.y, acc[i].y);
           acc[i].y = fmaf(-u.y, v.x, acc[i].y);
+        };
+        if (ns % 2 == 0) {   // (then every little vector's block is 16-byte aligned)
+#pragma unroll 5
+          for (int k = 0; k < ns; k += 2) {
+            const float4 u = __ldg((const float4*)(qj + k));
+            mac(p2(u.x, u.y), qs[k * n + r]);
+            mac(p2(u.z, u.w), qs[(k + 1) * n + r]);
+          }
+        } else {
+#pragma unroll 4
+          for (int k = 0; k < ns; k++) mac(__ldg(qj + k), qs[k * n + r]);
         }
       }
     }
@@ -593,7 +644,7 @@ __global__ void __launch_bounds__(LTPB) k_little_orth(float2* __restrict__ qi, f
   for (int i = blockIdx.x * LTPB + threadIdx.x; i < N; i += gridDim.x * LTPB) {
     const size_t o = (size_t)r * N + i;
     float2 q = qi[o], p = pi[o];
-#pragma unroll 4
+#pragma unroll 12
     for (int j = 0; j < nj; j++) {
       const float2 w = ds[j], a = __ldg(qbase + j * stride + o), b = __ldg(pbase + j * stride + o);
       q.x -= w.x * a.x - w.y * a.y; q.y -= w.x * a.y + w.y * a.x;
@@ -776,7 +827,7 @@ static qcd_status dfl_little_build(qcd_ctx* c) {
     QCD_TRY(devbuf_ensure(d->Af, sizeof(float2) * na));
     QCD_TRY(devbuf_ensure(d->Ainvf, sizeof(float2) * ni));
     ProfScope ps(c, FAM_DFL, 24.0 * (na + ni), 0.0, 2);
-    k_to_float2<<<1024, 256, 0, c->stream>>>((const double2*)d->A.p, (float2*)d->Af.p, na);
+    k_little_transpose<<<1024, 256, 0, c->stream>>>((const double2*)d->A.p, (float2*)d->Af.p, ns, na);
     k_to_float2<<<1024, 256, 0, c->stream>>>((const double2*)d->Ainv.p, (float2*)d->Ainvf.p, ni);
     QCD_CUDA_OK(cudaGetLastError());
   }
@@ -811,7 +862,7 @@ static qcd_status little_gcr_tile(qcd_ctx* c, DflState* d, float2* res, float2* 
   // one element per thread of the orthogonalisation (its time is the latency of the
   // loads along j), at most LITTLE_G CTAs per RHS
   const int Go = (N + LTPB - 1) / LTPB < LITTLE_G ? (N + LTPB - 1) / LTPB : LITTLE_G;
-  const size_t sm_q = sizeof(float2) * ((size_t)9 * ns * n + (size_t)9 * ns * ns + (size_t)ns * n);
+  const size_t sm_q = sizeof(float2) * ((size_t)2 * 9 * ns * LQR + (size_t)ns * n);
   const size_t sm_s = sizeof(float2) * ((size_t)ns * n + (size_t)ns * ns);
   QCD_CUDA_OK(cudaFuncSetAttribute(k_little_q, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_q));
   const float2* Ainv = (const float2*)d->Ainvf.p;
