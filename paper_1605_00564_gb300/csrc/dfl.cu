@@ -496,7 +496,8 @@ __global__ void k_to_float2(const double2* __restrict__ in, float2* __restrict__
 // addition of a warp takes the SM 16 cycles: the shuffle sums of 256 threads were
 // most of the time of the dots).  Masked right-hand sides have a zero residual and
 // stay zero.  A deflated 16^3x32 solve, 12 RHS, N_s 20, 24 steps: all deflation
-// kernels of an outer iteration 3.5 -> 1.75 ms.
+// kernels of an outer iteration 3.5 -> 1.75 ms; with each launch overlapping the end of
+// the one before it 1.41 -> 1.24.
 // ---------------------------------------------------------------------------
 constexpr int LTPB = 256;
 constexpr int LITTLE_G = 608;    // CTAs of the kernels that leave partial sums
@@ -523,6 +524,8 @@ __global__ void __launch_bounds__(LTPB, 4) k_little_q(const float2* __restrict__
   float2* xs = (float2*)smem_raw;                 // [9 ns][LQR]
   float2* red = xs + (size_t)9 * ns * LQR;        // [9][LQR][ns]
   float2* qs = red + (size_t)9 * ns * LQR;        // [ns][n]
+  launch_dependents();
+  dependency_wait();
   float2 acc[LITTLE_JR];
 #pragma unroll
   for (int i = 0; i < LITTLE_JR; i++) acc[i] = make_float2(0.f, 0.f);
@@ -536,7 +539,7 @@ __global__ void __launch_bounds__(LTPB, 4) k_little_q(const float2* __restrict__
         for (int i = threadIdx.x; i < ns * LQR; i += LTPB) {
           const int r = i / ns, k = i - r * ns;
           xs[(m * ns + k) * LQR + r] =
-              c0 + r < n ? p[((size_t)(c0 + r) * bg.nblk + nbr[m]) * ns + k] : make_float2(0.f, 0.f);
+              c0 + r < n ? __ldcg(p + ((size_t)(c0 + r) * bg.nblk + nbr[m]) * ns + k) : make_float2(0.f, 0.f);
         }
       __syncthreads();
       for (int t = threadIdx.x; t < 9 * ns; t += LTPB) {
@@ -591,13 +594,13 @@ __global__ void __launch_bounds__(LTPB, 4) k_little_q(const float2* __restrict__
         if (ns % 2 == 0) {   // (then every little vector's block is 16-byte aligned)
 #pragma unroll 5
           for (int k = 0; k < ns; k += 2) {
-            const float4 u = __ldg((const float4*)(qj + k));
+            const float4 u = __ldcg((const float4*)(qj + k));
             mac(p2(u.x, u.y), qs[k * n + r]);
             mac(p2(u.z, u.w), qs[(k + 1) * n + r]);
           }
         } else {
 #pragma unroll 4
-          for (int k = 0; k < ns; k++) mac(__ldg(qj + k), qs[k * n + r]);
+          for (int k = 0; k < ns; k++) mac(__ldcg(qj + k), qs[k * n + r]);
         }
       }
     }
@@ -616,8 +619,10 @@ __global__ void __launch_bounds__(LTPB, 4) k_little_q(const float2* __restrict__
 __global__ void k_little_sum(const double2* __restrict__ part, int nj, int G, double2* __restrict__ out, int n) {
   const int j = blockIdx.x, r = blockIdx.y;
   double2 t = make_double2(0, 0);
+  launch_dependents();
+  dependency_wait();
   for (int i = threadIdx.x; i < G; i += 32) {
-    const double2 v = part[((size_t)r * nj + j) * G + i];
+    const double2 v = __ldcg(part + ((size_t)r * nj + j) * G + i);
     t.x += v.x;
     t.y += v.y;
   }
@@ -635,24 +640,26 @@ __global__ void __launch_bounds__(LTPB) k_little_orth(float2* __restrict__ qi, f
   __shared__ float2 ds[64];
   __shared__ float sh[3][LTPB];
   const int r = blockIdx.y;
+  launch_dependents();
+  dependency_wait();
   if ((int)threadIdx.x < nj) {
-    const double2 v = d[(size_t)threadIdx.x * n + r];
+    const double2 v = __ldcg(d + (size_t)threadIdx.x * n + r);
     ds[threadIdx.x] = make_float2((float)v.x, (float)v.y);
   }
   __syncthreads();
   float n2 = 0.f, cr = 0.f, ci = 0.f;
   for (int i = blockIdx.x * LTPB + threadIdx.x; i < N; i += gridDim.x * LTPB) {
     const size_t o = (size_t)r * N + i;
-    float2 q = qi[o], p = pi[o];
+    float2 q = __ldcg(qi + o), p = __ldcg(pi + o);
 #pragma unroll 12
     for (int j = 0; j < nj; j++) {
-      const float2 w = ds[j], a = __ldg(qbase + j * stride + o), b = __ldg(pbase + j * stride + o);
+      const float2 w = ds[j], a = __ldcg(qbase + j * stride + o), b = __ldcg(pbase + j * stride + o);
       q.x -= w.x * a.x - w.y * a.y; q.y -= w.x * a.y + w.y * a.x;
       p.x -= w.x * b.x - w.y * b.y; p.y -= w.x * b.y + w.y * b.x;
     }
     qi[o] = q;
     pi[o] = p;
-    const float2 v = res[o];
+    const float2 v = __ldcg(res + o);
     n2 = fmaf(q.x, q.x, n2);
     n2 = fmaf(q.y, q.y, n2);
     cr = fmaf(q.x, v.x, cr);
@@ -684,9 +691,11 @@ __global__ void __launch_bounds__(LTPB) k_little_orth(float2* __restrict__ qi, f
 __global__ void k_little_scalars(const double2* __restrict__ part, int G, float4* __restrict__ out) {
   const int r = blockIdx.x;
   double2 a = make_double2(0, 0), c = make_double2(0, 0);
+  launch_dependents();
+  dependency_wait();
   for (int i = threadIdx.x; i < G; i += 32) {
-    a.x += part[(size_t)r * 2 * G + i].x;
-    const double2 v = part[((size_t)r * 2 + 1) * G + i];
+    a.x += __ldcg(part + (size_t)r * 2 * G + i).x;
+    const double2 v = __ldcg(part + ((size_t)r * 2 + 1) * G + i);
     c.x += v.x;
     c.y += v.y;
   }
@@ -708,17 +717,19 @@ __global__ void __launch_bounds__(LTPB) k_little_step(float2* __restrict__ x, fl
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* rs = (float2*)smem_raw;                 // [ns][n]
   float2* As = rs + (size_t)ns * n;               // [ns][ns]
+  launch_dependents();
   for (int blk = blockIdx.x; blk < bg.nblk; blk += gridDim.x) {
     __syncthreads();
     if (pnext)
       for (int i = threadIdx.x; i < ns * ns; i += LTPB) As[i] = __ldg(Ainv + (size_t)blk * ns * ns + i);
+    dependency_wait();   // (the inverses are constant)
     for (int i = threadIdx.x; i < ns * n; i += LTPB) {
       const int r = i / ns, k = i - r * ns;
       const size_t o = ((size_t)r * bg.nblk + blk) * ns + k;
-      float2 v = res[o];
+      float2 v = __ldcg(res + o);
       if (!start) {
-        const float4 c = sc[r];
-        float2 pp = p[o], qq = q[o], xx = first ? make_float2(0.f, 0.f) : x[o];
+        const float4 c = __ldcg(sc + r);
+        float2 pp = __ldcg(p + o), qq = __ldcg(q + o), xx = first ? make_float2(0.f, 0.f) : __ldcg(x + o);
         pp.x *= c.x; pp.y *= c.x;
         qq.x *= c.x; qq.y *= c.x;
         xx.x += c.y * pp.x - c.z * pp.y; xx.y += c.y * pp.y + c.z * pp.x;
@@ -867,16 +878,20 @@ static qcd_status little_gcr_tile(qcd_ctx* c, DflState* d, float2* res, float2* 
   QCD_CUDA_OK(cudaFuncSetAttribute(k_little_q, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_q));
   const float2* Ainv = (const float2*)d->Ainvf.p;
   const unsigned Gs = (unsigned)bg.nblk;
-  k_little_step<<<Gs, LTPB, sm_s, c->stream>>>(xl, res, nullptr, nullptr, P, Ainv, sc, 0, 1, bg, ns, n);
+  const dim3 threads(LTPB);
+  QCD_CUDA_OK(launch_after(c->stream, false, Gs, threads, sm_s, k_little_step, xl, res, nullptr, nullptr, P, Ainv, sc, 0,
+                           1, bg, ns, n));
   for (int i = 0; i < m; i++) {
     float2* pi = P + vlen * i;
     float2* qi = Q + vlen * i;
-    k_little_q<<<Gq, LTPB, sm_q, c->stream>>>((const float2*)d->Af.p, pi, qi, Q, vlen, i, part, bg, ns, n);
-    if (i > 0) k_little_sum<<<dim3(i, n), 32, 0, c->stream>>>(part, i, Gq, dots, n);
-    k_little_orth<<<dim3(Go, n), LTPB, 0, c->stream>>>(qi, pi, Q, P, vlen, i, dots, res, N, n, part);
-    k_little_scalars<<<n, 32, 0, c->stream>>>(part, Go, sc);
-    k_little_step<<<Gs, LTPB, sm_s, c->stream>>>(xl, res, pi, qi, i + 1 < m ? pi + vlen : nullptr, Ainv, sc, i == 0, 0,
-                                                 bg, ns, n);
+    QCD_CUDA_OK(launch_after(c->stream, true, Gq, threads, sm_q, k_little_q, (const float2*)d->Af.p, pi, qi, Q, vlen, i,
+                             part, bg, ns, n));
+    if (i > 0) QCD_CUDA_OK(launch_after(c->stream, true, dim3(i, n), 32, 0, k_little_sum, part, i, Gq, dots, n));
+    QCD_CUDA_OK(launch_after(c->stream, true, dim3(Go, n), threads, 0, k_little_orth, qi, pi, Q, P, vlen, i, dots, res, N,
+                             n, part));
+    QCD_CUDA_OK(launch_after(c->stream, true, n, 32, 0, k_little_scalars, part, Go, sc));
+    QCD_CUDA_OK(launch_after(c->stream, true, Gs, threads, sm_s, k_little_step, xl, res, pi, qi,
+                             i + 1 < m ? pi + vlen : nullptr, Ainv, sc, i == 0, 0, bg, ns, n));
   }
   QCD_CUDA_OK(cudaGetLastError());
   return QCD_OK;

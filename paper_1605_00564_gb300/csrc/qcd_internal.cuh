@@ -499,6 +499,30 @@ qcd_status layout_spinor_import(qcd_ctx* c, const double* in, void* out, int pre
 qcd_status layout_spinor_export(qcd_ctx* c, const void* in, double* out, int prec, int nrhs);
 qcd_status clover_export(qcd_ctx* c, double* out_dev);
 
+// Programmatic dependent launch.  A kernel launched with overlap may start while the
+// one before it still runs, once that one's CTAs have all called launch_dependents() or
+// ended; its CTAs must call dependency_wait() before they touch anything the kernels
+// before it read or write (it returns when those have completed and their writes are
+// visible, at once without overlap), and do not read what those wrote through the
+// read-only path (__ldg), which is for data that nobody writes while the kernel runs.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <typename... P, typename... A>
+cudaError_t launch_after(cudaStream_t stream, bool overlap, dim3 grid, dim3 block, size_t smem, void (*kernel)(P...),
+                         A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // out = D in (or D^+), internal layout, precision prec; mask may be null,
 // nactive = number of unmasked right-hand sides (for the timing records);
 // out_prec = QCD_PREC_H16 stores an FP32 operator's output as FP16 + scale,

@@ -524,10 +524,6 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
                : "memory");
 }
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-// programmatic dependent launch: let the next launch's CTAs onto free SMs; wait until
-// the previous launch has completed and its writes are visible
-__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // The block residual shared between neighbouring threads, six records q = 3 c + a
@@ -926,9 +922,9 @@ __device__ __forceinline__ int face_site_of(int l) {   // index of site l on a m
 // sites of a mu face and the first site of face f = 2 mu + side in the order of
 // the faces; 128 + 96 T in all (at most 2 per site of the block)
 template <int NT>
-__host__ __device__ constexpr int face_sites(int mu) { return mu == 0 ? 64 : 16 * NT; }
+__host__ __device__ constexpr int face_sites(int mu) { return NT == 4 || mu == 0 ? 64 : 16 * NT; }
 template <int NT>
-__host__ __device__ constexpr int face_first(int f) { return f < 2 ? 64 * f : 128 + (f - 2) * 16 * NT; }
+__host__ __device__ constexpr int face_first(int f) { return NT == 4 || f < 2 ? 64 * f : 128 + (f - 2) * 16 * NT; }
 template <int NT>
 __host__ __device__ constexpr int all_face_sites() { return 128 + 96 * NT; }
 
@@ -1068,14 +1064,21 @@ __global__ void __launch_bounds__(64 * NT, 8 / NT)
     float4* buf = (float4*)r_s;
     constexpr int NTASK = FS / 32;
     // task i of this warp: its face 2 mu + side and its 32 sites of it, from tf on
+    const int w = l >> 5, side4 = (w >> 1) & 1, tf4 = ((w & 1) << 5) | (l & 31);   // (T = 4)
     auto task = [&](int i, int& mu, int& side, int& tf) {
-      const int k = i * NW + (l >> 5);
+      if (NT == 4) {
+        mu = 2 * i + (w >> 2);
+        side = side4;
+        tf = tf4;
+        return true;
+      }
+      const int k = i * NW + w;
       const bool time = i == 0 && k < 4;   // (2 T > 4 warps)
       const int per_face = time ? 2 : NT / 2, j = time ? k : (k - 4) % NT;
       mu = time ? 0 : 1 + (k - 4) / NT;
       side = j / per_face;
       tf = (j % per_face) * 32 + (l & 31);
-      return NTASK == 2 * NW || k < NTASK;
+      return k < NTASK;
     };
     float4 h[2][3], u[2][3];
     int mu, side, tf;
@@ -1391,17 +1394,8 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
             // its launch and the staging of its fields.  Measured per half-cycle, FP16
             // fields, one RHS: 24^3x48 108.8 -> 105.2 us, 16^3x32 25.2 -> 24.1; 12 RHS:
             // 1095 -> 1093 and 229.5 -> 228.5.
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = grid;
-            cfg.blockDim = dim3(sg.vb);
-            cfg.dynamicSmemBytes = smem;
-            cfg.stream = c->stream;
-            cudaLaunchAttribute at[1];
-            at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-            at[0].val.programmaticStreamSerializationAllowed = 1;
-            cfg.attrs = at;
-            cfg.numAttrs = gather ? 1 : 0;
-            QCD_CUDA_OK(cudaLaunchKernelEx(&cfg, kernB, A, c->g, sg, (float)c->kappa, P.nmr, nrhs, mask));
+            QCD_CUDA_OK(launch_after(c->stream, gather, grid, sg.vb, smem, kernB, A, c->g, sg, (float)c->kappa, P.nmr,
+                                     nrhs, mask));
           } else {
             kernF<<<grid, sg.vb, smem, c->stream>>>(rin, rho, psi, delta, (const float4*)gauge, (const float4*)clover,
                                                     img, c->g, sg, col, gather, first, last, (float)c->kappa, P.nmr,
