@@ -356,7 +356,18 @@ __device__ __forceinline__ void gather_round(const BlockD& B, const Geom& g, con
 // both CTAs of the block
 __device__ __forceinline__ void sync_block() { cooperative_groups::this_cluster().sync(); }
 
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, 2)
+// RES: CTAs that share an SM.  Three (168 registers, 300 bytes of spills) where two leave
+// the last wave with one CTA per SM, whose four warps the FP64 pipe waits for; two (254
+// registers) on up to 2 CTAs per SM in all, and on 3 to 4, where 2 + 2 beats 3 + 1.
+// Measured with RES = 2 and 3, 8^3x16: 8 RHS (256 CTAs) 334 and 336 us, 10 to 14 (320 to
+// 448) 531 and 494, 16 (512) 660 and 684, 20 (640) 853 and 816; 16^3x32: one RHS (512) 671
+// and 693, two (1,024) 1,183 and 1,164, 12 6,646 and 6,551.
+inline bool d4_three(unsigned ctas) {
+  const unsigned per_sm = (ctas + 151) / 152;
+  return per_sm > 2 && per_sm != 4;
+}
+template <int RES>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, RES)
     k_sap_sweep_d4(const char* __restrict__ rho_src, char* __restrict__ rho, char* __restrict__ psi,
                    char* __restrict__ delta, const void* __restrict__ gauge, const void* __restrict__ clover, Geom g,
                    SapGeom sg, int colour, int gather, int psi_init, int last, double kappa, int nmr, int nrhs,
@@ -1372,8 +1383,9 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   else
     QCD_CUDA_OK(cudaFuncSetAttribute(kernD, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const size_t smem_d4 = (size_t)2 * 12 * BlockD::N * sizeof(double2);
+  auto kernC = d4_three(2 * grid.x) ? k_sap_sweep_d4<3> : k_sap_sweep_d4<2>;
   if (!f32 && b4)
-    QCD_CUDA_OK(cudaFuncSetAttribute(k_sap_sweep_d4, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_d4));
+    QCD_CUDA_OK(cudaFuncSetAttribute(kernC, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_d4));
   auto issue = [&]() -> qcd_status {
     for (int cy = 0; cy < P.ncy; cy++)
       for (int col = 0; col < 2; col++) {
@@ -1403,7 +1415,7 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
           }
         }
         else if (b4) {
-          k_sap_sweep_d4<<<2 * grid.x, BlockD::N, smem_d4, c->stream>>>(rin, rho, psi, delta, gauge, clover, c->g, sg,
+          kernC<<<2 * grid.x, BlockD::N, smem_d4, c->stream>>>(rin, rho, psi, delta, gauge, clover, c->g, sg,
                                                                         col, gather, first, last, c->kappa, P.nmr,
                                                                         nrhs, mask);
         } else
