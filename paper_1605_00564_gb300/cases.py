@@ -49,7 +49,8 @@ def sap_32c64():
     import torch
     lat = _lattice((64, 32, 32, 32), kappa=0.13)
     psi = torch.randn(lat.spinor_shape(12), dtype=torch.complex128, device="cuda")
-    lat.set_params(block=(4, 4, 4, 4), ncy=1, nmr=4, sap_half=1)
+    # launches 8 and 9 are the second application's middle cycle
+    lat.set_params(block=(4, 4, 4, 4), ncy=3, nmr=4, sap_half=1)
     for _ in range(2):
         lat.apply_sap(psi)
 
