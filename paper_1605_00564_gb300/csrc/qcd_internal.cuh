@@ -557,6 +557,8 @@ qcd_status blas_xmy(qcd_ctx* c, const void* x, const void* y, void* out, int pre
 // working residual (overwritten); rho_src = nullptr means rho itself
 qcd_status sap_apply(qcd_ctx* c, void* rho, void* psi, void* delta, int prec, int nrhs, const int* mask,
                      int nactive, int accumulate = 0, const void* rho_src = nullptr);
+// room for what the SAP keeps per gauge field (a failure is no error)
+void sap_reserve(qcd_ctx* c);
 
 // deflation (dfl.cu)
 qcd_status dfl_setup(qcd_ctx* c, const double* init_dev, int ns, int n_inv);
