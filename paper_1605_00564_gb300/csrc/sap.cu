@@ -1302,6 +1302,14 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
     sg.b[mu] = P.block[mu];
     sg.nb[mu] = c->g.L[mu] / sg.b[mu];
     sg.vb *= sg.b[mu];
+    // (qcd_set_params checks this, but a lattice that the default blocks do not fit
+    // starts with 2^4 ones unchecked: with an odd number of blocks in a direction
+    // block_of counts past the lattice)
+    if (c->g.L[mu] % sg.b[mu] != 0 || sg.nb[mu] % 2 != 0) {
+      qcd_set_error("SAP: %d sites in direction %d are no even number of blocks of %d; set the block shape", c->g.L[mu],
+                    mu, sg.b[mu]);
+      return QCD_ERR_ARG;
+    }
   }
   sg.lst[1] = 1;
   sg.lst[2] = sg.b[1];
