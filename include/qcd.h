@@ -92,7 +92,8 @@ typedef enum { QCD_PREC_F64 = 0, QCD_PREC_F32 = 1 } qcd_precision;
  *               preconditioner changes by their rounding; the outer flexible
  *               GCR is unaffected in what it converges to); 2 = in addition the
  *               block residual read by neighbouring sites is held as bf16;
- *               0 = FP32 copies.
+ *               0 = FP32 copies.  Blocks of more than 256 sites, and with 1
+ *               also blocks with an extent of 1, use FP32 copies throughout.
  *   basis_half  QCD_PREC_F32 only: 1 = the GCR images chi_k = D phi_k are
  *               stored as FP16 with one FP32 scale per site (52 bytes per site
  *               instead of 96; arithmetic stays FP32).  The recursive residual

@@ -508,8 +508,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, RES)
 //              block takes 172 KB and an SM holds one CTA, whose loads and
 //              barriers nothing hides;
 //   FromImage  the FP32 image read from L2 at every step (blocks of more than 256
-//              sites, whose copies exceed shared memory; 8 x 4^3 blocks have the
-//              sweep of their own below);
+//              sites, whose copies exceed shared memory, and blocks with an extent
+//              of 1; 8 x 4^3 blocks have the sweep of their own below);
 //   FromField  the same from the lexicographic fields, where there is no memory
 //              for an image.
 // Either staged form leaves room for two CTAs of a 4^4 block per SM.
@@ -1247,6 +1247,14 @@ __global__ void k_face_links(const float4* __restrict__ gauge, Geom g, SapGeom s
 // blocks of k_sap_sweep_b4
 bool face_blocks(const int b[4]) { return b[1] == 4 && b[2] == 4 && b[3] == 4 && (b[0] == 4 || b[0] == 8); }
 
+// whether the FP32 sweep stages links (and clover term) of such blocks, and whether
+// as 16-bit copies
+bool stageable(const qcd_solver_params& P, const int b[4]) {
+  const bool thin = b[0] == 1 || b[1] == 1 || b[2] == 1 || b[3] == 1;
+  return b[0] * b[1] * b[2] * b[3] <= 256 && (!thin || P.sap_half == 2);
+}
+bool sap_uses_half(const qcd_solver_params& P, const int b[4]) { return P.sap_half && stageable(P, b); }
+
 // Brings the context's block image for these blocks up to date; *img = nullptr
 // when there is no memory for it.  flinks only for blocks of T x 4^3, T = 4 or 8.
 qcd_status block_image(qcd_ctx* c, const SapGeom& sg, bool half, bool faces, const unsigned char** img,
@@ -1338,10 +1346,13 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   const int fam = sizeof(typename F::R) == 8 ? FAM_SAP_D : FAM_SAP_F;
   constexpr bool f32 = sizeof(typename F::R) == 4;
   const bool b4 = face_blocks(sg.b) && (f32 || sg.b[0] == 4);
-  // FP32 blocks of at most 256 sites are staged in shared memory; without memory
-  // for the FP32 image (FromField), or for the block-ordered vectors of a block of
-  // 4 or 8 x 4^3, the sweep runs on the lexicographic fields
-  const bool h16 = f32 && P.sap_half && sg.vb <= 256;
+  // FP32 blocks of at most 256 sites are staged in shared memory, unless an extent is
+  // 1: the two faces of such a direction are the same sites, which smem_gather_dir does
+  // not serve (the bf16 residual's and the unstaged sweeps gather per site; a second
+  // pass of smem_gather_dir cost the other shapes 1 to 5 %).  Without memory for the
+  // FP32 image (FromField), or for the block-ordered vectors of a block of 4 or 8 x 4^3,
+  // the sweep runs on the lexicographic fields
+  const bool h16 = f32 && sap_uses_half(P, sg.b);
   const unsigned char* img = nullptr;
   SapB4 A = {};
   bool use_b4 = false;
@@ -1364,7 +1375,7 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
       A.accumulate = accumulate;
     }
   }
-  const bool staged = f32 && sg.vb <= 256 && img;
+  const bool staged = f32 && stageable(P, sg.b) && img;
   // the register budget per thread follows from the block volume
   auto kernD = sg.vb <= 256   ? k_sap_sweep<FieldsD, 256, 1>
                : sg.vb <= 512 ? k_sap_sweep<FieldsD, 512, 1>
@@ -1495,7 +1506,7 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
 void sap_reserve(qcd_ctx* c) {
   const int* b = c->params.block;
   if (c->params.precision == QCD_PREC_F64) return;
-  const bool h16 = c->params.sap_half && b[0] * b[1] * b[2] * b[3] <= 256;
+  const bool h16 = sap_uses_half(c->params, b);
   devbuf_ensure(h16 ? c->sap_img16.buf : c->sap_img32.buf, (size_t)c->g.V * (h16 ? 288 : 480));
   if (face_blocks(b)) devbuf_ensure(c->flinks, (size_t)c->g.V * 96);
 }
