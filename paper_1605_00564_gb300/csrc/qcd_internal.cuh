@@ -430,7 +430,7 @@ struct SapImage {
 struct SapGraph {
   const void *rho_src, *rho, *psi, *delta, *gauge, *clover, *img, *flinks, *vec;
   const int* mask;
-  int nrhs, ncy, nmr, accumulate, half, prec, block[4];
+  int nrhs, ncy, nmr, accumulate, half, prec, bc_t, block[4];
   double kappa;
   cudaGraphExec_t exec;
 };

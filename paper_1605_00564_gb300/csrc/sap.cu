@@ -1454,6 +1454,7 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   key.img = img; key.flinks = A.flinks; key.vec = use_b4 ? c->sap_vec.p : nullptr;
   key.nrhs = nrhs; key.ncy = P.ncy; key.nmr = P.nmr; key.accumulate = accumulate; key.half = P.sap_half;
   key.prec = (int)sizeof(typename F::R);
+  key.bc_t = c->g.bc_t;   // in the captured launches' Geom; a new field may change it
   for (int mu = 0; mu < 4; mu++) key.block[mu] = P.block[mu];
   key.kappa = c->kappa;
   cudaGraphExec_t exec = nullptr;
@@ -1462,7 +1463,7 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
         gph.clover == key.clover && gph.mask == key.mask && gph.img == key.img && gph.flinks == key.flinks &&
         gph.vec == key.vec && gph.nrhs == key.nrhs && gph.ncy == key.ncy &&
         gph.nmr == key.nmr && gph.accumulate == key.accumulate && gph.half == key.half && gph.prec == key.prec &&
-        gph.kappa == key.kappa && memcmp(gph.block, key.block, sizeof(key.block)) == 0) {
+        gph.bc_t == key.bc_t && gph.kappa == key.kappa && memcmp(gph.block, key.block, sizeof(key.block)) == 0) {
       exec = gph.exec;
       break;
     }
