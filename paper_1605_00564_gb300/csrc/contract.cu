@@ -10,8 +10,7 @@ int contract_sites_per_cta(const qcd_ctx* c) {
 template <typename R, bool CANONICAL>
 static qcd_status launch_sites(qcd_ctx* c, const void* prop, int ns, double2* partials) {
   const size_t smem = nucleon::cta_smem<R>(ns);
-  QCD_CUDA_OK(cudaFuncSetAttribute(nucleon::k_sites<R, CANONICAL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)smem));
+  QCD_CUDA_OK(allow_smem(nucleon::k_sites<R, CANONICAL>, nucleon::cta_smem<R>(nucleon::MAX_SITES)));
   nucleon::k_sites<R, CANONICAL><<<c->g.V / ns, nucleon::cta_threads(ns), smem, c->stream>>>((const double2*)prop,
                                                                                              c->g.V, ns, partials);
   QCD_CUDA_OK(cudaGetLastError());

@@ -19,6 +19,8 @@
 
 namespace {
 
+constexpr int MAX_NS = 32;   // deflation fields (checked at qcd_deflation_setup)
+
 struct BlkGeom {
   int b[4], nb[4], lst[4], vb, nblk;
 };
@@ -516,6 +518,7 @@ constexpr int LITTLE_JR = 6;     // (j, r) sums per thread: 64 steps x 24 RHS / 
 // 128-bit words, the orthogonalisation below keeps 24 loads in flight: deflation 1.61
 // -> 1.41 ms per outer iteration (12 RHS, N_s 20, 24 steps).  The nine parts are summed in a fixed order.
 constexpr int LQR = 12;
+constexpr size_t little_q_smem(int ns, int n) { return sizeof(float2) * ((size_t)2 * 9 * ns * LQR + (size_t)ns * n); }
 __global__ void __launch_bounds__(LTPB, 4) k_little_q(const float2* __restrict__ At, const float2* __restrict__ p,
                                                    float2* __restrict__ q, const float2* __restrict__ qbase,
                                                    size_t stride, int nj, double2* __restrict__ part, BlkGeom bg,
@@ -873,9 +876,9 @@ static qcd_status little_gcr_tile(qcd_ctx* c, DflState* d, float2* res, float2* 
   // one element per thread of the orthogonalisation (its time is the latency of the
   // loads along j), at most LITTLE_G CTAs per RHS
   const int Go = (N + LTPB - 1) / LTPB < LITTLE_G ? (N + LTPB - 1) / LTPB : LITTLE_G;
-  const size_t sm_q = sizeof(float2) * ((size_t)2 * 9 * ns * LQR + (size_t)ns * n);
+  const size_t sm_q = little_q_smem(ns, n);
   const size_t sm_s = sizeof(float2) * ((size_t)ns * n + (size_t)ns * ns);
-  QCD_CUDA_OK(cudaFuncSetAttribute(k_little_q, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_q));
+  QCD_CUDA_OK(allow_smem(k_little_q, little_q_smem(MAX_NS, LITTLE_RHS)));
   const float2* Ainv = (const float2*)d->Ainvf.p;
   const unsigned Gs = (unsigned)bg.nblk;
   const dim3 threads(LTPB);
@@ -1003,7 +1006,7 @@ qcd_status dfl_low_mode(qcd_ctx* c, const void* rho, void* x, int n, const int* 
     for (int r0 = 0; r0 < n; r0 += LITTLE_RHS) {   // at most 64 tiles of outputs
       const int nr = n - r0 < LITTLE_RHS ? n - r0 : LITTLE_RHS;
       const ProjectShape sh = project_shape(ns, nr);
-      QCD_CUDA_OK(cudaFuncSetAttribute(k_dfl_project, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sh.smem));
+      QCD_CUDA_OK(allow_smem(k_dfl_project, project_shape(MAX_NS, LITTLE_RHS).smem));
       k_dfl_project<<<bg.nblk, GEMM_TPB, sh.smem, c->stream>>>(
           (const char*)d->phi.p, (const char*)rho + spinor_bytes(c, QCD_PREC_F32) * r0, res + (size_t)N * r0, c->g, bg,
           ns, nr, sh, mask ? mask + r0 : nullptr);

@@ -169,7 +169,7 @@ extern "C" qcd_status qcd_fh_gradient(qcd_ctx* c, const double* prop, const int 
   {
     ProfScope ps(c, FAM_CONTRACT, (double)V * (2304 + 2 * 2304), (double)V * 9 * 700 * 8);
     const size_t smem = nucleon_grad::cta_smem(ns);
-    QCD_CUDA_OK(cudaFuncSetAttribute(nucleon_grad::k_dC_dS, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QCD_CUDA_OK(allow_smem(nucleon_grad::k_dC_dS, nucleon_grad::cta_smem(nucleon_grad::MAX_SITES)));
     nucleon_grad::k_dC_dS<<<V / ns, nucleon_grad::cta_threads(ns), smem, c->stream>>>((const double2*)c->wsD[4].p,
                                                                (const double2*)c->contract.p, V, L3, ns, 0,
                                                                (double2*)c->wsD[5].p);

@@ -50,10 +50,8 @@ qcd_status scratch_on_current_device(double2** out) {
   if (!g_scratch_addr[dev]) {
     void* p = nullptr;
     QCD_CUDA_OK(cudaGetSymbolAddress(&p, g_nucleon_scratch));
-    QCD_CUDA_OK(cudaFuncSetAttribute(nucleon::k_sites<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)nucleon::cta_smem<double>(32)));
-    QCD_CUDA_OK(cudaFuncSetAttribute(nucleon::k_sites<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)nucleon::cta_smem<float>(32)));
+    QCD_CUDA_OK(allow_smem(nucleon::k_sites<double, true>, nucleon::cta_smem<double>(nucleon::MAX_SITES)));
+    QCD_CUDA_OK(allow_smem(nucleon::k_sites<float, true>, nucleon::cta_smem<float>(nucleon::MAX_SITES)));
     g_scratch_addr[dev] = (double2*)p;
   }
   *out = g_scratch_addr[dev];

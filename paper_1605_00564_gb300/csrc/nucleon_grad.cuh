@@ -38,9 +38,10 @@ namespace {
 using C64 = Cplx<double>;
 using diquark::cmsub;
 
-// sites of one CTA: the largest power of two <= 16 dividing the spatial volume
+// sites of one CTA: the largest power of two <= MAX_SITES dividing the spatial volume
+constexpr int MAX_SITES = 16;
 inline int sites_per_cta(long long L3) {
-  int ns = 16;
+  int ns = MAX_SITES;
   while (L3 % ns) ns >>= 1;
   return ns;
 }

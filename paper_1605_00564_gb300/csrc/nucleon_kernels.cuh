@@ -161,9 +161,10 @@ __global__ void k_timeslices(const double2* __restrict__ part, int per_t, int T,
   }
 }
 
-// sites per CTA: the largest power of two <= 32 dividing the spatial volume
+// sites per CTA: the largest power of two <= MAX_SITES dividing the spatial volume
+constexpr int MAX_SITES = 32;
 inline int sites_per_cta(long long L3) {
-  int ns = 32;
+  int ns = MAX_SITES;
   while (L3 % ns) ns >>= 1;
   return ns;
 }

@@ -499,6 +499,14 @@ qcd_status layout_spinor_import(qcd_ctx* c, const double* in, void* out, int pre
 qcd_status layout_spinor_export(qcd_ctx* c, const void* in, double* out, int prec, int nrhs);
 qcd_status clover_export(qcd_ctx* c, double* out_dev);
 
+// Raises a kernel's limit of dynamic shared memory to `most`, the most that any launch
+// of it takes.  Not to what the next launch takes: the limit belongs to the kernel, and a
+// host thread with a smaller launch would lower it under another thread's.
+template <typename... P>
+cudaError_t allow_smem(void (*kernel)(P...), size_t most) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Programmatic dependent launch.  A kernel launched with overlap may start while the
 // one before it still runs, once that one's CTAs have all called launch_dependents() or
 // ended; its CTAs must call dependency_wait() before they touch anything the kernels

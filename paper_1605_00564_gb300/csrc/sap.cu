@@ -1398,15 +1398,16 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   // links and clover term read per active site and launch: their FP16 copies
   // (36 B per link, 144 B clover) for the 16-bit staged blocks, else FP32
   const double gcb = h16 ? 4 * 36.0 + 144.0 : 4 * lb + cb;
+  // the largest block that the chosen kernel serves
+  const int most = use_b4 ? sg.vb : sg.vb <= 256 && (staged || !f32) ? 256 : sg.vb <= 512 ? 512 : 1024;
   if constexpr (f32)
-    QCD_CUDA_OK(use_b4 ? cudaFuncSetAttribute(kernB, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-                       : cudaFuncSetAttribute(kernF, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QCD_CUDA_OK(use_b4 ? allow_smem(kernB, smem) : allow_smem(kernF, smem / sg.vb * most));
   else
-    QCD_CUDA_OK(cudaFuncSetAttribute(kernD, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    QCD_CUDA_OK(allow_smem(kernD, smem / sg.vb * most));
   const size_t smem_d4 = (size_t)2 * 12 * BlockD::N * sizeof(double2);
   auto kernC = d4_three(2 * grid.x) ? k_sap_sweep_d4<3> : k_sap_sweep_d4<2>;
   if (!f32 && b4)
-    QCD_CUDA_OK(cudaFuncSetAttribute(kernC, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_d4));
+    QCD_CUDA_OK(allow_smem(kernC, smem_d4));
   auto issue = [&]() -> qcd_status {
     for (int cy = 0; cy < P.ncy; cy++)
       for (int col = 0; col < 2; col++) {

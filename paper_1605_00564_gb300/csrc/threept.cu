@@ -229,7 +229,7 @@ qcd_status threept_internal(qcd_ctx* c, const void* S_int, const void* S_sink, c
   const ThreePtMats M = three_pt_mats(direction);
   const int ns = nucleon_grad::sites_per_cta(L3);
   const size_t smem = nucleon_grad::cta_smem(ns);
-  QCD_CUDA_OK(cudaFuncSetAttribute(nucleon_grad::k_dC_dS, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  QCD_CUDA_OK(allow_smem(nucleon_grad::k_dC_dS, nucleon_grad::cta_smem(nucleon_grad::MAX_SITES)));
   std::vector<double2> pm(16 * (size_t)T);
   for (int p = 0; p < 2; p++) {
     const Mat4& P = p == 0 ? M.P : M.P53;
