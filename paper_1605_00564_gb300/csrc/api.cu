@@ -34,10 +34,16 @@ void qcd_set_error(const char* fmt, ...) {
     }                            \
   } while (0)
 
+// For the tests of what runs when device memory is short (not part of qcd.h): workspace
+// allocations of exactly this many bytes by the calling thread fail; 0: none do.
+static thread_local size_t g_fail_bytes = 0;
+extern "C" void qcd_test_fail_alloc(size_t bytes) { g_fail_bytes = bytes; }
+
 qcd_status devbuf_ensure(DevBuf& b, size_t bytes) {
   if (b.bytes >= bytes) return QCD_OK;
   devbuf_free(b);
-  cudaError_t e = cudaMalloc(&b.p, bytes ? bytes : 16);
+  const bool fail = g_fail_bytes != 0 && bytes == g_fail_bytes;
+  cudaError_t e = fail ? cudaErrorMemoryAllocation : cudaMalloc(&b.p, bytes ? bytes : 16);
   if (e != cudaSuccess) {
     b.p = nullptr;
     cudaGetLastError();

@@ -1255,8 +1255,8 @@ bool stageable(const qcd_solver_params& P, const int b[4]) {
 }
 bool sap_uses_half(const qcd_solver_params& P, const int b[4]) { return P.sap_half && stageable(P, b); }
 
-// Brings the context's block image for these blocks up to date; *img = nullptr
-// when there is no memory for it.  flinks only for blocks of T x 4^3, T = 4 or 8.
+// Brings the context's block image for these blocks up to date, and with faces (blocks
+// of T x 4^3, T = 4 or 8) the face links; nullptr for what there is no memory for.
 qcd_status block_image(qcd_ctx* c, const SapGeom& sg, bool half, bool faces, const unsigned char** img,
                        const float4** flinks) {
   SapImage& m = half ? c->sap_img16 : c->sap_img32;
@@ -1264,6 +1264,7 @@ qcd_status block_image(qcd_ctx* c, const SapGeom& sg, bool half, bool faces, con
   bool same = m.gauge_id == c->gauge_id && m.buf.p;
   for (int mu = 0; mu < 4; mu++) same = same && m.block[mu] == sg.b[mu];
   *img = nullptr;
+  *flinks = nullptr;
   if (!same) {
     m.gauge_id = 0;
     const qcd_status st = devbuf_ensure(m.buf, V * (half ? 288 : 480));
@@ -1281,6 +1282,7 @@ qcd_status block_image(qcd_ctx* c, const SapGeom& sg, bool half, bool faces, con
     for (int mu = 0; mu < 4; mu++) m.block[mu] = sg.b[mu];
     m.gauge_id = c->gauge_id;
   }
+  *img = (const unsigned char*)m.buf.p;
   if (faces && (c->flinks_id != c->gauge_id || c->flinks_nt != sg.b[0])) {
     c->flinks_id = 0;
     const qcd_status st = devbuf_ensure(c->flinks, V * 96);
@@ -1295,8 +1297,7 @@ qcd_status block_image(qcd_ctx* c, const SapGeom& sg, bool half, bool faces, con
     c->flinks_nt = sg.b[0];
     c->flinks_id = c->gauge_id;
   }
-  *img = (const unsigned char*)m.buf.p;
-  if (flinks) *flinks = (const float4*)c->flinks.p;
+  if (faces) *flinks = (const float4*)c->flinks.p;
   return QCD_OK;
 }
 
@@ -1350,8 +1351,8 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   // 1: the two faces of such a direction are the same sites, which smem_gather_dir does
   // not serve (the bf16 residual's and the unstaged sweeps gather per site; a second
   // pass of smem_gather_dir cost the other shapes 1 to 5 %).  Without memory for the
-  // FP32 image (FromField), or for the block-ordered vectors of a block of 4 or 8 x 4^3,
-  // the sweep runs on the lexicographic fields
+  // FP32 image (FromField), or for the face links or block-ordered vectors of a block of
+  // 4 or 8 x 4^3, the sweep runs on the lexicographic fields or vectors
   const bool h16 = f32 && sap_uses_half(P, sg.b);
   const unsigned char* img = nullptr;
   SapB4 A = {};
@@ -1359,7 +1360,7 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   if constexpr (f32) {
     QCD_TRY(block_image(c, sg, h16, b4, &img, &A.flinks));
     if (h16 && !img) return QCD_ERR_OOM;
-    if (b4 && img) {
+    if (b4 && img && A.flinks) {
       // psi_b, and rho_b where the caller's residual is its own working copy
       const size_t vec = (size_t)c->g.V * 96 * nrhs;
       const bool own = rho_src != rho;
