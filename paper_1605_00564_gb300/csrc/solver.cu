@@ -316,17 +316,26 @@ qcd_status solver_run(qcd_ctx* c, int n, const double* tol, qcd_rhs_stats* st) {
   return QCD_OK;
 }
 
+// Field-sized workspace of a solve per right-hand side.  FP32: the SAP sweep keeps its
+// increments in block order, and the residual too where it is given no copy of it (the
+// deflated preconditioner).
+static size_t solver_bytes(qcd_ctx* c) {
+  const qcd_solver_params& P = c->params;
+  const bool f32 = P.precision == QCD_PREC_F32;
+  const int pchi = (f32 && P.basis_half) ? QCD_PREC_H16 : P.precision;
+  const int sap_vectors = !f32 ? 0 : P.dfl && dfl_ready(c) ? 2 : 1;
+  return 4 * spinor_bytes(c, QCD_PREC_F64) + ((size_t)P.nkv + 3 + sap_vectors) * spinor_bytes(c, P.precision) +
+         (size_t)P.nkv * spinor_bytes(c, pchi);
+}
+extern "C" size_t qcd_test_solver_bytes(qcd_ctx* c) { return solver_bytes(c); }   // (for the tests; not part of qcd.h)
+
 // Largest tile of right-hand sides that fits the device memory budget.
 int solver_tile(qcd_ctx* c, int nrhs) {
   const qcd_solver_params& P = c->params;
   if (P.rhs_tile > 0) return P.rhs_tile < nrhs ? P.rhs_tile : nrhs;
   size_t freeb = 0, totalb = 0;
   cudaMemGetInfo(&freeb, &totalb);
-  const int pchi = (P.precision == QCD_PREC_F32 && P.basis_half) ? QCD_PREC_H16 : P.precision;
-  // (FP32: one more vector for the block-ordered increments of the 4^4 SAP sweep)
-  size_t per = 4 * spinor_bytes(c, QCD_PREC_F64) +
-               ((size_t)P.nkv + 3 + (P.precision == QCD_PREC_F32)) * spinor_bytes(c, P.precision) +
-               (size_t)P.nkv * spinor_bytes(c, pchi);
+  const size_t per = solver_bytes(c);
   size_t budget = freeb > ((size_t)4 << 30) ? freeb - ((size_t)4 << 30) : freeb / 2;
   int t = (int)(budget / (per ? per : 1));
   if (t < 1) t = 1;
