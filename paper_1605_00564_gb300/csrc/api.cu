@@ -261,7 +261,7 @@ qcd_status qcd_load_gauge(qcd_ctx* c, const double* U, int U_on_device, double c
   c->gauge_id++;   // the block images of the previous field are out of date
   QCD_TRY(layout_gauge_import(c, Ud));
   QCD_TRY(layout_clover_build(c));
-  sap_reserve(c);
+  if (c->params_set) sap_reserve(c);
   QCD_CUDA_OK(cudaStreamSynchronize(c->stream));
   c->have_gauge = 1;
   return QCD_OK;
@@ -274,6 +274,7 @@ qcd_status qcd_set_params(qcd_ctx* c, const qcd_solver_params* p) {
   for (int mu = 0; mu < 4; mu++) same_blocks = same_blocks && p->block[mu] == c->params.block[mu];
   if (!same_blocks) dfl_free(c);
   c->params = *p;
+  c->params_set = 1;
   if (c->have_gauge) sap_reserve(c);
   return QCD_OK;
 }

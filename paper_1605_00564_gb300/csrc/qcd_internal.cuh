@@ -447,6 +447,7 @@ struct qcd_ctx {
   double kappa = 0, csw = 0;
   int have_gauge = 0;
   qcd_solver_params params;
+  int params_set = 0;   // by the caller
   // fields
   DevBuf gaugeD, gaugeF, cloverD, cloverF;
   // SAP block images of the links and clover term (sap.cu), 16-bit and FP32,

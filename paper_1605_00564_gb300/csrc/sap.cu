@@ -1503,15 +1503,21 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
 
 }  // namespace
 
-// Allocates what the SAP of the present parameters keeps per gauge field, so that its
+// Allocates what the SAP of the caller's parameters keeps per gauge field, so that its
 // first application does not stop for it (60 us an allocation: a first application on
-// 16x8x8x16, two RHS, 626 -> 543 us).  block_image tries again where there is no memory now.
+// 16x8x8x16, two RHS, 626 -> 543 us), and gives back what was taken for earlier ones
+// and never used.  block_image tries again where there is no memory now.  (Not called
+// before the caller has set parameters: a context that never applies the SAP keeps none
+// of this.)
 void sap_reserve(qcd_ctx* c) {
   const int* b = c->params.block;
-  if (c->params.precision == QCD_PREC_F64) return;
-  const bool h16 = sap_uses_half(c->params, b);
-  devbuf_ensure(h16 ? c->sap_img16.buf : c->sap_img32.buf, (size_t)c->g.V * (h16 ? 288 : 480));
-  if (face_blocks(b)) devbuf_ensure(c->flinks, (size_t)c->g.V * 96);
+  const bool f32 = c->params.precision == QCD_PREC_F32, h16 = f32 && sap_uses_half(c->params, b);
+  const bool faces = f32 && face_blocks(b);
+  if ((!f32 || h16) && c->sap_img32.gauge_id == 0) devbuf_free(c->sap_img32.buf);
+  if (!h16 && c->sap_img16.gauge_id == 0) devbuf_free(c->sap_img16.buf);
+  if (!faces && c->flinks_id == 0) devbuf_free(c->flinks);
+  if (f32) devbuf_ensure(h16 ? c->sap_img16.buf : c->sap_img32.buf, (size_t)c->g.V * (h16 ? 288 : 480));
+  if (faces) devbuf_ensure(c->flinks, (size_t)c->g.V * 96);
 }
 
 qcd_status sap_apply(qcd_ctx* c, void* rho, void* psi, void* delta, int prec, int nrhs, const int* mask,
