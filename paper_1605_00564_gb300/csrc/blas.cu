@@ -183,13 +183,12 @@ __global__ void __launch_bounds__(RED_TPB) k_reduce_final(const double2* __restr
 }
 
 // CTAs per right-hand side of the reducing passes (a function of the volume alone:
-// a right-hand side gives the same bits in any batch).  A CTA ends in FP64 sums over
-// its threads, and a warp's FP64 addition takes the SM 16 cycles (1/64 of the FP32
-// rate): with one site per thread these sums took as long as the loads.  So
-// larger lattices give every thread at least four sites.
+// a right-hand side gives the same bits in any batch): one site per thread up to
+// 155,648 sites.  A thread sums its sites in FP32 and FP64 begins across threads, so no
+// more sites per thread than the cap asks for: four on 16^3x32, tried for fewer FP64
+// sums, lost the small sites beside a large one, 2e-8 of the result.
 int red_grid(const qcd_ctx* c) {
-  const int per = RED_TPB * (c->g.V >= 131072 ? 4 : c->g.V >= 65536 ? 2 : 1);
-  int g = (c->g.V + per - 1) / per;
+  int g = (c->g.V + RED_TPB - 1) / RED_TPB;
   return g < 4 * 152 ? g : 4 * 152;
 }
 
@@ -314,10 +313,15 @@ inline dim3 grid2(const qcd_ctx* c, int nrhs) { return dim3((c->g.V + 255) / 256
 // ---------------------------------------------------------------------------
 constexpr int GS_TPB = 256;
 
-// CTA sums of NV values per thread (GS_TPB threads, fixed order) in FP64: every warp
-// sums whole values from shared memory, 8 additions per lane and 5 across lanes,
-// instead of 5 across the lanes of each of the 8 warps and 8 more (with four sites per
-// thread the Gram-Schmidt passes of 12 RHS on 16^3x32 went from 4.0 to 5.5 TB/s).
+// CTA sums of NV values per thread (GS_TPB threads, fixed order) in FP64.  A warp's FP64
+// addition takes the SM 16 cycles (1/64 of the FP32 rate), and with one site per thread
+// these sums took as long as the loads.  So every warp sums whole values from shared
+// memory: FP32 ones 8 per lane as a pair hi + lo with the exact error of each addition
+// in lo (Knuth's TwoSum; what lo loses is below 2^-45 of the sum), then one FP64 addition
+// and 5 across lanes, instead of 5 across the lanes of each of the 8 warps and 8 more.
+// All passes of 16 iterations, 16^3x32, 12 RHS, FP32 and FP16 images: 15.8 and 14.3 ms
+// as at first, 11.9 and 10.1 with FP64 sums of 8 per lane, 10.8 and 8.6 so; one RHS 2.25
+// and 2.06, 2.00 and 1.66, 1.80 and 1.49.
 // Lane 0 of warp v % 8 passes the sum of value v to out(v, sum).
 template <int NV, typename R, typename Out>
 __device__ inline void cta_sums(const R (&v)[NV], R* sh /* [NV][GS_TPB] */, Out out) {
@@ -329,8 +333,19 @@ __device__ inline void cta_sums(const R (&v)[NV], R* sh /* [NV][GS_TPB] */, Out 
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
   for (int k = w; k < NV; k += NW) {
     double t = 0;
+    if constexpr (std::is_same<R, float>::value) {
+      float hi = sh[k * GS_TPB + l], lo = 0.f;
 #pragma unroll
-    for (int i = 0; i < NW; i++) t += (double)sh[k * GS_TPB + 32 * i + l];
+      for (int i = 1; i < NW; i++) {
+        const float v = sh[k * GS_TPB + 32 * i + l], s = hi + v, b = s - hi;
+        lo += (hi - (s - b)) + (v - b);
+        hi = s;
+      }
+      t = (double)hi + (double)lo;
+    } else {
+#pragma unroll
+      for (int i = 0; i < NW; i++) t += (double)sh[k * GS_TPB + 32 * i + l];
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     if (l == 0) out(k, t);
@@ -774,5 +789,19 @@ qcd_status blas_gs_finish_inner(qcd_ctx* c, void* chik, int pchi, const double* 
   k_sum_parts<<<dim3(1, nrhs), RED_TPB, 0, c->stream>>>((const double2*)c->red.p, 1, G, (double2*)rn2_dev, nrhs,
                                                         mask);
   QCD_CUDA_OK(cudaGetLastError());
+  return QCD_OK;
+}
+// For the tests (not part of qcd.h): the three passes of a Gram-Schmidt step on FP32
+// fields in the internal layout, chi [k + 1][n] and rho [n]: dots of chi_k with
+// chi_0 .. chi_{k-1}; |chi_k|^2 and (chi_k, rho) without a subtraction; |rho|^2 after
+// chi_k *= inv and rho -= ck chi_k.  All pointers device memory.
+extern "C" qcd_status qcd_test_gs(qcd_ctx* c, void* chi, void* rho, int k, int n, const double* inv, const double* ck,
+                                  double* dots, double* n2c, double* rn2) {
+  const size_t vec = spinor_bytes(c, QCD_PREC_F32) * n;
+  char* chik = (char*)chi + vec * k;
+  QCD_TRY(blas_gs_dots(c, chi, QCD_PREC_F32, vec, k, n, dots, nullptr, n));
+  QCD_TRY(blas_gs_orth(c, chik, QCD_PREC_F32, vec, 0, dots, rho, QCD_PREC_F32, n, n2c, nullptr, n));
+  QCD_TRY(blas_gs_finish_inner(c, chik, QCD_PREC_F32, inv, ck, rho, QCD_PREC_F32, n, rn2, nullptr, n));
+  QCD_CUDA_OK(cudaStreamSynchronize(c->stream));
   return QCD_OK;
 }
