@@ -504,7 +504,64 @@ __global__ void k_to_float2(const double2* __restrict__ in, float2* __restrict__
 constexpr int LTPB = 256;
 constexpr int LITTLE_G = 608;    // CTAs of the kernels that leave partial sums
 constexpr int LITTLE_RHS = 24;   // right-hand sides of one little solve
-constexpr int LITTLE_JR = 6;     // (j, r) sums per thread: 64 steps x 24 RHS / 256
+
+// hi + lo += v, without rounding but of lo
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float v) {
+  const float t = hi + v, b = t - hi;
+  lo += (hi - (t - b)) + (v - b);
+  hi = t;
+}
+
+// The dots of q's block (qs) with the nj vectors' (at qb, `stride` apart, their right-hand
+// sides rstride) added to the running sums.  At most ten products are summed in FP32 (in two
+// chains, which round less than the one of 8 to 10 that the dots had in a launch of their
+// own); what is summed over a block's chunks and a CTA's blocks, N_s products of each, keeps
+// the exact error of every addition beside it (Knuth's TwoSum).  A thread takes a chunk, so
+// that the loads of a block are one round; its sum goes to the first thread of its dot,
+// whose running sum waits in shared memory (in registers it would spill).
+__device__ __forceinline__ void little_dots(const float2* qb, size_t stride, size_t rstride, const float2* qs, float4* dot,
+                                         int ns, int n, int nj) {
+  const int lch = ns <= 10 ? 0 : ns <= 20 ? 1 : 2;               // 2^lch chunks
+  const int len = (((ns + (1 << lch) - 1) >> lch) + 1) & ~1;     // of len products
+  for (int t = threadIdx.x; t < (((nj * n) << lch) + 31 & ~31); t += LTPB) {   // (whole warps)
+    const int o = t >> lch, ch = t & ((1 << lch) - 1);
+    float2 sum[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+    if (o < nj * n) {
+      const int j = o / n, r = o - j * n;
+      const float2* qj = qb + j * stride + r * rstride;
+      auto mac = [](float2& s, float2 u, float2 v) {
+        s.x = fmaf(u.x, v.x, s.x);
+        s.x = fmaf(u.y, v.y, s.x);
+        s.y = fmaf(u.x, v.y, s.y);
+        s.y = fmaf(-u.y, v.x, s.y);
+      };
+      const int k0 = ch * len, kn = min(len, ns - k0);
+      float2 u[10];   // all loads before the first use
+      if (ns % 2 == 0) {   // (then every little vector's block is 16-byte aligned)
+#pragma unroll
+        for (int k = 0; k < 10; k += 2) {
+          const float4 w = k < kn ? __ldcg((const float4*)(qj + k0 + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+          u[k] = p2(w.x, w.y);
+          u[k + 1] = p2(w.z, w.w);
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 10; k++) u[k] = k < kn ? __ldcg(qj + k0 + k) : make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int k = 0; k < 10; k++)
+        if (k < kn) mac(sum[k & 1], u[k], qs[(k0 + k) * n + r]);
+    }
+    const float2 v = make_float2(sum[0].x + sum[1].x, sum[0].y + sum[1].y);
+    const bool first = ch == 0 && o < nj * n;
+    float4 d = first ? dot[o] : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c = 0; c < 1 << lch; c++) {
+      two_sum(d.x, d.z, __shfl_sync(0xffffffffu, v.x, (t & 31) - ch + c));
+      two_sum(d.y, d.w, __shfl_sync(0xffffffffu, v.y, (t & 31) - ch + c));
+    }
+    if (first) dot[o] = d;
+  }
+}
 
 // q = A p on the CTA's blocks, and the CTA's partial sums of (q_j, q), j < nj, to
 // part[(r nj + j) gridDim + cta].  At: the matrix with the row index of each of its
@@ -516,9 +573,12 @@ constexpr int LITTLE_JR = 6;     // (j, r) sums per thread: 64 steps x 24 RHS / 
 // of its loads: four CTAs of 64 registers per SM hold all 512 blocks of a 16^3x32
 // lattice at once (three, in two waves, are no faster than the old form); the dots read
 // 128-bit words, the orthogonalisation below keeps 24 loads in flight: deflation 1.61
-// -> 1.41 ms per outer iteration (12 RHS, N_s 20, 24 steps).  The nine parts are summed in a fixed order.
+// -> 1.41 ms per outer iteration (12 RHS, N_s 20, 24 steps).  The nine parts are summed in a
+// fixed order.
 constexpr int LQR = 12;
-constexpr size_t little_q_smem(int ns, int n) { return sizeof(float2) * ((size_t)2 * 9 * ns * LQR + (size_t)ns * n); }
+constexpr size_t little_q_smem(int ns, int n, int nj) {
+  return sizeof(float2) * ((size_t)2 * 9 * ns * LQR + (size_t)(ns * n + 1) / 2 * 2) + sizeof(float4) * nj * n;
+}
 __global__ void __launch_bounds__(LTPB, 4) k_little_q(const float2* __restrict__ At, const float2* __restrict__ p,
                                                    float2* __restrict__ q, const float2* __restrict__ qbase,
                                                    size_t stride, int nj, double2* __restrict__ part, BlkGeom bg,
@@ -527,15 +587,14 @@ __global__ void __launch_bounds__(LTPB, 4) k_little_q(const float2* __restrict__
   float2* xs = (float2*)smem_raw;                 // [9 ns][LQR]
   float2* red = xs + (size_t)9 * ns * LQR;        // [9][LQR][ns]
   float2* qs = red + (size_t)9 * ns * LQR;        // [ns][n]
+  float4* dot = (float4*)(qs + (size_t)(ns * n + 1) / 2 * 2);   // [nj][n] (sum re, im, their errors)
   launch_dependents();
   dependency_wait();
-  float2 acc[LITTLE_JR];
-#pragma unroll
-  for (int i = 0; i < LITTLE_JR; i++) acc[i] = make_float2(0.f, 0.f);
+  for (int o = threadIdx.x; o < nj * n; o += LTPB) dot[o] = make_float4(0.f, 0.f, 0.f, 0.f);
   for (int blk = blockIdx.x; blk < bg.nblk; blk += gridDim.x) {
-    int nbr[9];
-    little_neighbours(bg, blk, nbr);
     for (int c0 = 0; c0 < n; c0 += LQR) {
+      int nbr[9];   // (here: not in registers during the products below)
+      little_neighbours(bg, blk, nbr);
       __syncthreads();
 #pragma unroll
       for (int m = 0; m < 9; m++)
@@ -552,16 +611,25 @@ __global__ void __launch_bounds__(LTPB, 4) k_little_q(const float2* __restrict__
         float2 u[LQR];
 #pragma unroll
         for (int r = 0; r < LQR; r++) u[r] = p2(0.f, 0.f);
-#pragma unroll 10
-        for (int l = 0; l < ns; l++) {
-          const float2 w = __ldg(a + l * ns), wi = p2(-w.y, w.y);
+        auto row = [&](int l, float2 w) {
+          const float2 wi = p2(-w.y, w.y);
 #pragma unroll
           for (int r = 0; r < LQR; r += 2) {
             const float4 x = xv[(l * LQR + r) >> 1];
             u[r] = pfma(wi, p2(x.y, x.x), pfma(pbc(w.x), p2(x.x, x.y), u[r]));
             u[r + 1] = pfma(wi, p2(x.w, x.z), pfma(pbc(w.x), p2(x.z, x.w), u[r + 1]));
           }
+        };
+        int l = 0;
+        for (; l + 8 <= ns; l += 8) {   // 8 loads before the first use
+          float2 w[8];   // (left to the compiler they are not: 10,400 -> 13,400 cycles, N_s 20)
+#pragma unroll
+          for (int i = 0; i < 8; i++) w[i] = __ldg(a + (l + i) * ns);
+#pragma unroll
+          for (int i = 0; i < 8; i++) row(l + i, w[i]);
         }
+#pragma unroll 1
+        for (; l < ns; l++) row(l, __ldg(a + l * ns));
 #pragma unroll
         for (int r = 0; r < LQR; r++) red[(m * LQR + r) * ns + k] = u[r];
       }
@@ -582,39 +650,14 @@ __global__ void __launch_bounds__(LTPB, 4) k_little_q(const float2* __restrict__
     }
     if (nj == 0) continue;
     __syncthreads();
-#pragma unroll
-    for (int i = 0; i < LITTLE_JR; i++) {
-      const int o = threadIdx.x + i * LTPB;
-      if (o < nj * n) {
-        const int j = o / n, r = o - j * n;
-        const float2* qj = qbase + j * stride + ((size_t)r * bg.nblk + blk) * ns;
-        auto mac = [&](float2 u, float2 v) {
-          acc[i].x = fmaf(u.x, v.x, acc[i].x);
-          acc[i].x = fmaf(u.y, v.y, acc[i].x);
-          acc[i].y = fmaf(u.x, v.y, acc[i].y);
-          acc[i].y = fmaf(-u.y, v.x, acc[i].y);
-        };
-        if (ns % 2 == 0) {   // (then every little vector's block is 16-byte aligned)
-#pragma unroll 5
-          for (int k = 0; k < ns; k += 2) {
-            const float4 u = __ldcg((const float4*)(qj + k));
-            mac(p2(u.x, u.y), qs[k * n + r]);
-            mac(p2(u.z, u.w), qs[(k + 1) * n + r]);
-          }
-        } else {
-#pragma unroll 4
-          for (int k = 0; k < ns; k++) mac(__ldcg(qj + k), qs[k * n + r]);
-        }
-      }
-    }
+    little_dots(qbase + (size_t)blk * ns, stride, (size_t)bg.nblk * ns, qs, dot, ns, n, nj);
   }
-#pragma unroll
-  for (int i = 0; i < LITTLE_JR; i++) {
-    const int o = threadIdx.x + i * LTPB;
-    if (o < nj * n) {
-      const int j = o / n, r = o - j * n;
-      part[((size_t)r * nj + j) * gridDim.x + blockIdx.x] = make_double2((double)acc[i].x, (double)acc[i].y);
-    }
+  __syncthreads();
+  for (int o = threadIdx.x; o < nj * n; o += LTPB) {
+    const int j = o / n, r = o - j * n;
+    const float4 t = dot[o];
+    part[((size_t)r * nj + j) * gridDim.x + blockIdx.x] =
+        make_double2((double)t.x + (double)t.z, (double)t.y + (double)t.w);
   }
 }
 
@@ -876,9 +919,8 @@ static qcd_status little_gcr_tile(qcd_ctx* c, DflState* d, float2* res, float2* 
   // one element per thread of the orthogonalisation (its time is the latency of the
   // loads along j), at most LITTLE_G CTAs per RHS
   const int Go = (N + LTPB - 1) / LTPB < LITTLE_G ? (N + LTPB - 1) / LTPB : LITTLE_G;
-  const size_t sm_q = little_q_smem(ns, n);
   const size_t sm_s = sizeof(float2) * ((size_t)ns * n + (size_t)ns * ns);
-  QCD_CUDA_OK(allow_smem(k_little_q, little_q_smem(MAX_NS, LITTLE_RHS)));
+  QCD_CUDA_OK(allow_smem(k_little_q, little_q_smem(MAX_NS, LITTLE_RHS, 64)));
   const float2* Ainv = (const float2*)d->Ainvf.p;
   const unsigned Gs = (unsigned)bg.nblk;
   const dim3 threads(LTPB);
@@ -887,7 +929,7 @@ static qcd_status little_gcr_tile(qcd_ctx* c, DflState* d, float2* res, float2* 
   for (int i = 0; i < m; i++) {
     float2* pi = P + vlen * i;
     float2* qi = Q + vlen * i;
-    QCD_CUDA_OK(launch_after(c->stream, true, Gq, threads, sm_q, k_little_q, (const float2*)d->Af.p, pi, qi, Q, vlen, i,
+    QCD_CUDA_OK(launch_after(c->stream, true, Gq, threads, little_q_smem(ns, n, i), k_little_q, (const float2*)d->Af.p, pi, qi, Q, vlen, i,
                              part, bg, ns, n));
     if (i > 0) QCD_CUDA_OK(launch_after(c->stream, true, dim3(i, n), 32, 0, k_little_sum, part, i, Gq, dots, n));
     QCD_CUDA_OK(launch_after(c->stream, true, dim3(Go, n), threads, 0, k_little_orth, qi, pi, Q, P, vlen, i, dots, res, N,
@@ -1062,5 +1104,24 @@ qcd_status dfl_little_host(qcd_ctx* c, const double* in, double* out, int n, int
     out[2 * i] = h[i].x;
     out[2 * i + 1] = h[i].y;
   }
+  return QCD_OK;
+}
+
+// For the tests (not part of qcd.h): q = A p and the dots of q with nj vectors, as a little
+// GCR step computes them; n <= 24 right-hand sides, nj <= 64.  Device memory: p, q
+// [n][nblk][ns], qj [nj] such vectors, dots [nj][n].
+extern "C" qcd_status qcd_test_little_dots(qcd_ctx* c, const float2* p, const float2* qj, int nj, int n, float2* q,
+                                           double2* dots) {
+  DflState* d = dfl_of(c);
+  if (!d->ready || n < 1 || n > LITTLE_RHS || nj < 1 || nj > 64) return QCD_ERR_ARG;
+  QCD_TRY(devbuf_ensure(d->part, little_part_bytes(n, nj)));
+  double2* part = (double2*)d->part.p;
+  const int ns = d->ns, Gq = d->bg.nblk < LITTLE_G ? d->bg.nblk : LITTLE_G;
+  QCD_CUDA_OK(allow_smem(k_little_q, little_q_smem(MAX_NS, LITTLE_RHS, 64)));
+  k_little_q<<<Gq, LTPB, little_q_smem(ns, n, nj), c->stream>>>((const float2*)d->Af.p, p, q, qj,
+                                                                (size_t)d->bg.nblk * ns * n, nj, part, d->bg, ns, n);
+  k_little_sum<<<dim3(nj, n), 32, 0, c->stream>>>(part, nj, Gq, dots, n);
+  QCD_CUDA_OK(cudaGetLastError());
+  QCD_CUDA_OK(cudaStreamSynchronize(c->stream));
   return QCD_OK;
 }
