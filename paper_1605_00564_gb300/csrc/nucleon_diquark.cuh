@@ -38,13 +38,17 @@ __host__ __device__ constexpr int r_row(int m) { return m < 3 ? 0 : m < 5 ? 1 : 
 __host__ __device__ constexpr int r_col(int m) { return m == 0 ? 0 : (m == 2 || m == 4) ? 3 : 2; }
 __host__ __device__ constexpr int gsgn(int b) { return (b & 1) ? 1 : -1; }
 
-// R_{r_row(m), r_col(m)} of the colour pair (c, cp); get(al, a, alp, ap) reads S
+// R_{r_row(m), r_col(m)} of the colour pair (c, cp); get(al, a, alp, ap) reads S.  FP32:
+// four products at a time, since one chain of 16 made the correlator's rounding error 1.25
+// times that of the 36 permutations (1.18e-7 of the rms on random propagators; 0.93e-7 so).
+// FP64 has no use for the additions, which it would take 12 % longer for.
 template <typename R, typename Get>
 __device__ inline void diquark_r(Get get, int c, int cp, Cplx<R> (&r)[6]) {
   const int x1 = c == 2 ? 0 : c + 1, x2 = c == 0 ? 2 : c - 1;
   const int y1 = cp == 2 ? 0 : cp + 1, y2 = cp == 0 ? 2 : cp - 1;
 #pragma unroll
   for (int m = 0; m < 6; m++) r[m] = cmk((R)0, (R)0);
+  constexpr bool single = sizeof(R) == 4;
 #pragma unroll
   for (int k = 0; k < 4; k++) {
     Cplx<R> X1[4], X2[4], Y1[4], Y2[4];
@@ -58,17 +62,19 @@ __device__ inline void diquark_r(Get get, int c, int cp, Cplx<R> (&r)[6]) {
 #pragma unroll
     for (int m = 0; m < 6; m++) {
       const int u = r_row(m), v = r_col(m) ^ 1;
+      Cplx<R> s = single ? cmk((R)0, (R)0) : r[m];
       if (gsgn(k) * gsgn(r_col(m)) > 0) {
-        cmac(r[m], X1[u], Y2[v]);
-        cmsub(r[m], X1[v], Y2[u]);
-        cmsub(r[m], X2[u], Y1[v]);
-        cmac(r[m], X2[v], Y1[u]);
+        cmac(s, X1[u], Y2[v]);
+        cmsub(s, X1[v], Y2[u]);
+        cmsub(s, X2[u], Y1[v]);
+        cmac(s, X2[v], Y1[u]);
       } else {
-        cmsub(r[m], X1[u], Y2[v]);
-        cmac(r[m], X1[v], Y2[u]);
-        cmac(r[m], X2[u], Y1[v]);
-        cmsub(r[m], X2[v], Y1[u]);
+        cmsub(s, X1[u], Y2[v]);
+        cmac(s, X1[v], Y2[u]);
+        cmac(s, X2[u], Y1[v]);
+        cmsub(s, X2[v], Y1[u]);
       }
+      r[m] = single ? r[m] + s : s;
     }
   }
 }

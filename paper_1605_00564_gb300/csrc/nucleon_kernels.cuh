@@ -108,8 +108,15 @@ __global__ void __launch_bounds__(288) k_sites(const double2* __restrict__ prop,
     }
     // tr R / 2 = R_00 + R_22; tr[P+- X] = (tr X +- tr[g0 X]) / 2
     const Cplx<R> tr = r[0] + r[5];
-    accp = -(tr * (d - q) + (R)0.5 * (zd - zo));
-    accm = -(tr * (d + q) + (R)0.5 * (zd + zo));
+    if constexpr (sizeof(R) == 4) {   // (fewer roundings; FP64 keeps its bits)
+      accp = (R)0.5 * (zo - zd);
+      accm = (R)-0.5 * (zd + zo);
+      cmac(accp, -tr, d - q);
+      cmac(accm, -tr, d + q);
+    } else {
+      accp = -(tr * (d - q) + (R)0.5 * (zd - zo));
+      accm = -(tr * (d + q) + (R)0.5 * (zd + zo));
+    }
   }
   // CTA sum (fixed order): warp shuffles over full warps, then one thread
   // over the warp sums
