@@ -505,7 +505,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, RES)
 //   float      FP32 (float4 [12][vb] link rows 0 and 1, float4 [18][vb] clover in
 //              the order of CloverPairs; 480 B a site): links staged, clover
 //              read from the image (L2) at every step.  With both staged a 4^4
-//              block takes 172 KB and an SM holds one CTA, whose loads and
+//              block takes 147 KB and an SM holds one CTA, whose loads and
 //              barriers nothing hides;
 //   FromImage  the FP32 image read from L2 at every step (blocks of more than 256
 //              sites, whose copies exceed shared memory, and blocks with an extent
@@ -1023,6 +1023,8 @@ __global__ void __launch_bounds__(64 * NT, 8 / NT)
   launch_dependents();
   const int rhs = blockIdx.x % nrhs;   // RHS fastest, as in k_sap_sweep
   const int blk = blockIdx.x / nrhs;
+  // (without a dependency_wait: the CTAs of an active right-hand side, of which every
+  // application has one, wait, so the grid does not end before the previous one)
   if (mask && !mask[rhs]) return;
   const int nhalf = gridDim.x / nrhs;
   const size_t bidx = (size_t)A.colour * nhalf + blk;
