@@ -507,12 +507,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(128, RES)
 //              read from the image (L2) at every step.  With both staged a 4^4
 //              block takes 147 KB and an SM holds one CTA, whose loads and
 //              barriers nothing hides;
-//   FromImage  the FP32 image read from L2 at every step (blocks of more than 256
+//   FromImage  the FP32 image read from L2 at every step (blocks of 257 to 512
 //              sites, whose copies exceed shared memory, and blocks with an extent
 //              of 1; 8 x 4^3 blocks have the sweep of their own below);
 //   FromField  the same from the lexicographic fields, where there is no memory
 //              for an image.
-// Either staged form leaves room for two CTAs of a 4^4 block per SM.
+// Either staged form leaves room for two CTAs of a 4^4 block per SM.  Blocks of more
+// than 512 sites stay with k_sap_sweep: at the 64 registers that 1024 threads leave it,
+// the two-lane sweep spills 1.3 KB (8 x 8 x 4 x 4 blocks, 16^3x32, 2 cycles: 12 RHS
+// 3.05 ms against 2.48, one RHS 540 us against 442).
 // ---------------------------------------------------------------------------
 struct FromImage {};
 struct FromField {};
@@ -1256,6 +1259,8 @@ bool stageable(const qcd_solver_params& P, const int b[4]) {
   return b[0] * b[1] * b[2] * b[3] <= 256 && (!thin || P.sap_half == 2);
 }
 bool sap_uses_half(const qcd_solver_params& P, const int b[4]) { return P.sap_half && stageable(P, b); }
+// whether the FP32 sweep is one in two-lane arithmetic
+bool two_lane(int vb) { return vb <= 512; }
 
 // Brings the context's block image for these blocks up to date, and with faces (blocks
 // of T x 4^3, T = 4 or 8) the face links; nullptr for what there is no memory for.
@@ -1359,7 +1364,8 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   const unsigned char* img = nullptr;
   SapB4 A = {};
   bool use_b4 = false;
-  if constexpr (f32) {
+  const bool pair = f32 && two_lane(sg.vb);
+  if (pair) {
     QCD_TRY(block_image(c, sg, h16, b4, &img, &A.flinks));
     if (h16 && !img) return QCD_ERR_OOM;
     if (b4 && img && A.flinks) {
@@ -1380,9 +1386,8 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   }
   const bool staged = f32 && stageable(P, sg.b) && img;
   // the register budget per thread follows from the block volume
-  auto kernD = sg.vb <= 256   ? k_sap_sweep<FieldsD, 256, 1>
-               : sg.vb <= 512 ? k_sap_sweep<FieldsD, 512, 1>
-                              : k_sap_sweep<FieldsD, 1024, 1>;
+  auto kernD = k_sap_sweep<F, 1024, 1>;
+  if constexpr (!f32) kernD = sg.vb <= 256 ? k_sap_sweep<F, 256, 1> : sg.vb <= 512 ? k_sap_sweep<F, 512, 1> : kernD;
   auto kernB = sg.b[0] == 8    ? k_sap_sweep_b4<float, false, 8>
                : !h16            ? k_sap_sweep_b4<float, false, 4>
                : P.sap_half == 2 ? k_sap_sweep_b4<__half, true, 4>
@@ -1390,10 +1395,8 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   auto kernF = staged ? (!h16              ? k_sap_sweep_pair<float, false, 256, 2>
                          : P.sap_half == 2 ? k_sap_sweep_pair<__half, true, 256, 2>
                                            : k_sap_sweep_pair<__half, false, 256, 2>)
-               : img  ? (sg.vb <= 512 ? k_sap_sweep_pair<FromImage, false, 512, 1>
-                                      : k_sap_sweep_pair<FromImage, false, 1024, 1>)
-                      : (sg.vb <= 512 ? k_sap_sweep_pair<FromField, false, 512, 1>
-                                      : k_sap_sweep_pair<FromField, false, 1024, 1>);
+               : img  ? k_sap_sweep_pair<FromImage, false, 512, 1>
+                      : k_sap_sweep_pair<FromField, false, 512, 1>;
   const size_t smem = (size_t)sg.vb * (!f32                 ? 192
                                        : !staged && !use_b4 ? 96
                                        : !h16               ? 96 + Stage<float>::bytes
@@ -1403,10 +1406,9 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
   const double gcb = h16 ? 4 * 36.0 + 144.0 : 4 * lb + cb;
   // the largest block that the chosen kernel serves
   const int most = use_b4 ? sg.vb : sg.vb <= 256 && (staged || !f32) ? 256 : sg.vb <= 512 ? 512 : 1024;
-  if constexpr (f32)
-    QCD_CUDA_OK(use_b4 ? allow_smem(kernB, smem) : allow_smem(kernF, smem / sg.vb * most));
-  else
-    QCD_CUDA_OK(allow_smem(kernD, smem / sg.vb * most));
+  QCD_CUDA_OK(use_b4 ? allow_smem(kernB, smem)
+              : pair ? allow_smem(kernF, smem / sg.vb * most)
+                     : allow_smem(kernD, smem / sg.vb * most));
   const size_t smem_d4 = (size_t)2 * 12 * BlockD::N * sizeof(double2);
   auto kernC = d4_three(2 * grid.x) ? k_sap_sweep_d4<3> : k_sap_sweep_d4<2>;
   if (!f32 && b4)
@@ -1421,7 +1423,7 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
         ProfScope ps(c, fam, half * (nactive * bytes_rhs + gcb),
                      half * nactive * (flops_site - (gather ? 0.0 : flops_gather)));
         const char* rin = cy == 0 ? rho_src : rho;   // the first cycle reads the caller's residual
-        if constexpr (f32) {
+        if (pair) {
           if (use_b4) {
             A.colour = col;
             A.gather = gather;
@@ -1445,7 +1447,7 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
                                                                         nrhs, mask);
         } else
           kernD<<<grid, sg.vb, smem, c->stream>>>(rin, rho, psi, delta, gauge, clover, c->g, sg, col, gather, first,
-                                                  c->kappa, P.nmr, nrhs, mask);
+                                                  (typename F::R)c->kappa, P.nmr, nrhs, mask);
         QCD_CUDA_OK(cudaGetLastError());
       }
     return QCD_OK;
@@ -1513,7 +1515,8 @@ qcd_status launch_sweeps(qcd_ctx* c, const char* rho_src, char* rho, char* psi, 
 // of this.)
 void sap_reserve(qcd_ctx* c) {
   const int* b = c->params.block;
-  const bool f32 = c->params.precision == QCD_PREC_F32, h16 = f32 && sap_uses_half(c->params, b);
+  const bool f32 = c->params.precision == QCD_PREC_F32 && two_lane(b[0] * b[1] * b[2] * b[3]);
+  const bool h16 = f32 && sap_uses_half(c->params, b);
   const bool faces = f32 && face_blocks(b);
   if ((!f32 || h16) && c->sap_img32.gauge_id == 0) devbuf_free(c->sap_img32.buf);
   if (!h16 && c->sap_img16.gauge_id == 0) devbuf_free(c->sap_img16.buf);

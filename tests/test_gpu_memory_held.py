@@ -39,6 +39,7 @@ def held(steps):
     ([dict(sap_half=1), "load", dict(sap_half=0)], FIELDS + 480 + 96),
     (["load", dict(sap_half=1), dict(block=(4, 4, 4, 2))], FIELDS + 288),
     (["load", dict(sap_half=0), dict(precision="f64")], FIELDS),
+    (["load", dict(block=(8, 8, 4, 4))], FIELDS),     # more than 512 sites: no image
 ])
 def test_memory_held(steps, per_site):
     held(["load"])     # the kernels' own memory
