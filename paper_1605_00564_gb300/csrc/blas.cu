@@ -183,18 +183,24 @@ __global__ void __launch_bounds__(RED_TPB) k_reduce_final(const double2* __restr
 }
 
 // CTAs per right-hand side of the reducing passes (a function of the volume alone:
-// a right-hand side gives the same bits in any batch): one site per thread up to
-// 155,648 sites.  A thread sums its sites in FP32 and FP64 begins across threads, so no
-// more sites per thread than the cap asks for: four on 16^3x32, tried for fewer FP64
-// sums, lost the small sites beside a large one, 2e-8 of the result.
-int red_grid(const qcd_ctx* c) {
-  int g = (c->g.V + RED_TPB - 1) / RED_TPB;
+// a right-hand side gives the same bits in any batch).
+// Sums in FP32: one site per thread up to 155,648 sites.  A thread sums its sites in FP32
+// and FP64 begins across threads, so no more sites per thread than the cap asks for: four
+// on 16^3x32, tried for fewer FP64 sums, lost the small sites beside a large one, 2e-8 of
+// the result.
+// Sums in FP64, or none (free): more sites per thread cost no accuracy, and larger
+// lattices have four, for fewer CTAs that each begin and end (the vector passes of a
+// gradient call on 16^3x32, 12 and 24 RHS, 12.5 ms; with the solution update, k_caxpy_sm,
+// at one site per thread 13.0).
+int red_grid(const qcd_ctx* c, bool free) {
+  const int per = RED_TPB * (!free || c->g.V < 65536 ? 1 : c->g.V < 131072 ? 2 : 4);
+  int g = (c->g.V + per - 1) / per;
   return g < 4 * 152 ? g : 4 * 152;
 }
 
 template <typename X, typename Y, int OP>
 qcd_status reduce(qcd_ctx* c, const void* x, const void* y, int nrhs, void* out, const int* mask) {
-  int G = red_grid(c);
+  int G = red_grid(c, sizeof(typename Acc<X, Y>::R) == 8);
   QCD_TRY(devbuf_ensure(c->red, (size_t)G * nrhs * sizeof(double2)));
   ProfScope ps(c, FAM_BLAS, (double)c->g.V * nrhs * (X::bytes + (OP ? Y::bytes : 0)), (double)c->g.V * nrhs * 96, 2);
   k_reduce<X, Y, OP><<<dim3(G, nrhs), RED_TPB, 0, c->stream>>>((const char*)x, (const char*)y, c->g.V,
@@ -632,7 +638,7 @@ qcd_status blas_multi_caxpy(qcd_ctx* c, void* y, int py, const void* xbase, int 
     k_multi_caxpy<PD, PD><<<g, 256, 0, c->stream>>>((char*)y, (const char*)xbase, nx, xstride,
                                                     (const double2*)coef_dev, sign, c->g.V, nrhs, mask);
   else if (py == QCD_PREC_F64 && px == QCD_PREC_F32) {
-    const dim3 gs(red_grid(c), nrhs);
+    const dim3 gs(red_grid(c, true), nrhs);   // (no sums)
     const double2* cf = (const double2*)coef_dev;
     if (nx <= 8)
       k_caxpy_sm<8><<<gs, GS_TPB, 0, c->stream>>>((char*)y, (const char*)xbase, nx, xstride, cf, sign, c->g.V, nrhs,
@@ -696,7 +702,7 @@ qcd_status blas_convert(qcd_ctx* c, const void* in, int pin, void* out, int pout
 qcd_status blas_gs_dots(qcd_ctx* c, const void* chi, int prec, size_t jstride, int k, int nrhs, double* dots_dev,
                         const int* mask, int nactive) {
   if (k <= 0) return QCD_OK;
-  const int G = red_grid(c);
+  const int G = red_grid(c, prec == QCD_PREC_F64);
   QCD_TRY(devbuf_ensure(c->red, (size_t)G * k * nrhs * sizeof(double2)));
   const double vb = prec == QCD_PREC_F64 ? 192 : prec == QCD_PREC_H16 ? (double)PH::bytes : 96;
   ProfScope ps(c, FAM_BLAS, (double)c->g.V * nactive * (k + 1) * vb, (double)c->g.V * nactive * k * 48, 2);
@@ -725,7 +731,7 @@ qcd_status blas_gs_dots(qcd_ctx* c, const void* chi, int prec, size_t jstride, i
 // chi_k -= sum_j dots[j] chi_j; n2c[0][r] = |chi_k|^2 (re), n2c[1][r] = (chi_k, rho)
 qcd_status blas_gs_orth(qcd_ctx* c, void* chi, int prec, size_t jstride, int k, const double* dots_dev,
                         const void* rho, int prho, int nrhs, double* n2c_dev, const int* mask, int nactive) {
-  const int G = red_grid(c);
+  const int G = red_grid(c, prec == QCD_PREC_F64 || prho == QCD_PREC_F64);
   QCD_TRY(devbuf_ensure(c->red, (size_t)G * 2 * nrhs * sizeof(double2)));
   const double vb = prec == QCD_PREC_F64 ? 192 : prec == QCD_PREC_H16 ? (double)PH::bytes : 96;
   ProfScope ps(c, FAM_BLAS, (double)c->g.V * nactive * ((k + 2) * vb + (prho == QCD_PREC_F64 ? 192 : 96)),
@@ -770,7 +776,7 @@ qcd_status blas_gs_finish_inner(qcd_ctx* c, void* chik, int pchi, const double* 
     qcd_set_error("gs_finish: unsupported precision pair");
     return QCD_ERR_ARG;
   }
-  const int G = red_grid(c);
+  const int G = red_grid(c, f64);
   QCD_TRY(devbuf_ensure(c->red, (size_t)G * nrhs * sizeof(double2)));
   const dim3 grid(G, nrhs);
   char* cp = (char*)chik;
