@@ -570,7 +570,8 @@ __device__ __forceinline__ void little_dots(const float2* qb, size_t stride, siz
 // global memory, and the neighbours' p are broadcast reads from shared memory, six
 // 128-bit words for 12 products.  (One output per thread took two shared-memory words
 // per product, 86,000 per block and step, and staged the matrix.)  Bound by the latency
-// of its loads: four CTAs of 64 registers per SM hold all 512 blocks of a 16^3x32
+// of its loads and the barriers between its phases (16^3x32, 12 RHS, N_s 12: issue 22 %,
+// waits for barriers 9.0 and for loads 7.4 cycles per instruction): four CTAs of 64 registers per SM hold all 512 blocks of a 16^3x32
 // lattice at once (three, in two waves, are no faster than the old form); the dots read
 // 128-bit words, the orthogonalisation below keeps 24 loads in flight: deflation 1.61
 // -> 1.41 ms per outer iteration (12 RHS, N_s 20, 24 steps).  The nine parts are summed in a

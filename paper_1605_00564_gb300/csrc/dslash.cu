@@ -204,9 +204,11 @@ __global__ void __launch_bounds__(2 * SPLIT_SITES) k_dslash_split(const char* __
 // applies the operator to NR right-hand sides of a site with one read of the links
 // and the clover term.
 //
-// Bound by L2 and its latency: a site and right-hand side reads its four neighbours
+// Bound by the latency of L2: a site and right-hand side reads its four neighbours
 // in z and t, itself and its share of the links from L2, about 900 bytes (1,200 with
-// NR = 1), and the 16 to 20 warps that the registers leave an SM hide no more.  24^3x48
+// NR = 1), and the 16 to 20 warps that the registers leave an SM hide no more (16^3x32, 12
+// RHS: a warp waits 4.3 of its 8 cycles per instruction for loads, L2 is at 45 % of its
+// rate, the FMA pipe at 59 %, DRAM at 36 %).  24^3x48
 // against scalar arithmetic and one right-hand side per thread: 12 RHS 634 -> 602 us,
 // one RHS 84 -> 80.  (12 RHS, caller's layout: NR = 2 on 4 CTAs per SM 814 us, on 3 1002,
 // on 5 891; NR = 1 on 5 836, on 8 905.)
